@@ -1917,7 +1917,8 @@ __global__ void __launch_bounds__(kThreads) k_score_f32(const __grid_constant__ 
 // ---------------------------------------------------------------------------
 // k_select: grid (cl, granularity ? Hkv : 1, B) in clusters of cl CTAs of
 // 512 threads (1024 when a rank's slice of the visual tokens is long).
-// Dynamic shared memory: the N_v score keys, of which rank 0's copy is used.
+// Dynamic shared memory: the N_v score keys, of which rank 0's copy is used,
+// and for top-p budgets one float per digit and thread (top_p_cut).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int budget_k(const StepParams& p, float m_max, int nv) {
   if (nv <= 0) return 0;
@@ -1976,6 +1977,93 @@ struct RadixCut {
   bool whole;        // the cut fell on a bucket boundary: keep every key >= theta + 1
 };
 
+// Top-p cut (App. A.2): the fewest top keys whose scores sum to at least
+// ppm / 10^6 of all n scores.  A radix select over score mass, 4 bits a pass
+// from the top: every thread adds the candidates it owns to its own column of
+// col[16][NTH] (plain loads and stores, one bank per lane), warp d sums digit
+// d's row, and every thread takes the digit in which the mass is reached.
+// Bound by latency: eight passes of two barriers each.  The digit sums were
+// shared float atomics before, which retry while lanes meet on one address,
+// and scores fall into few digits: N_v = 6400, 16 sequences, 32 heads, the whole
+// call took 187 us (131 us of it this kernel), now 89 us.  The columns also make the sums (and with
+// them K_t) the same on every run.
+// wsum: 32 floats, wcnt: 2 x NTH / 32 ints.  Returns K (before the capacity
+// clamp); theta, krem and n_theta as in RadixCut (unset when K >= n).
+constexpr int kTopPDigits = 16;
+template <int NTH>
+__device__ __forceinline__ int top_p_cut(const uint32_t* key_s, int n, int ppm, float* col, float* wsum, int* wcnt,
+                                         uint32_t& theta, unsigned& krem, unsigned& n_theta) {
+  constexpr int NW = NTH / 32;
+  static_assert(NW >= kTopPDigits, "a warp per digit");
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (n <= 0 || ppm <= 0) return 0;
+  if (ppm >= 1000000) return n;
+  uint32_t prefix = 0, mask = 0;
+  float need = 0.f;  // score mass still to cover
+  for (int shift = 28; shift >= 0; shift -= 4) {
+#pragma unroll
+    for (int d = 0; d < kTopPDigits; ++d) col[d * NTH + tid] = 0.f;
+    for (int i = tid; i < n; i += NTH) {
+      const uint32_t k = key_s[i];
+      if ((k & mask) == prefix) col[((k >> shift) & 15u) * NTH + tid] += __uint_as_float(k);
+    }
+    __syncthreads();
+    if (warp < kTopPDigits) {
+      float a = 0.f;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) a += col[warp * NTH + 32 * w + lane];
+      a = warp_sum(a);
+      if (lane == 0) wsum[warp] = a;
+    }
+    __syncthreads();
+    float c[kTopPDigits], total = 0.f;
+#pragma unroll
+    for (int d = 0; d < kTopPDigits; ++d) c[d] = wsum[d];
+#pragma unroll
+    for (int d = kTopPDigits - 1; d >= 0; --d) total += c[d];
+    if (shift == 28) {
+      if (!(total > 0.f)) return n;  // no score mass to rank by
+      need = (float)ppm * 1e-6f * total;
+    }
+    // The highest digit that reaches the mass; the lowest non-empty one when
+    // the bucket's digits, rounded, fall short of it.
+    float run = 0.f, before = 0.f;
+    unsigned dsel = 0;
+    bool reached = false;
+#pragma unroll
+    for (int d = kTopPDigits - 1; d >= 0; --d) {
+      if (reached || !(c[d] > 0.f)) continue;
+      dsel = (unsigned)d;
+      before = run;
+      run += c[d];
+      reached = run >= need;
+    }
+    need -= before;
+    prefix |= dsel << shift;
+    mask |= 15u << shift;
+  }
+  // Keys above the threshold and equal to it.
+  int above = 0, eq = 0;
+  for (int i = tid; i < n; i += NTH) {
+    const uint32_t k = key_s[i];
+    above += k > prefix;
+    eq += k == prefix;
+  }
+  above = __reduce_add_sync(0xffffffffu, above);
+  eq = __reduce_add_sync(0xffffffffu, eq);
+  if (lane == 0) { wcnt[warp] = above; wcnt[NW + warp] = eq; }
+  __syncthreads();
+  above = eq = 0;
+  for (int w = 0; w < NW; ++w) { above += wcnt[w]; eq += wcnt[NW + w]; }
+  const float tv = __uint_as_float(prefix);
+  unsigned m_eq = tv > 0.f ? (unsigned)fminf(ceilf(need / tv), (float)n) : (unsigned)eq;
+  m_eq = max(1u, min(m_eq, (unsigned)eq));
+  theta = prefix;
+  krem = m_eq;
+  n_theta = (unsigned)eq;
+  return above + (int)m_eq;
+}
+
 template <int NTH>
 __global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepParams p) {
   constexpr int NW = NTH / 32;
@@ -1985,17 +2073,15 @@ __global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepPara
   __shared__ int wsum_s[32];
   __shared__ int sh_i[4];
   __shared__ int act_s, act_rank_s[8];  // active-token counts (diagnostics)
-  __shared__ float hsum_s[3][256];      // top-p: score sums per digit
-  __shared__ float vsum_s, vsum_rank_s[8];
+  __shared__ float tp_sum_s[32];        // top-p: score mass per digit
+  __shared__ int tp_cnt_s[2 * NW];      // top-p: key counts per warp
 
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank(), ncl = (int)cluster.num_blocks();
   const int gsel = blockIdx.y, b = blockIdx.z, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int i = tid; i < 3 * 256; i += NTH) (&hist_s[0][0])[i] = 0;
-  if (tid == 0) { act_s = 0; vsum_s = 0.f; }
+  if (tid == 0) act_s = 0;
   const bool topp = p.mode == MODE_TOP_P;
-  if (topp)
-    for (int i = tid; i < 3 * 256; i += NTH) (&hsum_s[0][0])[i] = 0.f;
   const Seq sq = load_seq(p, b, false);  // an input: read before the wait
   pdl_wait();
   pdl_trigger();
@@ -2024,7 +2110,8 @@ __global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepPara
   // This rank's slice of the visual tokens; its first logit row is requested
   // now so that it arrives while the statistics are merged (heads up to 32;
   // at 1024 threads the registers are too few for it).
-  const int per = (nv + ncl - 1) / ncl;
+  // Slices of whole 32-token words, so that a warp owns its activity words.
+  const int per = ((nv + ncl - 1) / ncl + 31) & ~31;
   const int i0 = min(nv, rank * per), i1 = min(nv, i0 + per);
   const int hbeg = p.granularity ? gsel * p.G : 0;
   const int hcnt = p.granularity ? p.G : H;
@@ -2119,16 +2206,15 @@ __global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepPara
   unsigned bad = 0;
   const bool diag = p.n_act || p.act_bits;
   int n_on = 0;
-  float vsum = 0.f;  // top-p: this thread's share of the visual score total
+  uint32_t* act_row = p.act_bits ? p.act_bits + ((int64_t)b * nsel + gsel) * p.act_words : nullptr;
+  // Stores the key of token i; returns whether S_i > delta (Sec. 4.3).
   auto emit = [&](int i, float a) {  // a: sum over the heads of exp2(z - M_h) / L_h
     const float sc = a * inv_cnt;
     if (!isfinite(sc)) bad = 1;
     key0[i] = __float_as_uint(sc);
-    vsum += sc;
-    if (diag && __float_as_uint(sc) > p.act_delta_bits) {  // S_i > delta (Sec. 4.3)
-      ++n_on;
-      if (p.act_bits) atomicOr(p.act_bits + ((int64_t)b * nsel + gsel) * p.act_words + (i >> 5), 1u << (i & 31));
-    }
+    const bool on = diag && __float_as_uint(sc) > p.act_delta_bits;
+    n_on += on;
+    return on;
   };
   // Long slices: LPT lanes share a token row, each reading one float4 of its
   // heads, so that a warp's load covers consecutive rows; eight loads per
@@ -2181,7 +2267,15 @@ __global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepPara
 #pragma unroll
       for (int k = 0; k < V / LPT; ++k) {
         const int tok = base + (k + off) * TPI + lane / LPT;
-        if (tok < i1) emit(tok, v[k]);
+        const bool on = tok < i1 && emit(tok, v[k]);
+        if (act_row && __any_sync(0xffffffffu, on)) {
+          // The lanes' tokens of one k span at most V * TPI / 32 words.
+#pragma unroll
+          for (int w = 0; w < V * TPI / 32; ++w) {
+            const unsigned m = __reduce_or_sync(0xffffffffu, on && ((tok - base) >> 5) == w ? 1u << (tok & 31) : 0u);
+            if (m && lane == 0) atomicOr(act_row + (base >> 5) + w, m);
+          }
+        }
       }
     }
   };
@@ -2197,10 +2291,12 @@ __global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepPara
     }
   }
   if (!done) {
-    for (int i = i0 + tid; i < i1; i += NTH) {
+    for (int wb = i0 + 32 * warp; wb < i1; wb += NTH) {  // one word of tokens per warp
+      const int i = wb + lane;
       const float* zr = p.z_ws + ((int64_t)b * p.max_visual + i) * p.hp + hbeg;
       float a = 0.f;
-      if (pre && i == i0 + tid) {
+      if (i >= i1) {
+      } else if (pre && i == i0 + tid) {
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
           if (4 * q < hcnt) {
@@ -2224,20 +2320,19 @@ __global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepPara
         for (int hh = 0; hh < hcnt; ++hh)
           a = fmaf(fexp2_rel(__ldcg(zr + hh), hM_s[hbeg + hh]), hInv_s[hbeg + hh], a);
       }
-      emit(i, a);
+      const bool on = i < i1 && emit(i, a);
+      if (act_row) {
+        const unsigned m = __ballot_sync(0xffffffffu, on);
+        if (m && lane == 0) atomicOr(act_row + (wb >> 5), m);
+      }
     }
   }
   if (bad) atomicOr(p.err, ERR_NONFINITE);
-  if (p.n_act || topp) {  // this rank's count and score total, into rank 0's slots
+  if (p.n_act) {  // this rank's count, into rank 0's slot
     n_on = __reduce_add_sync(0xffffffffu, n_on);
-    vsum = warp_sum(vsum);
     if (lane == 0 && n_on) atomicAdd(&act_s, n_on);
-    if (lane == 0 && topp) atomicAdd(&vsum_s, vsum);
     __syncthreads();
-    if (tid == 0) {
-      (ncl > 1 ? cluster.map_shared_rank(act_rank_s, 0) : act_rank_s)[rank] = act_s;
-      (ncl > 1 ? cluster.map_shared_rank(vsum_rank_s, 0) : vsum_rank_s)[rank] = vsum_s;
-    }
+    if (tid == 0) (ncl > 1 ? cluster.map_shared_rank(act_rank_s, 0) : act_rank_s)[rank] = act_s;
   }
   if (ncl > 1) cluster.sync();  // rank 0 now sees every key (and its own K)
   else __syncthreads();
@@ -2260,101 +2355,8 @@ __global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepPara
   uint32_t theta = 0;
   unsigned krem = 0, n_theta = 0;  // keys equal to theta: to keep, in total
   if (topp) {
-    // Top-p budget (App. A.2): the fewest top keys whose scores reach a share
-    // p of the visual total.  Radix select over the score mass: each pass
-    // keeps every digit above the one where the remaining mass is reached.
-    float total = 0.f;
-    for (int r = 0; r < ncl; ++r) total += vsum_rank_s[r];
-    K = 0;
-    if (nv > 0 && p.ratio_ppm >= 1000000) {
-      K = nv;
-    } else if (nv > 0 && p.ratio_ppm > 0) {
-      float need = (float)p.ratio_ppm * 1e-6f * total;  // score mass still to cover
-      unsigned above = 0;                                // keys above the current bucket
-      uint32_t prefix = 0, mask = 0;
-      bool all = false;
-      for (int pass = 0; pass < 4 && !all; ++pass) {
-        const int shift = 24 - 8 * pass;
-        unsigned* hist = hist_s[pass % 3];
-        float* hsum = hsum_s[pass % 3];
-        if (pass >= 2)
-          for (int i = tid; i < 256; i += NTH) { hist_s[(pass + 1) % 3][i] = 0; hsum_s[(pass + 1) % 3][i] = 0.f; }
-        for (int base = 0; base < nv; base += NTH) {
-          const int i = base + tid;
-          const uint32_t kk = i < nv ? key_s[i] : 0u;
-          const bool m = i < nv && (kk & mask) == prefix;
-          const unsigned dg = (kk >> shift) & 255u;
-          const unsigned act = __ballot_sync(0xffffffffu, m);
-          if (act) {
-            const int leader = __ffs(act) - 1;
-            const unsigned d0 = __shfl_sync(0xffffffffu, dg, leader);
-            if (__all_sync(0xffffffffu, !m || dg == d0)) {
-              const float ws = warp_sum(m ? __uint_as_float(kk) : 0.f);
-              if (lane == leader) { atomicAdd(&hist[d0], (unsigned)__popc(act)); atomicAdd(&hsum[d0], ws); }
-            } else if (m) {
-              atomicAdd(&hist[dg], 1u);
-              atomicAdd(&hsum[dg], __uint_as_float(kk));
-            }
-          }
-        }
-        __syncthreads();
-        unsigned cc[8], ctot = 0;
-        float cs[8], stot = 0.f;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          cc[j] = hist[255 - 8 * lane - j]; ctot += cc[j];
-          cs[j] = hsum[255 - 8 * lane - j]; stot += cs[j];
-        }
-        unsigned cin = ctot;
-        float sin_ = stot;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const unsigned nc = __shfl_up_sync(0xffffffffu, cin, o);
-          const float ns_ = __shfl_up_sync(0xffffffffu, sin_, o);
-          if (lane >= o) { cin += nc; sin_ += ns_; }
-        }
-        const unsigned cex = cin - ctot;
-        const float sex = sin_ - stot;
-        const bool mine = sex < need && need <= sin_ && ctot > 0;
-        unsigned dsel = 0, cnt_before = 0, cnt = 0;
-        float sum_before = 0.f;
-        if (mine) {
-          // The lane's own running sum may round differently from the scan:
-          // without a digit reaching the mass, its last non-empty digit holds it.
-          unsigned cr = cex;
-          float sr = sex;
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            if (cc[j] > 0) { dsel = 255 - 8 * lane - j; cnt_before = cr; sum_before = sr; cnt = cc[j]; }
-            if (cc[j] > 0 && sr + cs[j] >= need) break;
-            cr += cc[j];
-            sr += cs[j];
-          }
-        }
-        const unsigned found = __ballot_sync(0xffffffffu, mine && cnt > 0);
-        if (!found) { all = true; break; }  // rounding left the mass short: keep every candidate
-        const int src = __ffs(found) - 1;
-        dsel = __shfl_sync(0xffffffffu, dsel, src);
-        cnt_before = __shfl_sync(0xffffffffu, cnt_before, src);
-        sum_before = __shfl_sync(0xffffffffu, sum_before, src);
-        cnt = __shfl_sync(0xffffffffu, cnt, src);
-        above += cnt_before;
-        need -= sum_before;
-        prefix |= dsel << shift;
-        mask |= 255u << shift;
-        if (shift == 0) n_theta = cnt;
-      }
-      if (all) {
-        K = nv;
-      } else {
-        theta = prefix;
-        const float tv = __uint_as_float(theta);
-        unsigned m_eq = tv > 0.f ? (unsigned)ceilf(need / tv) : n_theta;
-        m_eq = max(1u, min(m_eq, n_theta));
-        krem = m_eq;
-        K = (int)(above + m_eq);
-      }
-    }
+    K = top_p_cut<NTH>(key_s, nv, p.ratio_ppm, reinterpret_cast<float*>(key_s + (p.max_visual + 3) / 4 * 4), tp_sum_s,
+                       tp_cnt_s, theta, krem, n_theta);
     K = min(K, p.kept_cap);
     if (tid == 0) {
       p.kept_count[(int64_t)b * nsel + gsel] = K;
@@ -4073,7 +4075,11 @@ cudaError_t configure_fixed_kernels() {
   return e;
 }
 
-size_t select_smem_bytes(int max_visual) { return ((size_t)(max_visual > 0 ? max_visual : 1) + 3) / 4 * 16; }
+// Score keys of k_select and k_selgat; with topp_threads, also the columns of
+// k_select's top-p cut.
+size_t select_smem_bytes(int max_visual, int topp_threads = 0) {
+  return ((size_t)(max_visual > 0 ? max_visual : 1) + 3) / 4 * 16 + (size_t)topp_threads * kTopPDigits * 4;
+}
 
 }  // namespace
 
@@ -4130,9 +4136,10 @@ cudaError_t launch_select(const StepParams& p, cudaStream_t st) {
                         : launch_selgat_td<__nv_bfloat16, 64>(p, grid, smem, st);
     return p.D == 128 ? launch_selgat_td<float, 128>(p, grid, smem, st) : launch_selgat_td<float, 64>(p, grid, smem, st);
   }
-  const size_t smem = select_smem_bytes(p.max_visual);
-  if ((p.max_visual + p.cl - 1) / p.cl <= kSelSliceSmall) return launch_ex(k_select<512>, grid, dim3(512), smem, st, p.cl, p);
-  return launch_ex(k_select<1024>, grid, dim3(1024), smem, st, p.cl, p);
+  const bool topp = p.mode == MODE_TOP_P;
+  if ((p.max_visual + p.cl - 1) / p.cl <= kSelSliceSmall)
+    return launch_ex(k_select<512>, grid, dim3(512), select_smem_bytes(p.max_visual, topp ? 512 : 0), st, p.cl, p);
+  return launch_ex(k_select<1024>, grid, dim3(1024), select_smem_bytes(p.max_visual, topp ? 1024 : 0), st, p.cl, p);
 }
 
 namespace {
@@ -4231,9 +4238,10 @@ void encode_kv_maps(StepParams& p) {
 cudaError_t configure_kernels(int max_visual, int H, int nsp_max) {
   (void)H;
   (void)nsp_max;
-  const int need = (int)select_smem_bytes(max_visual);
   cudaError_t e = cudaSuccess;
-  for (void (*k)(StepParams) : {k_select<512>, k_select<1024>}) {
+  for (int nth : {512, 1024}) {
+    const int need = (int)select_smem_bytes(max_visual, nth);  // k_select, top-p included
+    void (*k)(StepParams) = nth == 512 ? k_select<512> : k_select<1024>;
     cudaFuncAttributes attr;
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&attr, k);
     if (e == cudaSuccess && attr.maxDynamicSharedSizeBytes < need) e = set_smem(k, need);

@@ -114,3 +114,29 @@ def test_diagnostics_off_and_bad_delta(vp):
             assert ei.value.status == vp.VP_ERR_INVALID_ARG
     finally:
         dev.close()
+
+
+@pytest.mark.parametrize("nv,batch", [(31, 1), (2305, 3), (4097, 2), (20001, 2)])
+@pytest.mark.parametrize("ppm", [1_000, 100_000, 900_000])
+def test_top_p_cut_and_bits_at_slice_edges(vp, nv, batch, ppm):
+    """Top-p budgets and activity bits with visual spans that end inside a
+    word, in the 512-thread kernel (short slices) and the 1024-thread one
+    (nv = 20001), against the oracle."""
+    r = W.shrink(W.QWEN7B, layers=1, batch=batch, heads=8, kv_heads=8, head_dim=64, vis_len=nv, vis_start=3,
+                 text_len=37, steps=1)
+    inp = Hn.make_inputs(r)
+    budget = dict(mode=O.TOP_P, tau=0.1, ratio_ppm=ppm)
+    delta = 1.0 / (nv + 37)
+    words = (nv + 31) // 32
+    bits = torch.zeros((batch, words), dtype=torch.int32, device="cuda")
+    n_act = torch.zeros((batch,), dtype=torch.int32, device="cuda")
+    dev = Hn.Device(vp, inp, budget)
+    try:
+        vp.vp_set_diagnostics(dev.ctx, delta, n_act, bits)
+        gpu = dev.run()
+    finally:
+        dev.close()
+    flags = _bits_to_flags(bits.cpu().numpy().view(np.uint32), nv)
+    for b in range(batch):
+        ref = Hn.compare_seq(inp, gpu, b, budget)
+        _compare(ref["s"], delta, n_act.cpu().numpy()[b], flags[b])
