@@ -1695,6 +1695,10 @@ __global__ void __launch_bounds__(kTcThreads, NS <= 3 ? 2 : 1) k_score_tc(const 
 // visual rows in their order, then the rows after the span (vp_compact_kv).
 // Each thread copies 16-byte pieces; a warp covers whole rows, so the reads
 // of consecutive kept rows and of the text rows are coalesced per row.
+// Bound by HBM; a row costs three dependent trips (kept index, page, data), so
+// a thread keeps eight rows in flight: the indices of its next eight
+// rows, then their pages, then their data, then the stores (one row at a time
+// before).  8 x 4 x 2561 rows of 256 bytes, read and written: 12.5 -> 11.1 us.
 // ---------------------------------------------------------------------------
 constexpr int kCompactRows = 128;  // destination rows per CTA
 
@@ -1718,34 +1722,49 @@ __global__ void __launch_bounds__(256) k_compact(const __grid_constant__ Compact
   const int r0 = blockIdx.x * kCompactRows, r1 = min(Tn, r0 + kCompactRows);
   const char* src = static_cast<const char*>(c.src.data);
   char* dst = static_cast<char*>(c.dst);
-  for (int t = r0 + threadIdx.x / ppr; t < r1; t += rpi) {
-    const int piece = threadIdx.x % ppr;
-    int pos;  // source row
-    if (t < vs) {
-      pos = t;
-    } else if (t < vs + K) {
-      const int i = __ldcg(c.kept_idx + (int64_t)b * c.kept_cap + (t - vs));
-      pos = (i >= 0 && i < nv) ? vs + i : -1;
-      if (pos < 0) e |= ERR_KEPT;
-    } else {
-      pos = t - K + nv;
+  const int piece = threadIdx.x % ppr;
+  constexpr int U = 8;  // rows of a thread in flight
+  for (int t0 = r0 + threadIdx.x / ppr; t0 < r1; t0 += U * rpi) {
+    int pos[U], page[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {  // source row; -1 for none
+      const int t = t0 + u * rpi;
+      pos[u] = -1;
+      if (t >= r1) continue;
+      if (t < vs) pos[u] = t;
+      else if (t < vs + K) pos[u] = __ldcg(c.kept_idx + (int64_t)b * c.kept_cap + (t - vs));
+      else pos[u] = t - K + nv;
     }
-    const char* row = nullptr;
-    if (pos >= 0) {
-      if (c.paged) {
-        const int lp = pos >> c.page_shift;
-        const int page = lp < c.src.max_pages ? __ldg(c.src.block_table + (int64_t)b * c.src.max_pages + lp) : -1;
-        if (page >= 0 && page < c.src.num_pages)
-          row = src + ((int64_t)page * c.src.sb + (int64_t)g * c.src.sh + (int64_t)(pos & (c.page_size - 1)) * c.src.st) * c.esz;
-        else
-          e |= ERR_PAGE;
-      } else {
-        row = src + ((int64_t)b * c.src.sb + (int64_t)g * c.src.sh + (int64_t)pos * c.src.st) * c.esz;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int t = t0 + u * rpi;
+      if (t >= vs && t < vs + K && t < r1) {
+        const int i = pos[u];
+        pos[u] = i >= 0 && i < nv ? vs + i : -1;
+        if (pos[u] < 0) e |= ERR_KEPT;
+      }
+      page[u] = b;
+      if (c.paged && pos[u] >= 0) {
+        const int lp = pos[u] >> c.page_shift;
+        page[u] = lp < c.src.max_pages ? __ldg(c.src.block_table + (int64_t)b * c.src.max_pages + lp) : -1;
       }
     }
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (row) v = __ldg(reinterpret_cast<const uint4*>(row) + piece);
-    reinterpret_cast<uint4*>(dst + ((int64_t)b * c.dsb + (int64_t)g * c.dsh + (int64_t)t * c.dst_t) * c.esz)[piece] = v;
+    uint4 v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      v[u] = make_uint4(0u, 0u, 0u, 0u);
+      if (pos[u] < 0) continue;
+      if (c.paged && (page[u] < 0 || page[u] >= c.src.num_pages)) { e |= ERR_PAGE; continue; }
+      const int64_t row = c.paged ? pos[u] & (c.page_size - 1) : pos[u];
+      const char* a = src + ((int64_t)page[u] * c.src.sb + (int64_t)g * c.src.sh + row * c.src.st) * c.esz;
+      v[u] = __ldg(reinterpret_cast<const uint4*>(a) + piece);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int t = t0 + u * rpi;
+      if (t < r1)
+        reinterpret_cast<uint4*>(dst + ((int64_t)b * c.dsb + (int64_t)g * c.dsh + (int64_t)t * c.dst_t) * c.esz)[piece] = v[u];
+    }
   }
   if (e) atomicOr(c.err, e);
 }
