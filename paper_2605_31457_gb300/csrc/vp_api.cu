@@ -359,8 +359,7 @@ vp_status vp_decode_gather(vp_ctx* ctx, int32_t batch, const void* q,
   p.gpart_o = ctx->gpart_o; p.gpart_st = ctx->gpart_st; p.tickets = ctx->tickets; p.err = ctx->err;
   p.mt_o = ctx->mt_o; p.mt_st = ctx->mt_st; p.hmax = ctx->hmax;
   // Score splits as planned for the decode step; their weight covers the
-  // cache outside the visual span plus the kept rows.  The merge of the
-  // splits is the chunk gather with no kept chunks.
+  // cache outside the visual span plus the kept rows.
   const vp::Plan pl = vp::make_plan(batch, Hkv, D, ctx->num_sms, c.max_visual, c.max_seq, 0, granularity);
   p.hp = ctx->lay.hp;
   p.ns = pl.ns; p.nsp_max = ctx->lay.nsp_max; p.cl = 1;
@@ -369,10 +368,6 @@ vp_status vp_decode_gather(vp_ctx* ctx, int32_t batch, const void* q,
     if (w < 1) w = 1;
     p.split_w = (int)((w + pl.ns - 1) / pl.ns);
   }
-  p.nk = 0; p.nk_max = ctx->lay.nk_max;
-  p.nm = pl.ns > 1 ? (D / 16 < 8 ? D / 16 : 8) : 0;
-  p.nc = p.nm > 0 ? p.nm : 1;
-  p.gslice = 0;
   vp::encode_kv_maps(p);
   if (!p.use_tma)
     return fail(ctx, VP_ERR_UNSUPPORTED, "vp_decode_gather: the cache layout needs the bulk-tensor path "
@@ -380,7 +375,7 @@ vp_status vp_decode_gather(vp_ctx* ctx, int32_t batch, const void* q,
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   cudaError_t e = vp::launch_score(p, st);
   if (e != cudaSuccess) return cuda_fail(ctx, "vp_decode_gather: score kernel launch", e);
-  e = vp::launch_gather(p, st);
+  e = vp::launch_merge(p, st);
   if (e != cudaSuccess) return cuda_fail(ctx, "vp_decode_gather: merge kernel launch", e);
   ctx->last_score_path = VP_SCORE_MMA;
   ctx->last_kernels = 2;

@@ -286,6 +286,8 @@ cudaError_t launch_compact(const CompactParams& c, cudaStream_t s);
 cudaError_t launch_score(const StepParams& p, cudaStream_t s);
 cudaError_t launch_select(const StepParams& p, cudaStream_t s);
 cudaError_t launch_gather(const StepParams& p, cudaStream_t s);
+// Layers after the anchor layer: merges the score splits and writes the output.
+cudaError_t launch_merge(const StepParams& p, cudaStream_t s);
 // Kernel attributes: raises (never lowers) the select kernel's dynamic
 // shared-memory limit for these shapes and sets the other kernels' limits.
 cudaError_t configure_kernels(int max_visual, int H, int nsp_max);

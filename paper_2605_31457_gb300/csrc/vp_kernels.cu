@@ -2832,20 +2832,13 @@ __global__ void __launch_bounds__(32 * kGmWarps) k_gather_mma(const __grid_const
   const Seq sq = load_seq(p, b, false);
   // (b) first: it reads only the score kernel's partials, complete before the
   // select kernel lets this grid start.  Its shared memory is the ring's.
-  // After the anchor layer no select kernel runs in between: there (b)
-  // waits for the score kernel like everything else.
-  if (c < p.nm && !p.anchor) {
+  if (c < p.nm) {
     gather_text_slice<D, GM, C::THREADS>(p, c, hrow0, tw, tl);
     fence_proxy_async();
     __syncthreads();
   }
   pdl_wait();
   pdl_trigger();
-  if (c < p.nm && p.anchor) {
-    gather_text_slice<D, GM, C::THREADS>(p, c, hrow0, tw, tl);
-    fence_proxy_async();
-    __syncthreads();
-  }
   const int64_t pbase = ((int64_t)b * p.Hkv + g) * p.nk_max;
   unsigned err = 0;
   bool timed_out = false;
@@ -3111,6 +3104,78 @@ __global__ void __launch_bounds__(32 * kGmWarps) k_gather_mma(const __grid_const
   if (timed_out) err |= ERR_TIMEOUT;
   if (err) atomicOr(p.err, err);
   if (!lone) gather_finish<__nv_bfloat16, D, GM, C::THREADS>(p, b, g, hrow0, pbase, tw, fin, last);
+}
+
+// ---------------------------------------------------------------------------
+// k_merge (bf16, layers after the anchor layer): grid (H, B), 128 threads.
+// Combines the score splits' partials of one query head in log-sum-exp form
+// and writes the output.  Bound by latency: one round trip to L2.  A group of
+// D / 4 lanes holds a whole output row (4 dimensions per lane) and takes every
+// (128 / lanes)-th split, its records and partial rows requested together; the
+// groups meet in shared memory once.  (The chunk gather with no kept chunks,
+// which served this before, walked the splits' records serially per head and
+// passed its slices through global memory and a ticket, 10.5 us a call: a step
+// of 28 layers of the B = 1 decode with 27 such layers went 402 -> 236 us.)
+// ---------------------------------------------------------------------------
+constexpr int kMergeThreads = 128;
+
+template <int D>
+__global__ void __launch_bounds__(kMergeThreads) k_merge(const __grid_constant__ StepParams p) {
+  constexpr int LPR = D / 4, NG = kMergeThreads / LPR;  // lanes per row, groups
+  constexpr int U = 10;                                 // splits of a group in flight
+  __shared__ float4 acc_s[NG][LPR];
+  __shared__ float2 st_s[NG];
+  // The next kernel is the next layer's score kernel, which waits for this one
+  // before it reads a kept set or writes the workspace: it may start now.
+  pdl_trigger();
+  pdl_wait();
+  const int64_t row = (int64_t)blockIdx.y * p.H + blockIdx.x;
+  const int sg = threadIdx.x / LPR, l = threadIdx.x % LPR, ns = p.ns;
+  const float* st = p.split_st + row * p.nsp_max * ST_N;
+  const float* so = p.split_o + row * p.nsp_max * D + 4 * l;
+  float M = -CUDART_INF_F, L = 0.f;
+  float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int s0 = sg; s0 < ns; s0 += U * NG) {
+    float2 r[U];  // {max, sum}
+    float4 o[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int s = s0 + u * NG;
+      r[u] = s < ns ? __ldcg(reinterpret_cast<const float2*>(st + (int64_t)s * ST_N)) : make_float2(-CUDART_INF_F, 0.f);
+      o[u] = s < ns ? __ldcg(reinterpret_cast<const float4*>(so + (int64_t)s * D)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float Mn = M;
+#pragma unroll
+    for (int u = 0; u < U; ++u) Mn = fmaxf(Mn, r[u].x);
+    const float f = exp2_rel(M, Mn);
+    M = Mn;
+    L *= f;
+    a.x *= f; a.y *= f; a.z *= f; a.w *= f;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const float w = exp2_rel(r[u].x, M);
+      L = fmaf(w, r[u].y, L);
+      a.x = fmaf(w, o[u].x, a.x); a.y = fmaf(w, o[u].y, a.y); a.z = fmaf(w, o[u].z, a.z); a.w = fmaf(w, o[u].w, a.w);
+    }
+  }
+  acc_s[sg][l] = a;
+  if (l == 0) st_s[sg] = make_float2(M, L);
+  __syncthreads();
+  if (sg) return;
+#pragma unroll
+  for (int k = 1; k < NG; ++k) M = fmaxf(M, st_s[k].x);
+  float den = 0.f;
+  float4 n = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int k = 0; k < NG; ++k) {
+    const float w = exp2_rel(st_s[k].x, M);
+    const float4 v = acc_s[k][l];
+    den = fmaf(w, st_s[k].y, den);
+    n.x = fmaf(w, v.x, n.x); n.y = fmaf(w, v.y, n.y); n.z = fmaf(w, v.z, n.z); n.w = fmaf(w, v.w, n.w);
+  }
+  const float inv = den > 0.f ? 1.f / den : 0.f;
+  *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + row * D + 4 * l) =
+      make_uint2(pack_bf16(n.x * inv, n.y * inv), pack_bf16(n.z * inv, n.w * inv));
 }
 
 // ---------------------------------------------------------------------------
@@ -4002,7 +4067,7 @@ cudaError_t launch_gather_td(const StepParams& p, cudaStream_t st) {
   if (sizeof(T) == 2) {
     // A single ring slot when no chunk can hold more than one tile per warp.
     const int kmax = min(p.kept_cap, p.max_visual);
-    const bool one = p.nk == 0 || (kmax + p.nk - 1) / p.nk <= GmCfg<D, 1, 1>::MAX_CHUNK;
+    const bool one = (kmax + p.nk - 1) / p.nk <= GmCfg<D, 1, 1>::MAX_CHUNK;
     const long long n = (long long)p.nc * p.Hkv * p.B;
     if (p.G <= 8) {
       if (one) return launch_ex(k_gather_mma<D, 1, 1>, grid, dim3(32 * kGmWarps), GmCfg<D, 1, 1>::SMEM, st, 1, p);
@@ -4111,6 +4176,10 @@ cudaError_t launch_gather(const StepParams& p, cudaStream_t st) {
   if (p.dtype == 0)
     return p.D == 128 ? launch_gather_td<__nv_bfloat16, 128>(p, st) : launch_gather_td<__nv_bfloat16, 64>(p, st);
   return p.D == 128 ? launch_gather_td<float, 128>(p, st) : launch_gather_td<float, 64>(p, st);
+}
+
+cudaError_t launch_merge(const StepParams& p, cudaStream_t st) {
+  return launch_ex(p.D == 128 ? k_merge<128> : k_merge<64>, dim3(p.H, p.B), dim3(kMergeThreads), 0, st, 1, p);
 }
 
 cudaError_t launch_compact(const CompactParams& c, cudaStream_t st) {
