@@ -366,7 +366,7 @@ vp_status vp_decode_gather(vp_ctx* ctx, int32_t batch, const void* q,
   {
     long long w = 2LL * ((c.max_seq + 31) / 32 - c.max_visual / 32 + (kept_cap + 31) / 32);
     if (w < 1) w = 1;
-    p.split_w = (int)((w + pl.ns - 1) / pl.ns);
+    p.split_w = vp::split_floor(pl, batch, Hkv, ctx->num_sms, false, (int)((w + pl.ns - 1) / pl.ns));
   }
   vp::encode_kv_maps(p);
   if (!p.use_tma)

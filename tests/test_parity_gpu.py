@@ -91,6 +91,27 @@ def test_per_kv_head_selection(vp, budget):
     Hn.check_all(vp, Hn.make_inputs(r), budget)
 
 
+@pytest.mark.parametrize("score_path", [1, 2])
+@pytest.mark.parametrize("text", [(1, 129, 700), (64, 2000, 31)])
+def test_context_with_headroom(vp, score_path, text):
+    """Sequences far shorter than the context's max_seq: the splits of a grid
+    of one wave spread over them, some of one tile or none."""
+    r = small(text_len=text, vis_start=(0, 13, 31))
+    inp = Hn.make_inputs(r, t_cap=16000)
+    dev = Hn.Device(vp, inp, r.budget, max_seq=16000, score_path=score_path)
+    try:
+        gpu = dev.run()
+        vp.vp_decode_gather(dev.ctx, dev.B, dev.q, dev.kc, dev.vc, dev.span, dev.tl, dev.kept, dev.kept_cap, dev.count,
+                            dev.out)  # the anchor's set on the anchor's inputs: the same attention
+        vp.vp_check_errors(dev.ctx)
+        again = dev.out.float().cpu().numpy()
+    finally:
+        dev.close()
+    for b in range(r.batch):
+        Hn.compare_seq(inp, gpu, b, r.budget)
+    np.testing.assert_allclose(again, gpu["out"], rtol=0, atol=2e-2)
+
+
 def test_paged_cache(vp):
     r = small(batch=4, vis_len=(300, 577, 64, 1000), vis_start=(0, 13, 40, 0),
               text_len=(517, 70, 129, 33), paged=True, page_size=16)
