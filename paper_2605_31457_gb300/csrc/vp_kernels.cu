@@ -1770,45 +1770,108 @@ __global__ void __launch_bounds__(256) k_compact(const __grid_constant__ Compact
 }
 
 // ---------------------------------------------------------------------------
-// k_score_f32 (fp32 caches): lane-per-token dot products on the FMA pipes,
-// lane-per-dimension P.V; the same partials as k_score_mma.
+// k_score_f32 (fp32 caches): the partials of k_score_mma on the FMA pipes, in
+// full float32.  A warp takes a batch of token rows at a time: D / 4 lanes
+// hold a row (one 16-byte piece each: every load covers whole rows), so all of
+// a batch's K rows, and V rows for text, are in flight together.  The dot
+// products of a batch with the G heads are reduced over the lanes by halving
+// the (head, token) set at each exchange, heads first: about one shuffle per
+// value instead of five, and every lane ends with whole logits of one head,
+// whose statistics it keeps.  For P.V each lane owns four dimensions of every
+// head and reads the batch's probabilities from shared memory.  Bound by
+// memory latency at small calls, by HBM above.  (One lane per token row before:
+// 32 sectors per load and a serial walk over D.  4 sequences, 28/4 heads, up
+// to 1296 + 1500 tokens: the call 53.9 -> 24.0 us; the tiny reference, 8/2
+// heads of 64 dimensions, 576 + 128 tokens: 19.9 -> 13.6 us.)
 // ---------------------------------------------------------------------------
 template <int D, int GM>
+struct F32Batch {  // token rows (per row slot of the warp) of a batch: visual, text
+  static constexpr int VIS = GM == 16 ? 4 : 8, TXT = GM == 16 ? 2 : GM == 4 && D == 128 ? 8 : 4;
+};
+
+template <int D, int GM>
 struct F32Smem {
+  static constexpr int RPW = 128 / D;  // rows a warp holds side by side
   float q[GM][D];
-  float pr[kWarps][GM][32];
-  const float* vrow[kWarps][32];
+  float pr[kWarps][F32Batch<D, GM>::TXT * RPW][GM];
   float wst[kWarps][GM][ST_N];
   float ow[kWarps][GM][D];
   ScoreTail<GM, D> tail;
 };
 
-template <int D, int GM>
-__device__ __forceinline__ void dot_row_f32(const float* row, const float (*q_s)[D], float (&z)[GM]) {
+constexpr int ilog2(int x) { return x <= 1 ? 0 : 1 + ilog2(x / 2); }
+
+// Logits of NT token rows (kf: this lane's piece of each) against the GM heads
+// in q_s, reduced over the LPR = D / 4 lanes of the row: lane l gets the
+// NT >> TS values of head f32_head(l) at rows f32_row(l) + 0, 1, ...
+template <int D, int GM, int NT>
+struct F32Dot {
+  static constexpr int LPR = D / 4, HS = ilog2(GM), TS = ilog2(LPR) - HS, TPL = NT >> TS;
+  static_assert(HS >= 1 && TS >= 0 && TPL >= 1, "the lanes of a row split heads, then tokens");
+  static __device__ __forceinline__ int head(int l) {
+    int h = 0;
 #pragma unroll
-  for (int h = 0; h < GM; ++h) z[h] = 0.f;
-#pragma unroll 4
-  for (int d0 = 0; d0 < D; d0 += 4) {
-    float kf[4];
-    load_f<4>(row + d0, kf);
-#pragma unroll
-    for (int h = 0; h < GM; ++h) {
-      const float4 qv = *reinterpret_cast<const float4*>(&q_s[h][d0]);
-      z[h] = fmaf(qv.x, kf[0], z[h]);
-      z[h] = fmaf(qv.y, kf[1], z[h]);
-      z[h] = fmaf(qv.z, kf[2], z[h]);
-      z[h] = fmaf(qv.w, kf[3], z[h]);
-    }
+    for (int k = 0; k < HS; ++k) h |= (l & (LPR >> (k + 1))) ? GM >> (k + 1) : 0;
+    return h;
   }
-}
+  static __device__ __forceinline__ int row(int l) {
+    int t = 0;
+#pragma unroll
+    for (int k = 0; k < TS; ++k) t |= (l & (LPR >> (HS + k + 1))) ? NT >> (k + 1) : 0;
+    return t;
+  }
+  static __device__ __forceinline__ int lane_of(int h) {  // a lane of the row that holds head h
+    int l = 0;
+#pragma unroll
+    for (int k = 0; k < HS; ++k) l |= (h & (GM >> (k + 1))) ? LPR >> (k + 1) : 0;
+    return l;
+  }
+  static __device__ __forceinline__ float swap_add(float lo, float hi, int o, int l) {
+    const bool up = (l & o) != 0;
+    return (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, o);
+  }
+  static __device__ __forceinline__ void run(const float4 (&kf)[NT], const float (*q_s)[D], int l, float (&z)[TPL]) {
+    float v[NT][GM / 2];
+#pragma unroll
+    for (int j = 0; j < GM / 2; ++j) {
+      const float4 qa = *reinterpret_cast<const float4*>(&q_s[j][4 * l]);
+      const float4 qb = *reinterpret_cast<const float4*>(&q_s[j + GM / 2][4 * l]);
+#pragma unroll
+      for (int t = 0; t < NT; ++t) {
+        const float a = fmaf(qa.x, kf[t].x, fmaf(qa.y, kf[t].y, fmaf(qa.z, kf[t].z, qa.w * kf[t].w)));
+        const float b = fmaf(qb.x, kf[t].x, fmaf(qb.y, kf[t].y, fmaf(qb.z, kf[t].z, qb.w * kf[t].w)));
+        v[t][j] = swap_add(a, b, LPR / 2, l);
+      }
+    }
+#pragma unroll
+    for (int k = 1; k < HS; ++k)
+#pragma unroll
+      for (int t = 0; t < NT; ++t)
+#pragma unroll
+        for (int j = 0; j < (GM >> (k + 1)); ++j)
+          v[t][j] = swap_add(v[t][j], v[t][j + (GM >> (k + 1))], LPR >> (k + 1), l);
+#pragma unroll
+    for (int k = 0; k < TS; ++k)
+#pragma unroll
+      for (int t = 0; t < (NT >> (k + 1)); ++t)
+        v[t][0] = swap_add(v[t][0], v[t + (NT >> (k + 1))][0], LPR >> (HS + k + 1), l);
+#pragma unroll
+    for (int t = 0; t < TPL; ++t) z[t] = v[t][0];
+  }
+};
 
 template <int D, int GM>
-__global__ void __launch_bounds__(kThreads) k_score_f32(const __grid_constant__ StepParams p) {
-  constexpr int DPL = D / 32;
+__global__ void __launch_bounds__(kThreads, 2) k_score_f32(const __grid_constant__ StepParams p) {
+  using Sm = F32Smem<D, GM>;
+  constexpr int LPR = D / 4, RPW = Sm::RPW, NV = F32Batch<D, GM>::VIS, NX = F32Batch<D, GM>::TXT;
+  using DV = F32Dot<D, GM, NV>;
+  using DX = F32Dot<D, GM, NX>;
+  constexpr int TOKBITS = 1 << DV::TS;  // lanes [0, TOKBITS) of a row share a head
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  auto& sm = *reinterpret_cast<F32Smem<D, GM>*>(smem_raw);
+  auto& sm = *reinterpret_cast<Sm*>(smem_raw);
   const int s = blockIdx.x, g = blockIdx.y, b = blockIdx.z;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int l = lane % LPR, rs = lane / LPR;  // piece of the row, row slot of the warp
   pdl_wait();
   const int G = p.G, H = p.H;
   const Seq sq = load_seq(p, b, s == 0 && g == 0);
@@ -1819,116 +1882,158 @@ __global__ void __launch_bounds__(kThreads) k_score_f32(const __grid_constant__ 
   }
   __syncthreads();
   const SplitRange rg = split_range(sq, s, p.ns);
-
-  float m_v[GM], l1v[GM], ltv[GM], m_t[GM], l1t[GM], ltt[GM], acc[GM][DPL];
-#pragma unroll
-  for (int h = 0; h < GM; ++h) {
-    m_v[h] = m_t[h] = -CUDART_INF_F;
-    l1v[h] = ltv[h] = l1t[h] = ltt[h] = 0.f;
-#pragma unroll
-    for (int j = 0; j < DPL; ++j) acc[h][j] = 0.f;
-  }
+  const int head = DV::head(l);  // the head of this lane's logits (the same for both batch sizes)
+  const bool hv = head < G;
+  const float inv_tau = p.inv_tau;
   unsigned err = 0;
+  auto piece = [&](const float* row) {
+    return row ? __ldg(reinterpret_cast<const float4*>(row) + l) : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
 
-  for (int base = rg.va + warp * 32; base < rg.vb; base += kWarps * 32) {
-    const int i = base + lane;
-    bool valid = i < rg.vb;
-    float z[GM];
-    if (valid) {
-      const float* row = kv_row<float>(p.k, p, b, g, sq.vs + i);
-      if (row) dot_row_f32<D, GM>(row, sm.q, z); else { valid = false; err |= ERR_PAGE; }
+  // Visual tokens: logits to the workspace, statistics per lane.
+  float m_v = -CUDART_INF_F, l1v = 0.f, ltv = 0.f;
+  for (int base = rg.va + warp * NV * RPW; base < rg.vb; base += kWarps * NV * RPW) {
+    float4 kf[NV];
+    unsigned ok = 0;
+#pragma unroll
+    for (int t = 0; t < NV; ++t) {
+      const int i = base + t * RPW + rs;
+      const float* row = nullptr;
+      if (i < rg.vb) {
+        row = kv_row<float>(p.k, p, b, g, sq.vs + i);
+        if (!row) err |= ERR_PAGE;
+      }
+      ok |= (unsigned)(row != nullptr) << t;
+      kf[t] = piece(row);
+    }
+    float z[DV::TPL];
+    DV::run(kf, sm.q, l, z);
+    const int t0 = DV::row(l);
+    float mn = m_v;
+#pragma unroll
+    for (int t = 0; t < DV::TPL; ++t) {
+      const int i = base + (t0 + t) * RPW + rs;
+      z[t] = ((ok >> (t0 + t)) & 1u) ? z[t] * p.c_log2 : -CUDART_INF_F;
+      if (i < rg.vb && hv) p.z_ws[((int64_t)b * p.max_visual + i) * p.hp + g * G + head] = z[t];
+      mn = fmaxf(mn, z[t]);
+    }
+    if (mn > m_v) {
+      l1v *= exp2_rel(m_v, mn);
+      ltv *= exp2_tau(m_v, mn, inv_tau);
+      m_v = mn;
     }
 #pragma unroll
-    for (int h = 0; h < GM; ++h) {
-      if (h >= G) break;
-      const float zz = valid ? z[h] * p.c_log2 : -CUDART_INF_F;
-      if (i < rg.vb) p.z_ws[((int64_t)b * p.max_visual + i) * p.hp + g * G + h] = zz;
-      const float mn = fmaxf(m_v[h], warp_max(zz));
-      if (mn > m_v[h]) {
-        l1v[h] *= exp2_rel(m_v[h], mn);
-        ltv[h] *= exp2_tau(m_v[h], mn, p.inv_tau);
-        m_v[h] = mn;
+    for (int t = 0; t < DV::TPL; ++t)
+      if (z[t] != -CUDART_INF_F) {
+        l1v += exp2f(z[t] - m_v);
+        ltv += exp2f((z[t] - m_v) * inv_tau);
       }
-      if (valid) {
-        l1v[h] += exp2f(zz - mn);
-        ltv[h] += exp2f((zz - mn) * p.inv_tau);
-      }
-    }
   }
 
-  for (int base = rg.ta + warp * 32; base < rg.tb; base += kWarps * 32) {
-    const int ti = base + lane;
-    bool valid = ti < rg.tb;
-    const int pos = text_pos(sq, ti);
-    float z[GM];
-    const float* vrow = nullptr;
-    if (valid) {
-      const float* row = kv_row<float>(p.k, p, b, g, pos);
-      vrow = kv_row<float>(p.v, p, b, g, pos);
-      if (row && vrow) dot_row_f32<D, GM>(row, sm.q, z); else { valid = false; vrow = nullptr; err |= ERR_PAGE; }
+  // Text tokens: a running maximum per head, the same in every lane of the warp.
+  float m_t = -CUDART_INF_F, l1t = 0.f, ltt = 0.f;
+  float4 acc[GM];
+#pragma unroll
+  for (int h = 0; h < GM; ++h) acc[h] = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int base = rg.ta + warp * NX * RPW; base < rg.tb; base += kWarps * NX * RPW) {
+    float4 kf[NX], vf[NX];
+    unsigned ok = 0;
+#pragma unroll
+    for (int t = 0; t < NX; ++t) {
+      const int ti = base + t * RPW + rs;
+      const float* kr = nullptr;
+      const float* vr = nullptr;
+      if (ti < rg.tb) {
+        const int pos = text_pos(sq, ti);
+        kr = kv_row<float>(p.k, p, b, g, pos);
+        vr = kv_row<float>(p.v, p, b, g, pos);
+        if (!kr || !vr) { err |= ERR_PAGE; kr = vr = nullptr; }
+      }
+      ok |= (unsigned)(kr != nullptr) << t;
+      kf[t] = piece(kr);
+      vf[t] = piece(vr);
+    }
+    float z[DX::TPL];
+    DX::run(kf, sm.q, l, z);
+    const int t0 = DX::row(l);
+    float mn = m_t;
+#pragma unroll
+    for (int t = 0; t < DX::TPL; ++t) {
+      z[t] = ((ok >> (t0 + t)) & 1u) ? z[t] * p.c_log2 : -CUDART_INF_F;
+      mn = fmaxf(mn, z[t]);
     }
 #pragma unroll
-    for (int h = 0; h < GM; ++h) {
-      if (h >= G) break;
-      const float zz = valid ? z[h] * p.c_log2 : -CUDART_INF_F;
-      const float mn = fmaxf(m_t[h], warp_max(zz));
-      if (mn > m_t[h]) {
-        const float a = exp2_rel(m_t[h], mn);
-        l1t[h] *= a;
-        ltt[h] *= exp2_tau(m_t[h], mn, p.inv_tau);
+    for (int o = 1; o < TOKBITS; o <<= 1) mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+    if (RPW == 2) mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, 16));
+    if (__any_sync(0xffffffffu, mn > m_t)) {
+      const float f = exp2_rel(m_t, mn);
+      l1t *= f;
+      ltt *= exp2_tau(m_t, mn, inv_tau);
+      m_t = mn;
 #pragma unroll
-        for (int j = 0; j < DPL; ++j) acc[h][j] *= a;
-        m_t[h] = mn;
+      for (int h = 0; h < GM; ++h) {
+        const float fh = __shfl_sync(0xffffffffu, f, DX::lane_of(h));
+        acc[h].x *= fh; acc[h].y *= fh; acc[h].z *= fh; acc[h].w *= fh;
       }
-      float pr = 0.f;
-      if (valid) {
-        pr = exp2f(zz - mn);
-        l1t[h] += pr;
-        ltt[h] += exp2f((zz - mn) * p.inv_tau);
-      }
-      sm.pr[warp][h][lane] = pr;
     }
-    sm.vrow[warp][lane] = vrow;
+#pragma unroll
+    for (int t = 0; t < DX::TPL; ++t) {
+      float e = 0.f;
+      if (z[t] != -CUDART_INF_F) {
+        e = exp2f(z[t] - m_t);
+        l1t += e;
+        ltt += exp2f((z[t] - m_t) * inv_tau);
+      }
+      sm.pr[warp][(t0 + t) * RPW + rs][head] = e;
+    }
     __syncwarp();
-    const int nt = min(32, rg.tb - base);
-    for (int t0 = 0; t0 < nt; t0 += 4) {
-      float vv[4][DPL];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const float* vr = t0 + u < nt ? sm.vrow[warp][t0 + u] : nullptr;
-        if (vr) load_f<DPL>(vr + lane * DPL, vv[u]);
-        else {
+    for (int t = 0; t < NX; ++t) {
+      const float* pr = sm.pr[warp][t * RPW + rs];
 #pragma unroll
-          for (int j = 0; j < DPL; ++j) vv[u][j] = 0.f;
+      for (int h4 = 0; h4 < GM; h4 += 4) {
+        const float4 e = *reinterpret_cast<const float4*>(pr + h4);
+        const float pe[4] = {e.x, e.y, e.z, e.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          float4& a = acc[h4 + j];
+          a.x = fmaf(pe[j], vf[t].x, a.x); a.y = fmaf(pe[j], vf[t].y, a.y);
+          a.z = fmaf(pe[j], vf[t].z, a.z); a.w = fmaf(pe[j], vf[t].w, a.w);
         }
       }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-#pragma unroll
-        for (int h = 0; h < GM; ++h) {
-          if (h >= G) break;
-          const float pr = t0 + u < nt ? sm.pr[warp][h][t0 + u] : 0.f;
-#pragma unroll
-          for (int j = 0; j < DPL; ++j) acc[h][j] = fmaf(pr, vv[u][j], acc[h][j]);
-        }
-      }
     }
-    __syncwarp();
+    __syncwarp();  // the probabilities are read before the next batch's
   }
   pdl_trigger();
   if (err) atomicOr(p.err, err);
 
+  // Warp records: the lanes (and row slots) of a head merge theirs.
+  float M = m_v;
+#pragma unroll
+  for (int o = 1; o < TOKBITS; o <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+  if (RPW == 2) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 16));
+  l1v *= exp2_rel(m_v, M);
+  ltv *= exp2_tau(m_v, M, inv_tau);
+  auto head_sum = [&](float x) {
+#pragma unroll
+    for (int o = 1; o < TOKBITS; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if (RPW == 2) x += __shfl_xor_sync(0xffffffffu, x, 16);
+    return x;
+  };
+  l1v = head_sum(l1v); ltv = head_sum(ltv); l1t = head_sum(l1t); ltt = head_sum(ltt);
+  if ((l & (TOKBITS - 1)) == 0 && rs == 0) {
+    float* w = sm.wst[warp][head];
+    w[ST_MV] = M; w[ST_L1V] = l1v; w[ST_LTV] = ltv;
+    w[ST_MT] = m_t; w[ST_L1T] = l1t; w[ST_LTT] = ltt;
+    w[3] = w[7] = 0.f;
+  }
 #pragma unroll
   for (int h = 0; h < GM; ++h) {
-    const float a = warp_sum(l1v[h]), bb = warp_sum(ltv[h]);
-    const float c = warp_sum(l1t[h]), d = warp_sum(ltt[h]);
-    if (lane == 0) {
-      sm.wst[warp][h][ST_MV] = m_v[h]; sm.wst[warp][h][ST_L1V] = a; sm.wst[warp][h][ST_LTV] = bb;
-      sm.wst[warp][h][ST_MT] = m_t[h]; sm.wst[warp][h][ST_L1T] = c; sm.wst[warp][h][ST_LTT] = d;
-      sm.wst[warp][h][3] = sm.wst[warp][h][7] = 0.f;
+    if (RPW == 2) {
+      acc[h].x += __shfl_xor_sync(0xffffffffu, acc[h].x, 16); acc[h].y += __shfl_xor_sync(0xffffffffu, acc[h].y, 16);
+      acc[h].z += __shfl_xor_sync(0xffffffffu, acc[h].z, 16); acc[h].w += __shfl_xor_sync(0xffffffffu, acc[h].w, 16);
     }
-#pragma unroll
-    for (int j = 0; j < DPL; ++j) sm.ow[warp][h][lane * DPL + j] = acc[h][j];
+    if (rs == 0) *reinterpret_cast<float4*>(&sm.ow[warp][h][4 * l]) = acc[h];
   }
   score_epilogue<GM, D>(p, b, g, s, sm.wst, &sm.ow[0][0][0], GM * D, sm.tail);
 }

@@ -91,6 +91,17 @@ def test_per_kv_head_selection(vp, budget):
     Hn.check_all(vp, Hn.make_inputs(r), budget)
 
 
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("H,Hkv", [(8, 8), (12, 4), (28, 4), (32, 2)])
+@pytest.mark.parametrize("paged", [False, True])
+def test_fp32_batches(vp, D, H, Hkv, paged):
+    """fp32 caches: every head-group template, spans and texts that end inside
+    a batch of rows, one text token, an empty span."""
+    r = small(dtype=W.FP32, head_dim=D, heads=H, kv_heads=Hkv, batch=4, vis_len=(33, 577, 0, 7),
+              vis_start=(0, 13, 0, 1), text_len=(1, 270, 9, 65), paged=paged, page_size=4)
+    Hn.check_all(vp, Hn.make_inputs(r), r.budget)
+
+
 @pytest.mark.parametrize("score_path", [1, 2])
 @pytest.mark.parametrize("text", [(1, 129, 700), (64, 2000, 31)])
 def test_context_with_headroom(vp, score_path, text):
