@@ -163,6 +163,13 @@ __device__ __forceinline__ void ldsm_x4(unsigned addr, uint32_t& r0, uint32_t& r
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
                : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr));
 }
+// Transpose of an 8x8 b16 matrix held by the warp (lane l: row l / 4, columns
+// 2 (l % 4) and the next).
+__device__ __forceinline__ uint32_t movm_t(uint32_t a) {
+  uint32_t d;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;\n" : "=r"(d) : "r"(a));
+  return d;
+}
 __device__ __forceinline__ void ldsm_x4_t(unsigned addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
                : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr));
@@ -2853,100 +2860,76 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(const __grid_constant
 }
 
 // ---------------------------------------------------------------------------
-// k_gather_mma (bf16): grid (nc, Hkv, B), 4 warps.  CTA c (a) attends over
-// chunk c of the kept list (c < nk).  Warp w takes 32-token tiles w, w + 4,
-// ... of the chunk and streams the kept V rows through a private ring of
-// S slots: lane j copies row j of a tile with one bulk copy into a slot of
-// padded rows (a 16-byte shift per row: conflict-free ldmatrix), and the
-// token's logits with 4-byte cp.async (heads 0-3 into the row's pad bytes);
-// the slot's mbarrier completes once the row bytes and every lane's logits
-// have landed.  The kept-list entries are read three tiles ahead of their
-// copies (the first ones in the same round trip as the kept count).  S is 1
-// when no chunk holds more than one tile per warp (four CTAs share an SM);
-// otherwise 3 (two CTAs per SM) or 2 (three CTAs per SM, the same bytes in
-// flight per SM over more warps), whichever runs the grid in fewer waves, 3
-// on a tie (a lone CTA in a short last wave keeps more copies in flight).
-// The tile's logits give per-head probabilities; P.V runs on the tensor
-// cores as in the score kernel (A = V^T by ldmatrix.trans, B = P^T from a
-// per-warp bf16 buffer).  The warps' partials are merged in shared memory:
-// the only CTA of its (sequence, kv-head) combines them with the text part
-// and writes the output; otherwise they form the chunk's partial, and (b)
-// and the final combine are shared with k_gather.
+// k_gather_mma (bf16): grid (nc, Hkv, B), NW warps.  CTA c (a) attends over
+// chunk c of the kept list (c < nk), whose entries (and page ids) it stages in
+// shared memory first.  Warp w takes steps w, w + NW, ... of 16 kept rows.  P.V
+// runs on the tensor cores (m16n8k16, O^T = V^T P^T) on rows read straight
+// into registers: lane (gr, tg) reads 16-byte pieces tg, tg + 4, ... of rows
+// gr and gr + 8, so four lanes cover 64 contiguous bytes, and a transpose of
+// each 8x8 block in the warp (movmatrix) leaves token pairs of one dimension
+// per lane, which is the A operand; which dimension lands at which m is free
+// as long as the output agrees.  The B operand is the probability of head gr
+// for tokens 2 tg, 2 tg + 1, 2 tg + 8 and 2 tg + 9, whose logits the lane
+// reads itself.  Nothing but the list is staged or exchanged, every warp is
+// independent, and twenty warps (four-warp CTAs) share an SM.
+// The warps' partials are merged in shared memory: the only CTA of its
+// (sequence, kv-head) combines them with the text part and writes the output;
+// otherwise they form the chunk's partial, and (b) and the final combine are
+// shared with k_gather.
+// Bound by the rows in flight (4 KB per warp) and, in grids of few CTAs per
+// SM, by the start of each CTA: a copy-only kernel reads the same rows at 6.5
+// to 7.0 TB/s.  Rows went through shared-memory rings before, by bulk copies
+// or cp.async, 8 to 12 warps per SM.  64 sequences, 8 kv-heads, G = 4, kept
+// rows of 256 bytes: 1280 of 6400 per sequence 48.5 -> 41.8 us, 8192 of 16384
+// 231 -> 212 us, 29 of 576 8.0 -> 6.1 us.  Measured against it: operands from
+// prmt on pieces of four rows per lane 42 / 215 us; the same staged by
+// cp.async, two slots, 66 / 281 us; rows of the next step requested before a
+// step's products (128 registers, four CTAs) 41 / 229 us.
 // ---------------------------------------------------------------------------
-constexpr int kGmWarps = 4;
-constexpr int kGmSlots = 3;  // ring slots of the deeper form (the other has 2)
-
-template <int D, int NT, int S>
+template <int D, int NT, int NW>
 struct GmCfg {
   static constexpr int GM = 8 * NT;
-  static constexpr int THREADS = 32 * kGmWarps;
-  static constexpr int MT = D / 16;
-  // 32 V rows at a pitch of 2D + 16 bytes; the pad of row j holds token j's
-  // logits of heads 0-3, the other heads' logits sit in a separate array.
-  static constexpr int RP = 2 * D + 16;
-  static constexpr int SLOT = 32 * RP;
-  static constexpr int ZX = GM - 4;
-  // Kept rows per CTA: a single slot serves one tile per warp.
-  static constexpr int MAX_CHUNK = S == 1 ? 32 * kGmWarps : kGmMaxChunk;
-  // After part (a) the ring holds the warps' outputs, then the split weights;
-  // before it, the split weights of part (b).
-  static constexpr int OFF_TW = kGmWarps * GM * D * 4;
-  static constexpr int RING_BYTES = kGmWarps * S * SLOT;
-  static constexpr int REUSE_BYTES = OFF_TW + 2 * GM * kNsMax * 4;
-  static constexpr int RING = RING_BYTES > REUSE_BYTES ? RING_BYTES : REUSE_BYTES;
-  static constexpr int OFF_BAR = RING;                          // full[warps][slots]
-  static constexpr int OFF_P = OFF_BAR + kGmWarps * S * 8;      // bf16 [warps][GM][32] probabilities
-  static constexpr int OFF_ZX = OFF_P + kGmWarps * GM * 32 * 2; // float [warps][slots][ZX][32] logits
-  static constexpr int OFF_MASK = OFF_ZX + kGmWarps * S * ZX * 32 * 4;  // copied rows per slot
-  static constexpr int OFF_WST = OFF_MASK + kGmWarps * S * 4;           // float [warps][GM][2]
-  static constexpr int OFF_FIN = OFF_WST + kGmWarps * GM * 2 * 4;       // float [GM][4]
+  static constexpr int THREADS = 32 * NW;
+  static constexpr int MT = D / 16;   // m-tiles (16 dimensions each)
+  // The warps' outputs; before part (a) and in the finish, the split weights.
+  static constexpr int OUT_BYTES = NW * GM * D * 4, TW_BYTES = 2 * GM * kNsMax * 4;
+  static constexpr int OFF_WST = OUT_BYTES > TW_BYTES ? OUT_BYTES : TW_BYTES;  // float [warps][GM][2]
+  static constexpr int OFF_FIN = OFF_WST + NW * GM * 2 * 4;              // float [GM][4]
   static constexpr int OFF_LAST = OFF_FIN + GM * 4 * 4;
-  static constexpr size_t SMEM = (size_t)OFF_LAST + 16;
-  static_assert(RP % 16 == 0 && (RP / 16) % 8 == 1, "row pitch: 16-byte aligned rows, one bank group apart");
-  static_assert(OFF_BAR % 8 == 0 && OFF_P % 16 == 0 && OFF_ZX % 16 == 0 && OFF_WST % 16 == 0, "alignment");
+  static constexpr int OFF_ENT = OFF_LAST + 16;  // int [kGmMaxChunk] entries, paged: then page ids
+  static constexpr size_t smem(bool paged) { return (size_t)OFF_ENT + kGmMaxChunk * (paged ? 8 : 4); }
 };
 
-template <int D, int NT, int S>
-__global__ void __launch_bounds__(32 * kGmWarps) k_gather_mma(const __grid_constant__ StepParams p) {
-  using C = GmCfg<D, NT, S>;
+template <int D, int NT, int NW, bool PAGED>
+__global__ void __launch_bounds__(32 * NW, (NT == 1 ? 20 : 12) / NW) k_gather_mma(const __grid_constant__ StepParams p) {
+  using C = GmCfg<D, NT, NW>;
   constexpr int GM = C::GM;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* smem = smem_raw;
   const int c = blockIdx.x, g = blockIdx.y, b = blockIdx.z;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int gr = lane >> 2, tg = lane & 3;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::OFF_BAR) + warp * S;
-  __nv_bfloat16* P = reinterpret_cast<__nv_bfloat16*>(smem + C::OFF_P) + warp * GM * 32;
-  float* zx = reinterpret_cast<float*>(smem + C::OFF_ZX) + warp * S * C::ZX * 32;
-  uint32_t* mask_s = reinterpret_cast<uint32_t*>(smem + C::OFF_MASK) + warp * S;
   float (*wst)[GM][2] = reinterpret_cast<float (*)[GM][2]>(smem + C::OFF_WST);
   float (*fin)[4] = reinterpret_cast<float (*)[4]>(smem + C::OFF_FIN);
   int* last = reinterpret_cast<int*>(smem + C::OFF_LAST);
-  unsigned char* ring = smem + warp * S * C::SLOT;
+  int* ent = reinterpret_cast<int*>(smem + C::OFF_ENT);
 
-  // A slot's phase completes on lane 0's arrival (with the row bytes as its
-  // transaction count) once the rows and every lane's logits have landed.
-  if (tid < kGmWarps * S) mbar_init(reinterpret_cast<uint64_t*>(smem + C::OFF_BAR) + tid, 1);
-  mbar_fence_init();
-  __syncthreads();
   const int G = p.G, H = p.H;
   const int64_t hrow0 = (int64_t)b * H + g * G;
-  float (*tw)[kNsMax] = reinterpret_cast<float (*)[kNsMax]>(smem + C::OFF_TW);
+  float (*tw)[kNsMax] = reinterpret_cast<float (*)[kNsMax]>(smem);
   float (*tl)[kNsMax] = tw + GM;
   // The sequence's record is a caller input: read it before the wait.
   const Seq sq = load_seq(p, b, false);
   // (b) first: it reads only the score kernel's partials, complete before the
-  // select kernel lets this grid start.  Its shared memory is the ring's.
+  // select kernel lets this grid start.
   if (c < p.nm) {
     gather_text_slice<D, GM, C::THREADS>(p, c, hrow0, tw, tl);
-    fence_proxy_async();
     __syncthreads();
   }
   pdl_wait();
   pdl_trigger();
   const int64_t pbase = ((int64_t)b * p.Hkv + g) * p.nk_max;
   unsigned err = 0;
-  bool timed_out = false;
   // The only CTA of its (sequence, kv-head) combines the text part with its
   // chunk itself: no partial round trip through global memory, no ticket.
   const bool lone = p.nc == 1 && p.nk == 1;
@@ -2955,180 +2938,138 @@ __global__ void __launch_bounds__(32 * kGmWarps) k_gather_mma(const __grid_const
   if (c < p.nk) {
     const int sel = p.granularity ? b * p.Hkv + g : b;
     const int32_t* kept = p.kept_idx + (int64_t)sel * p.kept_cap;
-    // Kept-list entry of row `lane` of this warp's tile k for a chunk
-    // starting at j, read now (entries past the chunk are read in bounds
-    // and masked at use; with no kept capacity the list may be absent and
-    // nothing is read).  The copies of tile k are issued S tiles before it
-    // is consumed and its entry QD tiles before that: an iteration can take
-    // less than a round trip to L2.
-    constexpr int QD = 3;
-    auto raw_entry = [&](int j, int k) {
-      return p.kept_cap > 0 ? ldcg_now(kept + min(j + 32 * (warp + kGmWarps * k) + lane, p.kept_cap - 1)) : -1;
-    };
-    // The first S + QD tiles' entries are read in the same round trip as the
-    // count, at the chunk start a full list would give (exact for chunk 0
-    // and whenever the count is the cap); a different start reloads them.
+    // The chunk's list entries, staged in shared memory: the first ones are
+    // read in the same round trip as the count, at the chunk start a full list
+    // would give (exact for chunk 0 and whenever the count is the cap); a
+    // different start reads them again.  An out-of-range index is flagged and
+    // staged as -1.
+    constexpr int EPT = 4;  // entries of a thread in flight
     const int j0s = min(p.kept_cap, c * ((p.kept_cap + p.nk - 1) / p.nk));
-    int raw[S + QD];
+    int first[EPT];
 #pragma unroll
-    for (int k = 0; k < S + QD; ++k) raw[k] = raw_entry(j0s, k);
+    for (int u = 0; u < EPT; ++u) {
+      const int j = j0s + tid + u * C::THREADS;
+      first[u] = j < p.kept_cap ? ldcg_now(kept + j) : -1;
+    }
     const int K = max(0, min(__ldcg(p.kept_count + sel), min(sq.nv, p.kept_cap)));
     const int per = (K + p.nk - 1) / p.nk;
-    const int j0 = min(K, c * per), j1 = min(K, min(j0 + per, j0 + C::MAX_CHUNK));
-    if (per > C::MAX_CHUNK) err |= ERR_KEPT;  // the plan keeps every chunk within the limit
-    const int ntile = (j1 - j0 + 31) / 32;
-    const int nj = warp < ntile ? (ntile - warp + kGmWarps - 1) / kGmWarps : 0;  // this warp's tiles
-    const float* zb = p.z_ws + (int64_t)b * p.max_visual * p.hp + g * G;
-    int issued = 0;  // tiles of this warp whose copies were issued
-
-    // Kept index of row `lane` of this warp's tile k from its entry, or -1
-    // (past the chunk; an out-of-range index is flagged and skipped).
-    auto row_index = [&](int k, int e) {
-      const int j = 32 * (warp + kGmWarps * k) + lane;
-      int i = -1;
-      if (k < nj && j0 + j < j1) {
-        i = e;
-        if (i < 0 || i >= sq.nv) { err |= ERR_KEPT; i = -1; }
-      }
-      return i;
-    };
-    if (j0 != j0s) {  // CTA-uniform
+    const int j0 = min(K, c * per), j1 = min(K, min(j0 + per, j0 + kGmMaxChunk));
+    if (per > kGmMaxChunk) err |= ERR_KEPT;  // the plan keeps every chunk within the limit
+    const int n = j1 - j0, nstep = (n + 15) / 16;
+    const int nj = warp < nstep ? (nstep - warp + NW - 1) / NW : 0;  // this warp's steps
+    for (int i0 = 0; i0 < 16 * nstep; i0 += EPT * C::THREADS) {
+      int e[EPT], pg[EPT];
 #pragma unroll
-      for (int k = 0; k < S + QD; ++k) raw[k] = raw_entry(j0, k);
+      for (int u = 0; u < EPT; ++u) {
+        const int i = i0 + tid + u * C::THREADS;
+        e[u] = i < n ? (i0 == 0 && j0 == j0s ? first[u] : __ldcg(kept + j0 + i)) : -1;
+      }
+#pragma unroll
+      for (int u = 0; u < EPT; ++u) {
+        const int i = i0 + tid + u * C::THREADS;
+        if (i < n && (e[u] < 0 || e[u] >= sq.nv)) { err |= ERR_KEPT; e[u] = -1; }
+        if constexpr (PAGED) {
+          const int lp = (sq.vs + e[u]) >> p.page_shift;
+          pg[u] = e[u] >= 0 && lp < p.v.max_pages ? __ldg(p.v.block_table + (int64_t)b * p.v.max_pages + lp) : 0;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < EPT; ++u) {
+        const int i = i0 + tid + u * C::THREADS;
+        if constexpr (PAGED)
+          if (pg[u] < 0 || pg[u] >= p.v.num_pages) { err |= ERR_PAGE; e[u] = -1; pg[u] = 0; }
+        if (i < 16 * nstep) {
+          ent[i] = e[u];
+          if constexpr (PAGED) ent[kGmMaxChunk + i] = pg[u];
+        }
+      }
     }
-    auto issue = [&](int k, int i) {  // all lanes; i = this lane's kept index
-      if (k >= nj) return;
-      const int slot = k % S;
-      const __nv_bfloat16* vr = nullptr;
-      if (i >= 0) {
-        vr = kv_row<__nv_bfloat16>(p.v, p, b, g, sq.vs + i);
-        if (!vr) { err |= ERR_PAGE; i = -1; }
-      }
-      const unsigned m = __ballot_sync(0xffffffffu, vr != nullptr);
-      unsigned char* row = ring + slot * C::SLOT + lane * C::RP;
-      // The slot was last read by this warp's ldmatrix and loads (generic
-      // proxy); its rows are next written by bulk copies (async proxy).
-      fence_proxy_async();
-      __syncwarp();  // every lane is done reading this slot
-      if (lane == 0) mask_s[slot] = m;
-      // Logits of this lane's token: heads 0-3 into its row's pad.
-      if (vr) {
-        const float* zr = zb + (int64_t)i * p.hp;
-        for (int h = 0; h < G; ++h)
-          cp_async4(h < 4 ? smem_u32(row + 2 * D + 4 * h) : smem_u32(zx + (slot * C::ZX + h - 4) * 32 + lane), zr + h);
-      }
-      cp_async_arrive_counted(full + slot);
-      __syncwarp();  // every lane's arrival is counted before lane 0's
-      if (lane == 0) mbar_expect_tx(full + slot, (unsigned)__popc(m) * (2 * D));
-      __syncwarp();
-      if (vr) bulk_g2s(row, vr, 2 * D, full + slot);
-      issued = k + 1;
-    };
-    // Prologue: the first S tiles; the next QD tiles' entries stay queued.
-#pragma unroll
-    for (int k = 0; k < S; ++k) issue(k, row_index(k, raw[k]));
-    int q[QD];
-#pragma unroll
-    for (int t = 0; t < QD; ++t) q[t] = raw[S + t];
-
+    __syncthreads();
+    const int gh = min(gr, G - 1);  // lanes of heads past G read a head's logits in bounds; their products are not used
+    const float* zb = p.z_ws + (int64_t)b * p.max_visual * p.hp + g * G;
+    const __nv_bfloat16* vb = reinterpret_cast<const __nv_bfloat16*>(p.v.data) + (int64_t)g * p.v.sh + 8 * tg;
+    const __nv_bfloat16* vseq = vb + (PAGED ? 0 : (int64_t)b * p.v.sb + (int64_t)sq.vs * p.v.st);
+    constexpr int NX = D / 32;  // 16-byte pieces of a row per lane
     // Probabilities are taken relative to each head's largest logit over all
     // tokens (from the select kernel), so no running maximum is needed.
-    float mh[GM], lsum[GM];
+    float mh[NT], lsum[NT];
     float acc[NT][C::MT][4];
 #pragma unroll
-    for (int h = 0; h < GM; ++h) {
-      mh[h] = h < G ? __ldcg(p.hmax + hrow0 + h) : -CUDART_INF_F;
-      lsum[h] = 0.f;
-    }
-#pragma unroll
-    for (int nn = 0; nn < NT; ++nn)
+    for (int nn = 0; nn < NT; ++nn) {
+      mh[nn] = 8 * nn + gr < G ? __ldcg(p.hmax + hrow0 + 8 * nn + gr) : 0.f;
+      lsum[nn] = 0.f;
 #pragma unroll
       for (int mi = 0; mi < C::MT; ++mi)
 #pragma unroll
         for (int e = 0; e < 4; ++e) acc[nn][mi][e] = 0.f;
-    // ldmatrix.trans lane roles for V^T (A operand, rows = dimensions).
-    const int vrow = (lane & 7) + 8 * (lane >> 4), vcol = 8 * ((lane >> 3) & 1);
-
-    for (int k = 0; k < nj; ++k) {
-      const int slot = k % S;
-      if (!mbar_wait(full + slot, (k / S) & 1)) { timed_out = true; break; }
-      const uint32_t mask = mask_s[slot];
-      const bool live = (mask >> lane) & 1u;
-      const float4 z4 = *reinterpret_cast<const float4*>(ring + slot * C::SLOT + lane * C::RP + 2 * D);
-      float z[GM];
-#pragma unroll
-      for (int h = 0; h < GM; ++h) {
-        z[h] = -CUDART_INF_F;
-        if (live && h < G) {
-          if (h < 4) z[h] = h == 0 ? z4.x : h == 1 ? z4.y : h == 2 ? z4.z : z4.w;
-          else z[h] = zx[(slot * C::ZX + (h >= 4 ? h - 4 : 0)) * 32 + lane];
-        }
-      }
-
-      // Probabilities of this tile (the warp's buffer was last read by the
-      // previous tile's P.V, before the loop's closing __syncwarp).
-#pragma unroll
-      for (int h = 0; h < GM; ++h) {
-        if (h >= G) continue;
-        const float pe = exp2_rel(z[h], mh[h]);
-        lsum[h] += pe;
-        P[h * 32 + lane] = __float2bfloat16_rn(pe);
-      }
-      __syncwarp();
-      const unsigned vt = smem_u32(ring + slot * C::SLOT);
-#pragma unroll
-      for (int sb = 0; sb < 2; ++sb) {
-        uint32_t pb[NT][2];
-#pragma unroll
-        for (int nn = 0; nn < NT; ++nn) {
-          const __nv_bfloat16* pr = P + (8 * nn + gr) * 32 + 16 * sb + 2 * tg;
-          pb[nn][0] = *reinterpret_cast<const uint32_t*>(pr);
-          pb[nn][1] = *reinterpret_cast<const uint32_t*>(pr + 8);
-        }
-        // Rows that were not copied hold stale bytes: zero their words.  (B
-        // columns of heads past G hold stale bytes too; those heads' sums
-        // are never read.)
-        const uint32_t rb = mask >> (16 * sb);
-        if ((rb & 0xffffu) == 0xffffu) {  // all 16 rows copied (warp-uniform)
-#pragma unroll
-          for (int mi = 0; mi < C::MT; ++mi) {
-            uint32_t a0, a1, a2, a3;
-            ldsm_x4_t(vt + (16 * sb + vrow) * C::RP + (16 * mi + vcol) * 2, a0, a1, a2, a3);
-#pragma unroll
-            for (int nn = 0; nn < NT; ++nn) mma_bf16(acc[nn][mi], a0, a1, a2, a3, pb[nn][0], pb[nn][1]);
-          }
-          continue;
-        }
-        const uint32_t mlo = (((rb >> (2 * tg)) & 1u) ? 0x0000ffffu : 0u) | (((rb >> (2 * tg + 1)) & 1u) ? 0xffff0000u : 0u);
-        const uint32_t mhi = (((rb >> (2 * tg + 8)) & 1u) ? 0x0000ffffu : 0u) | (((rb >> (2 * tg + 9)) & 1u) ? 0xffff0000u : 0u);
-#pragma unroll
-        for (int mi = 0; mi < C::MT; ++mi) {
-          uint32_t a0, a1, a2, a3;
-          ldsm_x4_t(vt + (16 * sb + vrow) * C::RP + (16 * mi + vcol) * 2, a0, a1, a2, a3);
-          a0 &= mlo; a1 &= mlo; a2 &= mhi; a3 &= mhi;
-#pragma unroll
-          for (int nn = 0; nn < NT; ++nn) mma_bf16(acc[nn][mi], a0, a1, a2, a3, pb[nn][0], pb[nn][1]);
-        }
-      }
-      __syncwarp();
-      // Refill this slot with tile k + S; queue the entry of tile k + S + QD.
-      const int icur = row_index(k + S, q[0]);
-#pragma unroll
-      for (int t = 0; t + 1 < QD; ++t) q[t] = q[t + 1];
-      q[QD - 1] = raw_entry(j0, k + S + QD);
-      issue(k + S, icur);
     }
-    // After a timeout, let this warp's copies still in flight land (bounded)
-    // before the ring is reused below.
-    if (timed_out && lane == 0)
-      for (int k = max(0, issued - S); k < issued; ++k) mbar_wait(full + k % S, (k / S) & 1);
-    __syncwarp();
-
-    // Warp partials -> chunk partial (log-sum-exp over the warps).
+    auto word = [](const uint4& v, int w) { return w == 0 ? v.x : w == 1 ? v.y : w == 2 ? v.z : v.w; };
+    for (int k = 0; k < nj; ++k) {
+      const int* es = ent + 16 * (warp + NW * k);
+      const int er[2] = {es[gr], es[gr + 8]};  // the rows of V this lane reads
+      const int2 ea = *reinterpret_cast<const int2*>(es + 2 * tg), eb = *reinterpret_cast<const int2*>(es + 2 * tg + 8);
+      const int et[4] = {ea.x, ea.y, eb.x, eb.y};  // its tokens of the B operand
+      uint4 v[2][NX];
+      float z[NT][4];
 #pragma unroll
-    for (int h = 0; h < GM; ++h) {
-      const float l = warp_sum(lsum[h]);
-      if (lane == 0) { wst[warp][h][0] = mh[h]; wst[warp][h][1] = l; }
+      for (int hf = 0; hf < 2; ++hf) {
+        const int i = max(er[hf], 0);
+        const __nv_bfloat16* vr;
+        if constexpr (PAGED)
+          vr = vb + (int64_t)es[kGmMaxChunk + gr + 8 * hf] * p.v.sb + (int64_t)((sq.vs + i) & (p.page_size - 1)) * p.v.st;
+        else
+          vr = vseq + (int64_t)i * p.v.st;
+#pragma unroll
+        for (int x = 0; x < NX; ++x) v[hf][x] = __ldcg(reinterpret_cast<const uint4*>(vr + 32 * x));
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int nn = 0; nn < NT; ++nn) z[nn][u] = __ldcg(zb + (int64_t)max(et[u], 0) * p.hp + min(8 * nn + gh, G - 1));
+      // Rows that do not count: probability 0, finite words.
+      if (__any_sync(0xffffffffu, (er[0] | er[1]) < 0)) {
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf)
+          if (er[hf] < 0) {
+#pragma unroll
+            for (int x = 0; x < NX; ++x) v[hf][x] = make_uint4(0u, 0u, 0u, 0u);
+          }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (et[u] < 0) {
+#pragma unroll
+            for (int nn = 0; nn < NT; ++nn) z[nn][u] = -CUDART_INF_F;
+          }
+      }
+      uint32_t pb[NT][2];
+#pragma unroll
+      for (int nn = 0; nn < NT; ++nn) {
+        float pe[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          pe[u] = exp2_rel(z[nn][u], mh[nn]);
+          lsum[nn] += pe[u];
+        }
+        pb[nn][0] = pack_bf16(pe[0], pe[1]);
+        pb[nn][1] = pack_bf16(pe[2], pe[3]);
+      }
+#pragma unroll
+      for (int e = 0; e < C::MT; ++e) {
+        const int x = e >> 1, j = e & 1;
+        const uint32_t a0 = movm_t(word(v[0][x], j)), a1 = movm_t(word(v[0][x], j + 2));
+        const uint32_t a2 = movm_t(word(v[1][x], j)), a3 = movm_t(word(v[1][x], j + 2));
+#pragma unroll
+        for (int nn = 0; nn < NT; ++nn) mma_bf16(acc[nn][e], a0, a1, a2, a3, pb[nn][0], pb[nn][1]);
+      }
+    }
+
+    // Warp partials -> chunk partial (one reference maximum: sums add up).
+#pragma unroll
+    for (int nn = 0; nn < NT; ++nn) {
+      float l = lsum[nn];
+      l += __shfl_xor_sync(0xffffffffu, l, 1);
+      l += __shfl_xor_sync(0xffffffffu, l, 2);
+      if (tg == 0) { wst[warp][8 * nn + gr][0] = mh[nn]; wst[warp][8 * nn + gr][1] = l; }
     }
     // Lone CTA: request the text output and statistics (the merged slice this
     // CTA wrote in part (b), or the single split partial) before the sums.
@@ -3149,17 +3090,16 @@ __global__ void __launch_bounds__(32 * kGmWarps) k_gather_mma(const __grid_const
         }
       }
     }
-    __syncthreads();  // every warp is done with its ring
     float* ow = reinterpret_cast<float*>(smem) + warp * GM * D;
 #pragma unroll
     for (int nn = 0; nn < NT; ++nn)
 #pragma unroll
-      for (int mi = 0; mi < C::MT; ++mi) {
-        const int h0 = 8 * nn + 2 * tg, d0 = 16 * mi + gr;
-        ow[h0 * D + d0] = acc[nn][mi][0];
-        ow[(h0 + 1) * D + d0] = acc[nn][mi][1];
-        ow[h0 * D + d0 + 8] = acc[nn][mi][2];
-        ow[(h0 + 1) * D + d0 + 8] = acc[nn][mi][3];
+      for (int e = 0; e < C::MT; ++e) {
+        float* o = ow + (8 * nn + 2 * tg) * D + 32 * (e >> 1) + 8 * (gr >> 1) + 2 * (e & 1) + (gr & 1);
+        o[0] = acc[nn][e][0];
+        o[D] = acc[nn][e][1];
+        o[4] = acc[nn][e][2];
+        o[D + 4] = acc[nn][e][3];
       }
     __syncthreads();
     if (lone) {
@@ -3172,7 +3112,7 @@ __global__ void __launch_bounds__(32 * kGmWarps) k_gather_mma(const __grid_const
         float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
         float l = 0.f;
 #pragma unroll
-        for (int w = 0; w < kGmWarps; ++w) {
+        for (int w = 0; w < NW; ++w) {
           const float4 v = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(smem) + (w * GM + h) * D + d);
           o.x += v.x; o.y += v.y; o.z += v.z; o.w += v.w;
           l += wst[w][h][1];
@@ -3193,7 +3133,7 @@ __global__ void __launch_bounds__(32 * kGmWarps) k_gather_mma(const __grid_const
       const int h = i / D, d = i % D;
       float o = 0.f, l = 0.f;
 #pragma unroll
-      for (int w = 0; w < kGmWarps; ++w) {
+      for (int w = 0; w < NW; ++w) {
         o += reinterpret_cast<const float*>(smem)[(w * GM + h) * D + d];
         l += wst[w][h][1];
       }
@@ -3203,10 +3143,9 @@ __global__ void __launch_bounds__(32 * kGmWarps) k_gather_mma(const __grid_const
         p.gpart_st[((pbase + c) * G + h) * 2 + 1] = l;
       }
     }
-    __syncthreads();  // the ring is reused below
+    __syncthreads();  // the outputs' memory is reused below
   }
 
-  if (timed_out) err |= ERR_TIMEOUT;
   if (err) atomicOr(p.err, err);
   if (!lone) gather_finish<__nv_bfloat16, D, GM, C::THREADS>(p, b, g, hrow0, pbase, tw, fin, last);
 }
@@ -4139,25 +4078,11 @@ cudaError_t launch_score_d(const StepParams& p, cudaStream_t st) {
 template <int GM>
 size_t slice_smem() { return sizeof(SliceSmem<GM>); }
 
-// CTAs of a chunk-gather instance resident on one SM (queried once).
-template <int D, int NT, int S>
-int gm_blocks_per_sm() {
-  static const int n = [] {
-    int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_gather_mma<D, NT, S>, 32 * kGmWarps,
-                                                      GmCfg<D, NT, S>::SMEM) != cudaSuccess)
-      b = 0;
-    return b;
-  }();
-  return n;
-}
-// True when the two-slot form runs n CTAs in fewer waves than the three-slot one.
-template <int D, int NT>
-bool gm_fewer_waves(long long n, int num_sms) {
-  const long long r2 = (long long)gm_blocks_per_sm<D, NT, 2>() * num_sms;
-  const long long r3 = (long long)gm_blocks_per_sm<D, NT, kGmSlots>() * num_sms;
-  if (r2 <= 0 || r3 <= 0) return false;
-  return (n + r2 - 1) / r2 < (n + r3 - 1) / r3;
+constexpr int kGmWide = 512;
+template <int D, int NT, int NW>
+cudaError_t launch_gather_mma(const StepParams& p, dim3 grid, cudaStream_t st) {
+  return launch_ex(p.paged ? k_gather_mma<D, NT, NW, true> : k_gather_mma<D, NT, NW, false>, grid, dim3(32 * NW),
+                   GmCfg<D, NT, NW>::smem(p.paged), st, 1, p);
 }
 
 template <typename T, int D>
@@ -4170,20 +4095,16 @@ cudaError_t launch_gather_td(const StepParams& p, cudaStream_t st) {
   }
   const dim3 grid(p.nc, p.Hkv, p.B);
   if (sizeof(T) == 2) {
-    // A single ring slot when no chunk can hold more than one tile per warp.
-    const int kmax = min(p.kept_cap, p.max_visual);
-    const bool one = (kmax + p.nk - 1) / p.nk <= GmCfg<D, 1, 1>::MAX_CHUNK;
-    const long long n = (long long)p.nc * p.Hkv * p.B;
-    if (p.G <= 8) {
-      if (one) return launch_ex(k_gather_mma<D, 1, 1>, grid, dim3(32 * kGmWarps), GmCfg<D, 1, 1>::SMEM, st, 1, p);
-      if (gm_fewer_waves<D, 1>(n, p.num_sms))
-        return launch_ex(k_gather_mma<D, 1, 2>, grid, dim3(32 * kGmWarps), GmCfg<D, 1, 2>::SMEM, st, 1, p);
-      return launch_ex(k_gather_mma<D, 1, kGmSlots>, grid, dim3(32 * kGmWarps), GmCfg<D, 1, kGmSlots>::SMEM, st, 1, p);
-    }
-    if (one) return launch_ex(k_gather_mma<D, 2, 1>, grid, dim3(32 * kGmWarps), GmCfg<D, 2, 1>::SMEM, st, 1, p);
-    if (gm_fewer_waves<D, 2>(n, p.num_sms))
-      return launch_ex(k_gather_mma<D, 2, 2>, grid, dim3(32 * kGmWarps), GmCfg<D, 2, 2>::SMEM, st, 1, p);
-    return launch_ex(k_gather_mma<D, 2, kGmSlots>, grid, dim3(32 * kGmWarps), GmCfg<D, 2, kGmSlots>::SMEM, st, 1, p);
+    // Eight warps where one CTA per (sequence, kv-head) has a long list to
+    // itself: such a grid is about one wave, and at two CTAs per SM its last
+    // third leaves room, CTA by CTA, for the next call's score kernel (1280 of
+    // 6400, 64 sequences, 8 kv-heads: the call 229 us, with four warps 241,
+    // though the gather alone takes 43 against 42 us).  Chunked lists run
+    // several waves (8192 of 16384: 212 us with four warps, 230 with eight),
+    // short ones one or two steps per warp (29 of 576: 6.1 against 9.2 us).
+    if (p.nk == 1 && p.kept_cap >= kGmWide)
+      return p.G <= 8 ? launch_gather_mma<D, 1, 8>(p, grid, st) : launch_gather_mma<D, 2, 8>(p, grid, st);
+    return p.G <= 8 ? launch_gather_mma<D, 1, 4>(p, grid, st) : launch_gather_mma<D, 2, 4>(p, grid, st);
   }
   if (p.G <= 4) return launch_ex(k_gather<T, D, 4>, grid, dim3(kGatherThreads), gather_smem<T, D, 4>(), st, 1, p);
   if (p.G <= 8) return launch_ex(k_gather<T, D, 8>, grid, dim3(kGatherThreads), gather_smem<T, D, 8>(), st, 1, p);
@@ -4200,18 +4121,16 @@ cudaError_t configure_fixed_kernels() {
 #define VP_SET(kernel, bytes) if (e == cudaSuccess) e = set_smem(kernel, bytes)
   VP_SET((k_score_tc<8>), (TcCfg::SMEM));
   VP_SET((k_score_tc<16>), (TcCfg::SMEM));
-  VP_SET((k_gather_mma<128, 1, kGmSlots>), (GmCfg<128, 1, kGmSlots>::SMEM));
-  VP_SET((k_gather_mma<128, 2, kGmSlots>), (GmCfg<128, 2, kGmSlots>::SMEM));
-  VP_SET((k_gather_mma<64, 1, kGmSlots>), (GmCfg<64, 1, kGmSlots>::SMEM));
-  VP_SET((k_gather_mma<64, 2, kGmSlots>), (GmCfg<64, 2, kGmSlots>::SMEM));
-  VP_SET((k_gather_mma<128, 1, 2>), (GmCfg<128, 1, 2>::SMEM));
-  VP_SET((k_gather_mma<128, 2, 2>), (GmCfg<128, 2, 2>::SMEM));
-  VP_SET((k_gather_mma<64, 1, 2>), (GmCfg<64, 1, 2>::SMEM));
-  VP_SET((k_gather_mma<64, 2, 2>), (GmCfg<64, 2, 2>::SMEM));
-  VP_SET((k_gather_mma<128, 1, 1>), (GmCfg<128, 1, 1>::SMEM));
-  VP_SET((k_gather_mma<128, 2, 1>), (GmCfg<128, 2, 1>::SMEM));
-  VP_SET((k_gather_mma<64, 1, 1>), (GmCfg<64, 1, 1>::SMEM));
-  VP_SET((k_gather_mma<64, 2, 1>), (GmCfg<64, 2, 1>::SMEM));
+#define VP_SET_GM(D, NT)                                                          \
+  VP_SET((k_gather_mma<D, NT, 4, false>), (GmCfg<D, NT, 4>::smem(false)));          \
+  VP_SET((k_gather_mma<D, NT, 4, true>), (GmCfg<D, NT, 4>::smem(true)));            \
+  VP_SET((k_gather_mma<D, NT, 8, false>), (GmCfg<D, NT, 8>::smem(false)));          \
+  VP_SET((k_gather_mma<D, NT, 8, true>), (GmCfg<D, NT, 8>::smem(true)))
+  VP_SET_GM(128, 1);
+  VP_SET_GM(128, 2);
+  VP_SET_GM(64, 1);
+  VP_SET_GM(64, 2);
+#undef VP_SET_GM
   VP_SET((k_score_tma<128, 1, kTmaWarps, tma_slots<128>(), false>), (tma_smem<128, 1>()));
   VP_SET((k_score_tma<128, 2, kTmaWarps, tma_slots<128>(), false>), (tma_smem<128, 2>()));
   VP_SET((k_score_tma<64, 1, kTmaWarps, tma_slots<64>(), false>), (tma_smem<64, 1>()));
@@ -4255,12 +4174,6 @@ cudaError_t configure_fixed_kernels() {
   VP_SET((k_gather_slice<float, 64, 8>), (slice_smem<8>()));
   VP_SET((k_gather_slice<float, 64, 16>), (slice_smem<16>()));
 #undef VP_SET
-  if (e == cudaSuccess) {  // the chunk gather's occupancies, now that its shared memory is set
-    gm_blocks_per_sm<128, 1, 2>(); gm_blocks_per_sm<128, 1, kGmSlots>();
-    gm_blocks_per_sm<128, 2, 2>(); gm_blocks_per_sm<128, 2, kGmSlots>();
-    gm_blocks_per_sm<64, 1, 2>(); gm_blocks_per_sm<64, 1, kGmSlots>();
-    gm_blocks_per_sm<64, 2, 2>(); gm_blocks_per_sm<64, 2, kGmSlots>();
-  }
   return e;
 }
 

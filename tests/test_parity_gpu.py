@@ -123,6 +123,40 @@ def test_context_with_headroom(vp, score_path, text):
     np.testing.assert_allclose(again, gpu["out"], rtol=0, atol=2e-2)
 
 
+@pytest.mark.parametrize("H,Hkv,D", [(12, 4, 128), (28, 4, 64), (32, 2, 128)])
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("k", [1, 15, 16, 17, 257, 2049])
+def test_kept_row_steps(vp, H, Hkv, D, paged, k):
+    """The separate gather kernels (diagnostics keep the call off the fused one):
+    short lists in the slice gather, chunks that end inside a 16-row step, more
+    rows than one chunk holds; odd head groups, both layouts."""
+    r = small(heads=H, kv_heads=Hkv, head_dim=D, batch=2, vis_len=(2100, 40), vis_start=(3, 0), text_len=(50, 9),
+              paged=paged, page_size=8)
+    inp = Hn.make_inputs(r)
+    budget = dict(mode=O.FIXED_K, tau=0.1, fixed_k=k)
+    dev = Hn.Device(vp, inp, budget)
+    n_act = torch.zeros((2,), dtype=torch.int32, device="cuda")
+    try:
+        vp.vp_set_diagnostics(dev.ctx, 1e-3, n_act, None)
+        gpu = dev.run()
+    finally:
+        dev.close()
+    for b in range(2):
+        Hn.compare_seq(inp, gpu, b, budget)
+
+
+@pytest.mark.parametrize("paged", [False, True])
+def test_chunk_gather_long_lists(vp, paged):
+    """One CTA per (sequence, kv-head) with a list of more than 512 rows (the
+    eight-warp form), ragged spans."""
+    vis = tuple(640 + 3 * i for i in range(40))
+    r = small(heads=16, kv_heads=8, head_dim=64, batch=40, vis_len=vis, vis_start=(1,) * 40, text_len=(20,) * 40,
+              paged=paged, page_size=16)
+    inp = Hn.make_inputs(r)
+    budget = dict(mode=O.FIXED_RATIO, tau=0.1, ratio_ppm=850_000)
+    Hn.check_all(vp, inp, budget, seqs=(0, 7, 39))
+
+
 def test_paged_cache(vp):
     r = small(batch=4, vis_len=(300, 577, 64, 1000), vis_start=(0, 13, 40, 0),
               text_len=(517, 70, 129, 33), paged=True, page_size=16)
