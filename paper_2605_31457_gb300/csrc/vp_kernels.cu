@@ -175,6 +175,15 @@ __device__ __forceinline__ void ldsm_x4_t(unsigned addr, uint32_t& r0, uint32_t&
                : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr));
 }
 
+// Asynchronous 4-byte store to the shared memory of CTA `rank` of the cluster
+// (only in a launch with a cluster), counted by that CTA's mbarrier; addr and bar are this CTA's own addresses of
+// the same variables.
+__device__ __forceinline__ void st_async_u32(unsigned addr, uint32_t v, unsigned bar, int rank) {
+  asm volatile(
+      "{\n .reg .b32 a, m;\n mapa.shared::cluster.u32 a, %0, %3;\n mapa.shared::cluster.u32 m, %2, %3;\n"
+      " st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.u32 [a], %1, [m];\n}\n"
+      ::"r"(addr), "r"(v), "r"(bar), "r"(rank) : "memory");
+}
 // ---- mbarrier + bulk (TMA) copies
 __device__ __forceinline__ void mbar_init(uint64_t* bar, unsigned count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(count) : "memory");
@@ -3427,97 +3436,95 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather_slice(const __grid_co
 //      and the masses (Eq. 5, Eq. 6); rank 0 also takes the head mean, the
 //      head max (Sec. 4.3) and the budget K_t (Eq. 7 + clamp).
 //   2. Every CTA requests the text partials of the score splits for its
-//      dimensions, scores its slice of the visual tokens (S_i of Eq. 2) into
-//      rank 0's shared memory meanwhile, then sums the text part.
-//   3. Rank 0 cuts the Top-K_t set (Eq. 3) by a radix select over the keys
-//      held in registers and compacts it, ascending, into the output and its
-//      shared memory; the other CTAs copy it over distributed shared memory.
-//   4. Every CTA stages the V slices and logits of the kept tokens in shared
-//      memory in one round trip, attends over them for its dimensions (P.V on
-//      the tensor cores for bf16 caches) and combines the result with the
-//      text part in log-sum-exp form.  Nothing but the results leaves the
+//      dimensions and scores its slice of the visual tokens (S_i of Eq. 2)
+//      into every CTA's shared memory.
+//   3. Every CTA cuts the Top-K_t set (Eq. 3) itself, by a radix select over
+//      the keys held in registers, and compacts it, ascending, into its shared
+//      memory (rank 0 also into the output): a second pass through the cluster
+//      would cost a barrier and two dependent remote reads.
+//   4. Every CTA requests the V slices and logits of the kept tokens in one
+//      round trip, sums its text part meanwhile, attends over the kept rows
+//      for its dimensions (P.V on the tensor cores for bf16 caches) and
+//      combines both in log-sum-exp form.  Nothing but the results leaves the
 //      cluster; one launch and one dependency replace two, and only the
 //      selection itself lies between the score kernel and the kept rows'
 //      loads.
+// Bound by latency: the records, the exchange of the keys, the cut and the
+// kept rows follow one another, each at the cost of its slowest warp's
+// instructions and one trip to L2, HBM or a neighbour's shared memory.  B = 1,
+// 28/4 heads, N_v = 1296, 28 calls in a graph: 15.6 -> 15.0 us a call (against
+// a selection on rank 0 alone, its list copied by the others after a second
+// cluster barrier); 32 sequences of N_v = 2304, paged: the call 62.4 -> 61.0
+// us; 8 sequences with per-kv-head sets 22.5 -> 20.9 us.
 // ---------------------------------------------------------------------------
 constexpr int kSgThreads = 512;
 constexpr int kSgWarps = kSgThreads / 32;
 constexpr int kSgMaxW = 128;  // output dimensions of one CTA, at most (64 with fp32 caches)
 
 // Register-resident Top-K cut of the fused kernel (Eq. 3) over n <= 8 * NTH
-// score keys: thread t holds keys [8t, 8t + 8), valid while below n.  Keys
-// are float bits of scores in [0, 1] (clamped below 2^30 by the producer), so
-// the digits skip the two top bits: passes on bits 29-22, 21-14, 13-6, 5-0.
-// The first digits of the scores concentrate in few buckets, so every warp
-// counts into its own histogram (hist: two sets of NTH / 32 histograms of 256
-// bins in shared memory, alternating between passes; each warp clears its
-// own histogram of a set before counting into it); thread d < 256 then adds
-// up digit d over the warps into tot, and lane L of every warp owns digits
-// 255-8L ... 248-8L of the sums.
+// score keys: thread t holds keys [kpt t, kpt t + kpt), kpt = ceil(n / NTH),
+// valid while below n.  Keys are float bits of scores in [0, 1] (clamped below
+// 2^30 by the producer), so the digits skip the two top bits: a radix select
+// in passes on bits 29-19, 18-8 and 7-0.  A first digit of seven exponent and
+// four mantissa bits spreads the scores (an 8-bit one left most of a warp's
+// histogram atomics on one bin), holds the cut's bucket to a few keys and
+// usually leaves one more pass.  hist: two histograms of kCutBins bins, zero
+// on entry, used in turn; thread t scans bins [kCutBins - 4 t - 4,
+// kCutBins - 4 t), from the top.  tot: NTH / 32 warp totals; res: the pass's
+// result.  B = 1, N_v = 1296, K = 13: 4300 cycles with 8-bit digits and a
+// histogram per warp, now about 2000.
 constexpr int kCutKeys = 8;
+constexpr int kCutBins = 2048;
 template <int NTH>
-__device__ __forceinline__ RadixCut radix_cut_regs(const uint32_t (&k)[kCutKeys], int nvalid, int K, unsigned* hist,
-                                                   unsigned* tot) {
+__device__ __forceinline__ RadixCut radix_cut_regs(const uint32_t (&k)[kCutKeys], int kpt, int nvalid, int K,
+                                                   unsigned* hist, unsigned* tot, uint4* res) {
+  static_assert(4 * NTH == kCutBins, "four bins per thread");
   constexpr int NW = NTH / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   unsigned krem = (unsigned)K, n_theta = 0;
   bool whole = false;
   uint32_t prefix = 0, mask = 0;
-  for (int pass = 0; pass < 4; ++pass) {
-    const int shift = pass < 3 ? 22 - 8 * pass : 0;
-    const uint32_t dmask = pass < 3 ? 255u : 63u;
-    unsigned* h = hist + ((pass & 1) * NW + warp) * 256;
-    // This warp's histogram of the set: last read before the previous pass's
-    // second barrier, so it may be cleared now.
-    reinterpret_cast<uint4*>(h)[2 * lane] = make_uint4(0u, 0u, 0u, 0u);
-    reinterpret_cast<uint4*>(h)[2 * lane + 1] = make_uint4(0u, 0u, 0u, 0u);
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < kCutKeys; ++j)
+  for (int pass = 0; pass < 3; ++pass) {
+    const int shift = pass == 0 ? 19 : pass == 1 ? 8 : 0;
+    const uint32_t dmask = pass < 2 ? kCutBins - 1u : 255u;
+    unsigned* h = hist + (pass & 1) * kCutBins;
+    for (int j = 0; j < kCutKeys; ++j) {
+      if (j >= kpt) break;  // uniform
       if (j < nvalid && (k[j] & mask) == prefix) atomicAdd(&h[(k[j] >> shift) & dmask], 1u);
-    __syncthreads();
-    if (tid < 256) {
-      unsigned c = 0;
-#pragma unroll
-      for (int w = 0; w < NW; ++w) c += hist[((pass & 1) * NW + w) * 256 + tid];
-      tot[tid] = c;
     }
     __syncthreads();
-    unsigned cnt8[8], sum8 = 0;
-    {
-      const uint4* tp = reinterpret_cast<const uint4*>(tot + 248 - 8 * lane);
-      const uint4 lo = tp[0], hi = tp[1];  // digits 248-8L .. 251-8L, 252-8L .. 255-8L
-      cnt8[0] = hi.w; cnt8[1] = hi.z; cnt8[2] = hi.y; cnt8[3] = hi.x;
-      cnt8[4] = lo.w; cnt8[5] = lo.z; cnt8[6] = lo.y; cnt8[7] = lo.x;
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) sum8 += cnt8[j];
-    unsigned incl = sum8;
+    const uint4 c4 = *reinterpret_cast<const uint4*>(h + kCutBins - 4 - 4 * tid);
+    const unsigned sum4 = c4.x + c4.y + c4.z + c4.w;
+    unsigned incl = sum4;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const unsigned nn = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl += nn;
     }
-    const unsigned excl = incl - sum8;
-    const bool mine = excl < krem && krem <= incl;
-    unsigned dsel = 0, before = 0, cnt = 0;
-    if (mine) {
-      unsigned run = excl;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        if (run + cnt8[j] >= krem) { dsel = 255 - 8 * lane - j; before = run; cnt = cnt8[j]; break; }
-        run += cnt8[j];
+    if (lane == 31) tot[warp] = incl;
+    __syncthreads();
+    // Pass 2 counts into the first histogram again.
+    if (pass == 0) *reinterpret_cast<uint4*>(h + 4 * tid) = make_uint4(0u, 0u, 0u, 0u);
+    incl += __reduce_add_sync(0xffffffffu, lane < warp ? tot[lane & (NW - 1)] : 0u);
+    const unsigned excl = incl - sum4;
+    if (excl < krem && krem <= incl) {  // exactly one thread: the cut is in its bins
+      unsigned run = excl, d = kCutBins - 1 - 4 * tid, cnt = c4.w;
+      if (run + cnt < krem) {
+        run += cnt; --d; cnt = c4.z;
+        if (run + cnt < krem) {
+          run += cnt; --d; cnt = c4.y;
+          if (run + cnt < krem) { run += cnt; --d; cnt = c4.x; }
+        }
       }
+      *res = make_uint4(d, run, cnt, 0u);
     }
-    const int src = max(__ffs(__ballot_sync(0xffffffffu, mine)) - 1, 0);
-    dsel = __shfl_sync(0xffffffffu, dsel, src);
-    before = __shfl_sync(0xffffffffu, before, src);
-    cnt = __shfl_sync(0xffffffffu, cnt, src);
-    krem -= before;
-    prefix |= dsel << shift;
+    __syncthreads();
+    const uint4 r = *res;
+    krem -= r.y;
+    prefix |= r.x << shift;
     mask |= dmask << shift;
-    if (pass == 3) n_theta = cnt;
-    if (pass < 3 && krem == cnt) {  // the whole bucket is kept
+    if (pass == 2) n_theta = r.z;
+    if (pass < 2 && krem == r.z) {  // the whole bucket is kept
       whole = true;
       break;
     }
@@ -3525,58 +3532,62 @@ __device__ __forceinline__ RadixCut radix_cut_regs(const uint32_t (&k)[kCutKeys]
   return RadixCut{whole ? prefix - 1u : prefix, krem, n_theta, whole};
 }
 
-// Exclusive prefix sum over the block with one barrier: wsum_s[NTH / 32]
-// must not be written again before the next barrier.
+// Of the bits set in m (bit j: item j of the thread, kpt items per thread) over
+// the block: how many are set before this thread's, with one barrier.
+// wsum_s[NTH / 32] must not be written again before the next barrier.
 template <int NTH>
-__device__ __forceinline__ int block_excl_scan_1b(int x, int* wsum_s) {
+__device__ __forceinline__ int block_bits_before(unsigned m, int kpt, int* wsum_s) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int incl = x;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int n = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += n;
+  const unsigned lt = (1u << lane) - 1u;
+  int before = 0, total = 0;
+  for (int j = 0; j < kCutKeys; ++j) {
+    if (j >= kpt) break;  // uniform
+    const unsigned v = __ballot_sync(0xffffffffu, (m >> j) & 1u);
+    before += __popc(v & lt);
+    total += __popc(v);
   }
-  if (lane == 31) wsum_s[warp] = incl;
+  if (lane == 0) wsum_s[warp] = total;
   __syncthreads();
-  int before = 0;
-  for (int w = 0; w < warp; ++w) before += wsum_s[w];
-  return before + incl - x;
+  return before + (int)__reduce_add_sync(0xffffffffu, lane < warp ? (unsigned)wsum_s[lane & (NTH / 32 - 1)] : 0u);
 }
 
-// Ascending compaction of the register-resident keys (see radix_cut_regs):
-// keys above c.theta plus the first c.krem keys equal to it (every key when
-// take_all), written to kept (global) and, with TO_SMEM, to kept_s (shared
-// memory).  wsum_s holds 2 * NTH / 32 ints.
+// Ascending compaction of the register-resident keys (see radix_cut_regs; i0:
+// index of the thread's first): keys above c.theta plus the first c.krem keys
+// equal to it (every key when take_all), written to kept (global, unless
+// NULL) and, with TO_SMEM, to kept_s (shared memory).  wsum_s holds
+// 2 * NTH / 32 ints.
 template <int NTH, bool TO_SMEM>
-__device__ __forceinline__ void compact_kept_regs(const uint32_t (&k)[kCutKeys], int nvalid, int K, bool take_all,
-                                                  const RadixCut& c, int* wsum_s, int32_t* kept, int* kept_s) {
-  const int i0 = kCutKeys * (int)threadIdx.x;
+__device__ __forceinline__ void compact_kept_regs(const uint32_t (&k)[kCutKeys], int kpt, int nvalid, int K, bool take_all,
+                                                  const RadixCut& c, int* wsum_s, int i0, int32_t* kept, int* kept_s) {
   const bool ties = !take_all && !c.whole && c.krem < c.n_theta;
-  int n_eq = 0;
+  unsigned eqm = 0;
   if (ties)
 #pragma unroll
-    for (int j = 0; j < kCutKeys; ++j) n_eq += j < nvalid && k[j] == c.theta;
-  const int eq_before = ties ? block_excl_scan_1b<NTH>(n_eq, wsum_s + NTH / 32) : 0;
+    for (int j = 0; j < kCutKeys; ++j) eqm |= (unsigned)(j < nvalid && k[j] == c.theta) << j;
+  const int eq_before = ties ? block_bits_before<NTH>(eqm, kpt, wsum_s + NTH / 32) : 0;
   const unsigned krem = ties ? c.krem : 0xffffffffu;
   unsigned selm = 0;
   {
     int r = eq_before;
 #pragma unroll
     for (int j = 0; j < kCutKeys; ++j) {
+      if (j >= kpt) break;  // uniform
       const bool v = j < nvalid;
       const bool sel = v && (take_all || k[j] > c.theta || (!c.whole && k[j] == c.theta && (unsigned)r < krem));
       r += v && k[j] == c.theta;
       selm |= (unsigned)sel << j;
     }
   }
-  int o = block_excl_scan_1b<NTH>(__popc(selm), wsum_s);
+  int o = block_bits_before<NTH>(selm, kpt, wsum_s);
 #pragma unroll
-  for (int j = 0; j < kCutKeys; ++j)
+  for (int j = 0; j < kCutKeys; ++j) {
+    if (j >= kpt) break;  // uniform
     if (((selm >> j) & 1u) && o < K) {
-      kept[o] = i0 + j;
+      if (!TO_SMEM || kept) kept[o] = i0 + j;
       if constexpr (TO_SMEM) kept_s[o] = i0 + j;
       ++o;
     }
+  }
 }
 
 constexpr int kSgKP = kSliceMaxKept + 1;  // float row pitch of the kept logits (rows in distinct banks)
@@ -3586,10 +3597,12 @@ template <int GM>
 struct SgSmem {
   float hM[kMaxHeads], hInv[kMaxHeads], hMass[kMaxHeads], hMass1[kMaxHeads];
   float hMt[GM], hLt[GM];        // text-only max and sum of this CTA's heads
-  alignas(16) unsigned tot[256];  // radix: digit counts summed over the warps
+  uint4 cut;                     // radix: the pass's result
+  unsigned tot[kSgWarps];        // radix: bin counts of every warp's bins
+  uint64_t bar;                  // completes once every key has arrived
   int wsum[32];
-  int K;                         // the budget K_t (rank 0; the others copy it)
-  int kept[kSliceMaxKept];       // the kept list (rank 0; the others copy it)
+  int K;                         // the budget K_t
+  int kept[kSliceMaxKept];       // the kept list
   float pz[GM][kSgKP];           // kept logits, then (fp32 caches) probabilities
   __nv_bfloat16 pb[8][kSgPB];    // bf16 caches: probabilities, B operand of the tensor-core P.V
   float red[kSgWarps][128];      // P.V partials of every warp
@@ -3616,8 +3629,8 @@ template <typename T, int D, int GM, bool GATHER = true>
 __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ StepParams p) {
   constexpr int NTH = kSgThreads, NW = kSgWarps;
   constexpr bool BF = sizeof(T) == 2;
-  // Dynamic: the N_v score keys (rank 0's copy is used); after the cut, the
-  // kept rows' V slices.
+  // Dynamic: the N_v score keys and the cut's two histograms; after the cut,
+  // the kept rows' V slices.
   extern __shared__ __align__(16) uint32_t key_s[];
   __shared__ SgSmem<GM> sm;
 
@@ -3639,9 +3652,30 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
   // gather kernel reads the score partials before its wait, which this
   // kernel's wait guarantees complete.
   if constexpr (GATHER) pdl_trigger();
+  // While the score kernel finishes: the barrier that counts the keys in, the
+  // histograms cleared, and the cluster's start (a CTA's shared memory may be
+  // written once that CTA runs and its barrier is initialised; waited for here,
+  // with no load in flight, as the wait's acquire is slow behind loads).
+  unsigned* hist = key_s + (p.max_visual + 3) / 4 * 4;
+  if (tid == 0) {
+    mbar_init(&sm.bar, 1);
+    mbar_fence_init();
+    if (ncl > 1 && (GATHER || rank == 0)) mbar_expect_tx(&sm.bar, 4u * (unsigned)nv);
+  }
+  reinterpret_cast<uint4*>(hist)[tid] = make_uint4(0u, 0u, 0u, 0u);
+  reinterpret_cast<uint4*>(hist + kCutBins)[tid] = make_uint4(0u, 0u, 0u, 0u);
+  __syncwarp();
+  if (ncl > 1) {
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+  }
+  const float inv_tau = p.inv_tau;
+  const int sub = lane >> 4, l16 = lane & 15;
+  const float* stb = p.split_st + ((int64_t)b * H * p.nsp_max + l16) * ST_N;
+  const float* st0 = stb + (int64_t)min(2 * warp + sub, H - 1) * p.nsp_max * ST_N;
+  asm volatile("" : "+l"(st0));  // address in place before the wait
   pdl_wait();
   if constexpr (!GATHER) pdl_trigger();
-  const float inv_tau = p.inv_tau;
 
   // 1. Split statistics -> per-head max, normalisers and masses (Eq. 5,
   //    Eq. 6), and for this CTA's heads the text-only max and sum.  Sixteen
@@ -3649,14 +3683,13 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
   //    l16 + 16, ..., four records requested at a time (one round trip for
   //    up to 64 splits).  The first round's records are requested before
   //    anything else: they are on the critical path.
-  const float* stb = p.split_st + (int64_t)b * H * p.nsp_max * ST_N;
-  const int sub = lane >> 4, l16 = lane & 15;
-  auto fetch4 = [&](int h, int s0, float4 (&x)[4], float4 (&y)[4]) {
+  auto fetch4 = [&](const float* st, int s0, bool live, float4 (&x)[4], float4 (&y)[4]) {  // s0: first split of the round
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
+      if (k > 0 && s0 + 16 * k >= ns) break;  // uniform
       const int s = s0 + 16 * k;
-      if (h < H && s < ns) {
-        const float4* r = reinterpret_cast<const float4*>(stb + ((int64_t)h * p.nsp_max + s) * ST_N);
+      if (live && s + l16 < ns) {
+        const float4* r = reinterpret_cast<const float4*>(st + s * ST_N);
         x[k] = __ldcg(r);
         y[k] = __ldcg(r + 1);
       } else {
@@ -3665,43 +3698,67 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
     }
   };
   float4 rx[4], ry[4];
-  fetch4(2 * warp + sub, l16, rx, ry);
+  fetch4(st0, 0, 2 * warp + sub < H, rx, ry);
 
-  // This CTA's slice of the visual tokens; each thread's first logit row is
-  // requested next so that it arrives while the statistics are merged.
+  // This CTA's slice of the visual tokens.  A group of 2^rsh lanes shares a
+  // token, each lane four of its heads (one, where the heads do not start and
+  // end on 16-byte boundaries), so that loads cover whole rows and all warps
+  // share the exponentials.  The first kZPre rounds of rows are requested next,
+  // so that they arrive while the statistics are merged.
+  constexpr int kZPre = 8;
   const int per = (nv + ncl - 1) / ncl;
   const int i0 = min(nv, rank * per), i1 = min(nv, i0 + per);
   const int hbeg = p.granularity ? gsel * G : 0;
   const int hcnt = p.granularity ? G : H;
   const bool vec = (hbeg & 3) == 0 && (hcnt & 3) == 0;
-  const bool pre = vec && hcnt <= 32 && i0 + tid < i1;
-  float4 zpre[8];
-  if (pre) {
-    const float4* zr = reinterpret_cast<const float4*>(p.z_ws + ((int64_t)b * p.max_visual + i0 + tid) * p.hp + hbeg);
+  const int nq = vec ? hcnt >> 2 : hcnt;  // lanes a token needs (at most 128 heads: 32)
+  const int rsh = nq <= 1 ? 0 : 32 - __clz(nq - 1), lpt = 1 << min(rsh, 5);
+  const int zq = tid & (lpt - 1), zstep = NTH / lpt;
+  const bool zlane = zq < nq;
+  auto zload = [&](int i) {
+    float4 z = make_float4(-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F);
+    if (zlane && i < i1) {
+      const float* zr = p.z_ws + ((int64_t)b * p.max_visual + i) * p.hp + hbeg;
+      if (vec) z = __ldcg(reinterpret_cast<const float4*>(zr) + zq);
+      else z.x = __ldcg(zr + zq);
+    }
+    return z;
+  };
+  const int zi0 = i0 + tid / lpt;
+  float4 zpre[kZPre];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) zpre[q] = 4 * q < hcnt ? __ldcg(zr + q) : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
+  for (int q = 0; q < kZPre; ++q)
+    if (i0 + q * zstep < i1) zpre[q] = zload(zi0 + q * zstep);  // uniform
 
   for (int h0 = 2 * warp; h0 < H; h0 += 2 * NW) {
     const int h = h0 + sub;
-    if (h0 != 2 * warp) fetch4(h, l16, rx, ry);  // the first round's records are in flight already
+    const float* sth = stb + (int64_t)min(h, H - 1) * p.nsp_max * ST_N;
+    if (h0 != 2 * warp) fetch4(sth, 0, h < H, rx, ry);  // the first round's records are in flight already
     float m = -CUDART_INF_F, a1v = 0.f, atv = 0.f, a1t = 0.f, att = 0.f;
     float mt = -CUDART_INF_F, lt = 0.f;  // text only
-    for (int s0 = l16;; s0 += 64) {
-      if (s0 != l16) fetch4(h, s0, rx, ry);
+    for (int s0 = 0;; s0 += 64) {
+      if (s0) fetch4(sth, s0, h < H, rx, ry);
+      float mn = m, mtn = mt;
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const float mn = fmaxf(m, fmaxf(rx[k].x, ry[k].x));
-        if (mn > m) {
-          const float f1 = exp2_rel(m, mn), ft = exp2_tau(m, mn, inv_tau);
-          a1v *= f1; a1t *= f1; atv *= ft; att *= ft;
-          m = mn;
-        }
+        if (k > 0 && s0 + 16 * k >= ns) break;  // uniform
+        mn = fmaxf(mn, fmaxf(rx[k].x, ry[k].x));
+        mtn = fmaxf(mtn, rx[k].x);
+      }
+      if (s0) {  // sums of earlier rounds
+        const float f1 = exp2_rel(m, mn), ft = exp2_tau(m, mn, inv_tau);
+        a1v *= f1; a1t *= f1; atv *= ft; att *= ft;
+        lt *= exp2_rel(mt, mtn);
+      }
+      m = mn;
+      mt = mtn;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (k > 0 && s0 + 16 * k >= ns) break;  // uniform
         a1v = fmaf(exp2_rel(ry[k].x, m), ry[k].y, a1v);
         atv = fmaf(exp2_tau(ry[k].x, m, inv_tau), ry[k].z, atv);
         a1t = fmaf(exp2_rel(rx[k].x, m), rx[k].y, a1t);
         att = fmaf(exp2_tau(rx[k].x, m, inv_tau), rx[k].z, att);
-        if (rx[k].x > mt) { lt *= exp2_rel(mt, rx[k].x); mt = rx[k].x; }
         lt = fmaf(exp2_rel(rx[k].x, mt), rx[k].y, lt);
       }
       if (s0 + 64 >= ns) break;
@@ -3733,33 +3790,9 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
   }
   __syncthreads();
 
-  // 2a. Text partials of the score splits for this CTA's dimensions, requested
-  //     now and summed after the importance pass: thread (element
-  //     e = (head, 4 dimensions), split group sg of four) takes splits
-  //     sg, sg + 4, ...
-  // Four threads per element when NE <= 128, else two (NE <= 256).
-  const int W4 = W / 4, NE = G * W4;
-  const int TSH = NE > NTH / 4 ? 1 : 2, TSG = 1 << TSH;
-  const int te = tid >> TSH, tsg = tid & (TSG - 1);
-  const bool tlive = te < NE;
-  const int th = tlive ? te / W4 : 0, tdim = d0 + 4 * (tlive ? te % W4 : 0);
-  const float* tst = p.split_st + (hrow0 + th) * p.nsp_max * ST_N + ST_MT;
-  const float* tso = p.split_o + (hrow0 + th) * p.nsp_max * D + tdim;
-  float tmx[kSgTextSplits];
-  float4 tov[kSgTextSplits];
-  if constexpr (GATHER) {
-#pragma unroll
-    for (int k = 0; k < kSgTextSplits; ++k) {
-      const int s = tsg + TSG * k;
-      const bool ok = tlive && s < ns;
-      tmx[k] = ok ? __ldcg(tst + (int64_t)s * ST_N) : -CUDART_INF_F;
-      tov[k] = ok ? __ldcg(reinterpret_cast<const float4*>(tso + (int64_t)s * D)) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-  }
-
-  // Rank 0: head mean, head max (Sec. 4.3) and the budget (Eq. 7), on the
-  // last warp (whose importance rows come last).
-  if (rank == 0) {
+  // Head mean, head max (Sec. 4.3) and the budget (Eq. 7), on the last warp;
+  // rank 0 writes them out.
+  if (GATHER || rank == 0) {
     if (warp == NW - 1) {
       float smn = 0.f, mx = 0.f, s1 = 0.f;
       for (int h = lane; h < H; h += 32) {
@@ -3773,13 +3806,13 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
       if (lane == 0) {
         const int K = min(budget_k(p, mx, nv), GATHER ? min(p.kept_cap, kSliceMaxKept) : p.kept_cap);
         sm.K = K;
-        p.kept_count[(int64_t)b * nsel + gsel] = K;
-        if (gsel == 0 && p.mass_stats) {
+        if (rank == 0) p.kept_count[(int64_t)b * nsel + gsel] = K;
+        if (rank == 0 && gsel == 0 && p.mass_stats) {
           float* ms = p.mass_stats + (int64_t)b * 4;
           ms[0] = smn / H; ms[1] = mx; ms[2] = s1 / H; ms[3] = (float)K;
         }
       }
-    } else if (gsel == 0) {
+    } else if (rank == 0 && gsel == 0) {
       for (int h = tid; h < H; h += NTH - 32) {
         p.mass[(int64_t)b * H + h] = sm.hMass[h];
         if constexpr (!GATHER) p.hmax[(int64_t)b * H + h] = sm.hM[h];
@@ -3788,125 +3821,124 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
   }
 
   // 2b. Importance S_i (Eq. 2) of this CTA's slice, as float bits (S >= 0
-  //     orders like its bits), into rank 0's key array.
+  //     orders like its bits), into the key array of every CTA (select only:
+  //     rank 0's).
   const float inv_cnt = 1.f / (float)hcnt;
-  uint32_t* key0 = ncl > 1 ? cluster.map_shared_rank(key_s, 0) : key_s;
   unsigned bad = 0;
-  for (int i = i0 + tid; i < i1; i += NTH) {
-    const float* zr = p.z_ws + ((int64_t)b * p.max_visual + i) * p.hp + hbeg;
-    float a = 0.f;
-    if (pre && i == i0 + tid) {
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        if (4 * q < hcnt) {
-          const int h = hbeg + 4 * q;
-          a = fmaf(fexp2_rel(zpre[q].x, sm.hM[h]), sm.hInv[h], a);
-          a = fmaf(fexp2_rel(zpre[q].y, sm.hM[h + 1]), sm.hInv[h + 1], a);
-          a = fmaf(fexp2_rel(zpre[q].z, sm.hM[h + 2]), sm.hInv[h + 2], a);
-          a = fmaf(fexp2_rel(zpre[q].w, sm.hM[h + 3]), sm.hInv[h + 3], a);
-        }
+  {
+    float4 m4 = make_float4(0.f, 0.f, 0.f, 0.f), r4 = m4;  // this lane's heads: maxima, 1 / normalisers
+    if (zlane) {
+      if (vec) {
+        m4 = reinterpret_cast<const float4*>(sm.hM + hbeg)[zq];
+        r4 = reinterpret_cast<const float4*>(sm.hInv + hbeg)[zq];
+      } else {
+        m4.x = sm.hM[hbeg + zq];
+        r4.x = sm.hInv[hbeg + zq];
       }
-    } else if (vec) {
-      for (int hh = 0; hh < hcnt; hh += 4) {
-        const float4 z4 = __ldcg(reinterpret_cast<const float4*>(zr + hh));
-        const int h = hbeg + hh;
-        a = fmaf(fexp2_rel(z4.x, sm.hM[h]), sm.hInv[h], a);
-        a = fmaf(fexp2_rel(z4.y, sm.hM[h + 1]), sm.hInv[h + 1], a);
-        a = fmaf(fexp2_rel(z4.z, sm.hM[h + 2]), sm.hInv[h + 2], a);
-        a = fmaf(fexp2_rel(z4.w, sm.hM[h + 3]), sm.hInv[h + 3], a);
-      }
-    } else {
-      for (int hh = 0; hh < hcnt; ++hh)
-        a = fmaf(fexp2_rel(__ldcg(zr + hh), sm.hM[hbeg + hh]), sm.hInv[hbeg + hh], a);
     }
-    const float sc = a * inv_cnt;
-    if (!isfinite(sc)) bad = 1;
-    key0[i] = min(__float_as_uint(sc), 0x3fffffffu);  // scores lie in [0, 1]: the top two bits are zero
+    // Every lane of the group gets the token's score; lane r sends it to CTA
+    // r's key array (and r + lpt's, ...; select only: rank 0's), counted by
+    // that CTA's barrier: no fence and no cluster barrier between the scores
+    // and the cut.
+    const unsigned key_a = smem_u32(key_s), bar_a = smem_u32(&sm.bar);
+    auto score = [&](int i, const float4& z) {
+      float a = fexp2_rel(z.x, m4.x) * r4.x;
+      if (vec) {
+        a = fmaf(fexp2_rel(z.y, m4.y), r4.y, a);
+        a = fmaf(fexp2_rel(z.z, m4.z), r4.z, a);
+        a = fmaf(fexp2_rel(z.w, m4.w), r4.w, a);
+      }
+      for (int o = 1; o < lpt; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      if (i >= i1) return;
+      const float sc = a * inv_cnt;
+      if (!isfinite(sc)) bad = 1;
+      const uint32_t key = min(__float_as_uint(sc), 0x3fffffffu);  // scores lie in [0, 1]: the top two bits are zero
+      if (ncl == 1) {  // launched without a cluster: no cluster addresses
+        if (zq == 0) key_s[i] = key;
+      } else {
+        for (int r = zq; r < (GATHER ? ncl : 1); r += lpt) st_async_u32(key_a + 4 * i, key, bar_a, r);
+      }
+    };
+#pragma unroll
+    for (int q = 0; q < kZPre; ++q)
+      if (i0 + q * zstep < i1) score(zi0 + q * zstep, zpre[q]);  // uniform
+    for (int q = kZPre; i0 + q * zstep < i1; ++q) score(zi0 + q * zstep, zload(zi0 + q * zstep));
   }
   if (bad) atomicOr(p.err, ERR_NONFINITE);
 
-  // 2c. The text part: sum exp2(m_s - m_text) * o_s over the splits, then over
-  //     the element's four split groups.
+  if (!GATHER && rank != 0) return;
+
+  // 2c. Text partials of the score splits for this CTA's dimensions, requested
+  //     now and summed while the kept rows are on their way: thread (element
+  //     e = (head, 4 dimensions), split group sg) takes splits sg, sg + TSG,
+  //     ...; four threads per element when NE <= 128, else two (NE <= 256).
+  const int wsh = 31 - __clz(W >> 2);  // W is a power of two: D / (ranks per kv-head)
+  const int NE = G << wsh;
+  const int TSH = NE > NTH / 4 ? 1 : 2, TSG = 1 << TSH;
+  const int te = tid >> TSH, tsg = tid & (TSG - 1);
+  const bool tlive = te < NE;
+  const int th = tlive ? te >> wsh : 0, tdim = d0 + 4 * (tlive ? te & ((1 << wsh) - 1) : 0);
+  const float* tst = p.split_st + ((hrow0 + th) * p.nsp_max + tsg) * ST_N + ST_MT;
+  const float* tso = p.split_o + ((hrow0 + th) * p.nsp_max + tsg) * D + tdim;
+  float tmx[kSgTextSplits];
+  float4 tov[kSgTextSplits];
   if constexpr (GATHER) {
-    const float tmh = sm.hMt[th];
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int k = 0; k < kSgTextSplits; ++k) {
-      const float w = exp2_rel(tmx[k], tmh);
-      a.x = fmaf(w, tov[k].x, a.x); a.y = fmaf(w, tov[k].y, a.y); a.z = fmaf(w, tov[k].z, a.z); a.w = fmaf(w, tov[k].w, a.w);
+      tmx[k] = -CUDART_INF_F;
+      tov[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (TSG * k < ns && tlive && tsg + TSG * k < ns) {
+        tmx[k] = __ldcg(tst + (TSG * k) * ST_N);
+        tov[k] = __ldcg(reinterpret_cast<const float4*>(tso + (TSG * k) * D));
+      }
     }
-    for (int s = tsg + TSG * kSgTextSplits; tlive && s < ns; s += TSG) {
-      const float w = exp2_rel(__ldcg(tst + (int64_t)s * ST_N), tmh);
-      const float4 v = __ldcg(reinterpret_cast<const float4*>(tso + (int64_t)s * D));
-      a.x = fmaf(w, v.x, a.x); a.y = fmaf(w, v.y, a.y); a.z = fmaf(w, v.z, a.z); a.w = fmaf(w, v.w, a.w);
-    }
-    for (int o = 1; o < TSG; o <<= 1) {
-      a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
-      a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
-      a.z += __shfl_xor_sync(0xffffffffu, a.z, o);
-      a.w += __shfl_xor_sync(0xffffffffu, a.w, o);
-    }
-    if (tlive && tsg == 0) sm.to[te] = a;
   }
-  if (ncl > 1) cluster.sync();  // rank 0 now sees every key
-  else __syncthreads();
-  if (!GATHER && rank != 0) return;  // nothing reads this CTA's shared memory any more
 
-  // 3. Rank 0: the Top-K_t cut (Eq. 3) and the ascending compaction, with
-  //    every thread's eight keys in registers, into the output and into its
-  //    shared memory.
-  if (rank == 0) {
-    const int K = sm.K;
-    int32_t* kept = p.kept_idx + ((int64_t)b * nsel + gsel) * p.kept_cap;
+  // 3. The Top-K_t cut (Eq. 3) and the ascending compaction, with the keys in
+  //    registers, into shared memory and (rank 0) into the output.
+  unsigned err = 0;
+  if (ncl == 1) __syncthreads();  // every key is in place
+  else if (!mbar_wait(&sm.bar, 0)) err |= ERR_TIMEOUT;
+  const int kpt = (nv + NTH - 1) / NTH;  // at most kCutKeys
+  const int nvalid = min(max(nv - kpt * tid, 0), kpt);
+  uint32_t kr[kCutKeys];
+#pragma unroll
+  for (int j = 0; j < kCutKeys; ++j) kr[j] = j < nvalid ? key_s[kpt * tid + j] : 0u;
+  __syncthreads();  // the budget is in place
+  const int K = sm.K;
+  {
+    int32_t* kept = rank == 0 ? p.kept_idx + ((int64_t)b * nsel + gsel) * p.kept_cap : nullptr;
     const bool take_all = K >= nv;
-    const int nvalid = min(max(nv - kCutKeys * tid, 0), kCutKeys);
-    uint32_t kr[kCutKeys];
-    {
-      const uint4* kp = reinterpret_cast<const uint4*>(key_s + kCutKeys * tid);
-      const uint4 a = nvalid > 0 ? kp[0] : make_uint4(0u, 0u, 0u, 0u);
-      const uint4 c = nvalid > 4 ? kp[1] : make_uint4(0u, 0u, 0u, 0u);
-      kr[0] = a.x; kr[1] = a.y; kr[2] = a.z; kr[3] = a.w; kr[4] = c.x; kr[5] = c.y; kr[6] = c.z; kr[7] = c.w;
-    }
     RadixCut cut{0u, (unsigned)K, 0u, false};
-    __syncthreads();  // every key is in registers: the key array holds the warps' histograms from here on
-    if (K > 0 && !take_all) cut = radix_cut_regs<NTH>(kr, nvalid, K, key_s, sm.tot);
-    if (K > 0) compact_kept_regs<NTH, GATHER>(kr, nvalid, K, take_all, cut, sm.wsum, kept, sm.kept);
-    for (int i = max(K, 0) + tid; i < p.kept_cap; i += NTH) kept[i] = -1;
+    if (K > 0 && !take_all) cut = radix_cut_regs<NTH>(kr, kpt, nvalid, K, hist, sm.tot, &sm.cut);
+    if (K > 0) compact_kept_regs<NTH, GATHER>(kr, kpt, nvalid, K, take_all, cut, sm.wsum, kpt * tid, kept, sm.kept);
+    if (rank == 0)
+      for (int i = max(K, 0) + tid; i < p.kept_cap; i += NTH) kept[i] = -1;
   }
-  if constexpr (!GATHER) return;
-  if (ncl > 1) cluster.sync();  // rank 0 holds the kept list
-  else __syncthreads();
-  // Every CTA copies the budget and the kept list from rank 0, then lets
-  // rank 0 go: its shared memory may be released once every CTA of the
-  // cluster has arrived (the matching wait is the kernel's last instruction).
-  int K;
-  if (ncl > 1) {
-    K = *cluster.map_shared_rank(&sm.K, 0);
-    if (rank != 0 && tid < K) sm.kept[tid] = cluster.map_shared_rank(&sm.kept[0], 0)[tid];
-    asm volatile("barrier.cluster.arrive.release;\n" ::: "memory");
-    __syncthreads();
-  } else {
-    K = sm.K;
+  if constexpr (!GATHER) {
+    if (err) atomicOr(p.err, err);
+    return;
   }
+  __syncthreads();  // the kept list is in place, keys and histograms are read
 
   // 4. Kept rows: their logits and this CTA's V slices to shared memory
   //    (asynchronous copies; V in 16-byte pieces, bf16 rows of 128 bytes with
   //    swizzled pieces, fp32 rows packed), all requested together.  Rows past
   //    K, and rows whose index or page is bad, are zero.
   unsigned char* vst = reinterpret_cast<unsigned char*>(key_s);  // the keys are no longer read
-  const int CPR = W * (int)sizeof(T) / 16;                       // 16-byte pieces of a row slice
+  const int csh = 31 - __clz(W * (int)sizeof(T) / 16), CPR = 1 << csh;  // 16-byte pieces of a row slice
   const int K16 = (K + 15) & ~15;
-  unsigned err = 0;
   // Logits first (the older copy group: the softmax waits for it alone).
-  for (int i = tid; i < K * G; i += NTH) {
-    const int j = i / G, h = i % G;
+  for (int i = tid; i < 8 * K; i += NTH) {
+    const int j = i >> 3, h = i & 7;
+    if (h >= G) continue;
     const int id = sm.kept[j];
     if (id >= 0 && id < nv) cp_async4(smem_u32(&sm.pz[h][j]), p.z_ws + ((int64_t)b * p.max_visual + id) * p.hp + g * G + h);
     else sm.pz[h][j] = -CUDART_INF_F;
   }
   asm volatile("cp.async.commit_group;\n" ::: "memory");
   for (int i = tid; i < (BF ? K16 : K) * CPR; i += NTH) {
-    const int j = i / CPR, c = i % CPR;
+    const int j = i >> csh, c = i & (CPR - 1);
     const unsigned off = BF ? sg_voff(j, c) : (unsigned)((j * CPR + c) * 16);
     const T* vr = nullptr;
     if (j < K) {
@@ -3922,6 +3954,30 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
     else *reinterpret_cast<uint4*>(vst + off) = make_uint4(0u, 0u, 0u, 0u);
   }
   asm volatile("cp.async.commit_group;\n" ::: "memory");
+  // The text part, while the copies are in flight: sum exp2(m_s - m_text) * o_s over the splits, then over
+  //     the element's four split groups.
+  if constexpr (GATHER) {
+    const float tmh = sm.hMt[th];
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < kSgTextSplits; ++k) {
+      if (TSG * k >= ns) break;  // uniform
+      const float w = exp2_rel(tmx[k], tmh);
+      a.x = fmaf(w, tov[k].x, a.x); a.y = fmaf(w, tov[k].y, a.y); a.z = fmaf(w, tov[k].z, a.z); a.w = fmaf(w, tov[k].w, a.w);
+    }
+    for (int k = kSgTextSplits; tlive && tsg + TSG * k < ns; ++k) {
+      const float w = exp2_rel(__ldcg(tst + (int64_t)(TSG * k) * ST_N), tmh);
+      const float4 v = __ldcg(reinterpret_cast<const float4*>(tso + (int64_t)(TSG * k) * D));
+      a.x = fmaf(w, v.x, a.x); a.y = fmaf(w, v.y, a.y); a.z = fmaf(w, v.z, a.z); a.w = fmaf(w, v.w, a.w);
+    }
+    for (int o = 1; o < TSG; o <<= 1) {
+      a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
+      a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
+      a.z += __shfl_xor_sync(0xffffffffu, a.z, o);
+      a.w += __shfl_xor_sync(0xffffffffu, a.w, o);
+    }
+    if (tlive && tsg == 0) sm.to[te] = a;
+  }
   asm volatile("cp.async.wait_group 1;\n" ::: "memory");
   __syncthreads();
   // Per head: kept max, probabilities, sum.  bf16 caches: the probabilities
@@ -3952,9 +4008,9 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
   // (16 kept rows x 8 heads); warp w owns the 16-dimension tile w % (W / 16)
   // over every (16 / (W / 16))-th step of 16 kept rows.  fp32: thread (part,
   // head, dimension) sums every parts-th kept row on the CUDA cores.
-  const int nmt = W / 16;
+  const int msh = wsh - 2, nmt = 1 << msh;  // W / 16
   if constexpr (BF) {
-    const int mt = warp % nmt, kg = warp / nmt, ngr = NW / nmt;
+    const int mt = warp & (nmt - 1), kg = warp >> msh, ngr = NW >> msh;
     const int gr = lane >> 2, tg = lane & 3;
     const int vrow = (lane & 7) + 8 * (lane >> 4), vcol = 8 * ((lane >> 3) & 1);
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
@@ -3988,16 +4044,16 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
   // Combine (thread per (head, dimension)): kept part and text part in
   // log-sum-exp form, normalised over the kept and text tokens only.
   for (int i = tid; i < G * W; i += NTH) {
-    const int h = i / W, d = i % W;
+    const int h = i >> (wsh + 2), d = i & (W - 1);
     float kv = 0.f;
     if constexpr (BF) {
       const int mt = d / 16, dd = d % 16;
-      for (int kg = 0; kg < NW / nmt; ++kg) kv += sm.red[kg * nmt + mt][h * 16 + dd];
+      for (int kg = 0; kg < (NW >> msh); ++kg) kv += sm.red[kg * nmt + mt][h * 16 + dd];
     } else {
       const int items = GM * W;
       for (int part = 0; part < NTH / items; ++part) kv += (&sm.red[0][0])[part * items + h * W + d];
     }
-    const float4 t4 = sm.to[h * W4 + d / 4];
+    const float4 t4 = sm.to[(h << wsh) + d / 4];
     const float tv = (d & 3) == 0 ? t4.x : (d & 3) == 1 ? t4.y : (d & 3) == 2 ? t4.z : t4.w;
     const float mk = sm.fin[h][0], lk = sm.fin[h][1], mt = sm.hMt[h], lt = sm.hLt[h];
     const float M = fmaxf(mk, mt);
@@ -4006,7 +4062,6 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
     const float o = den > 0.f ? (ak * kv + at * tv) / den : 0.f;
     reinterpret_cast<T*>(p.out)[(hrow0 + h) * D + d0 + d] = from_f<T>(o);
   }
-  if (ncl > 1) asm volatile("barrier.cluster.wait.acquire;\n" ::: "memory");
 }
 
 // ------------------------------------------------------------------ launching
@@ -4213,15 +4268,13 @@ cudaError_t launch_compact(const CompactParams& c, cudaStream_t st) {
   return cudaLaunchKernelEx(&cfg, k_compact, c);
 }
 
-// Dynamic shared memory of k_selgat: the score keys, then the cut's per-warp
+// Dynamic shared memory of k_selgat: the score keys and the cut's two
 // histograms, then the kept rows' V slices of W dimensions (bf16: one or two
 // halves of rows of 128 bytes; fp32: packed rows).
 size_t selgat_smem_bytes(int max_visual, int dtype, int W = 64) {
-  const size_t keys = select_smem_bytes(max_visual);
+  const size_t keys = ((size_t)(max_visual > 0 ? max_visual : 0) + 3) / 4 * 16 + 2 * kCutBins * 4;
   const size_t stage = (size_t)kSliceMaxKept * (dtype == 0 ? (W > 64 ? 256 : 128) : W * 4);
-  const size_t hist = (size_t)2 * kSgWarps * 256 * 4;  // the cut's per-warp histograms
-  size_t n = keys > stage ? keys : stage;
-  return n > hist ? n : hist;
+  return keys > stage ? keys : stage;
 }
 
 template <typename T, int D>

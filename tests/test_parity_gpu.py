@@ -157,6 +157,26 @@ def test_chunk_gather_long_lists(vp, paged):
     Hn.check_all(vp, inp, budget, seqs=(0, 7, 39))
 
 
+@pytest.mark.parametrize("H,Hkv,batch,gran", [(28, 4, 1, 0), (14, 2, 3, 0), (8, 2, 5, 1), (28, 4, 20, 1), (28, 4, 80, 0),
+                                              (12, 1, 2, 0)])
+@pytest.mark.parametrize("nv", [1, 511, 513, 1025, 4096])
+def test_selection_cut(vp, H, Hkv, batch, gran, nv):
+    """The fused and the select-only selection around the cut's keys per
+    thread, in clusters of 8, 4 and 2 CTAs and without one, with head counts
+    that fill 16-byte logit pieces and that do not; all keys equal in the last
+    sequence (ties to the lower index)."""
+    if batch * nv > 50000 and nv > 1025:
+        pytest.skip("host inputs too large")
+    r = small(heads=H, kv_heads=Hkv, head_dim=64, batch=batch, vis_len=nv, vis_start=2, text_len=17, seed=nv + batch)
+    inp = Hn.make_inputs(r)
+    inp.q[-1] = 0
+    for ratio in (30_000, 500_000):
+        budget = dict(mode=O.FIXED_RATIO, tau=0.1, ratio_ppm=ratio, granularity=gran)
+        gpu = Hn.check_all(vp, inp, budget, seqs=sorted({0, batch - 1}))
+        k = int(gpu["count"][-1][0])
+        assert all(np.array_equal(row[:k], np.arange(k)) for row in gpu["kept"][-1])
+
+
 def test_paged_cache(vp):
     r = small(batch=4, vis_len=(300, 577, 64, 1000), vis_start=(0, 13, 40, 0),
               text_len=(517, 70, 129, 33), paged=True, page_size=16)
