@@ -148,7 +148,7 @@ vp_status vp_init(const vp_config* cfg, vp_ctx** out_ctx);
  * previous call of this library on the same stream finish (programmatic
  * dependent launch), and vp_decode_step reads q, the caches, spans, lengths
  * and page table before it waits for that call (it waits before its first
- * workspace write).  So no input of vp_decode_step may be written by the
+ * write to memory that call still uses).  So no input of vp_decode_step may be written by the
  * immediately preceding call of this library on the stream; any other kernel
  * or copy in between removes the overlap.  vp_compact_kv's output caches are
  * exempt (its kernel completes before the next call starts), and

@@ -41,6 +41,7 @@ struct vp_ctx {
   int64_t tcalls = 0;
   int32_t last_score_path = 0;  // vp_last_launch: score kernel and kernel count of the last call
   int32_t last_kernels = 0;
+  bool second_set = false;  // which set of the score kernel's outputs the next call uses
 };
 
 namespace {
@@ -62,6 +63,16 @@ vp_status cuda_fail(vp_ctx* ctx, const char* what, cudaError_t e) {
 }
 
 int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
+
+// The set of the score kernel's outputs for a call about to be enqueued.
+void take_set(vp_ctx* ctx, vp::StepParams& p) {
+  const size_t off = ctx->second_set ? ctx->lay.o_set2 / sizeof(float) : 0;
+  p.z_ws = ctx->z_ws + off;
+  p.split_st = ctx->split_st + off;
+  p.split_o = ctx->split_o + off;
+  p.ws_free = ctx->lay.o_set2 != 0;
+  if (p.ws_free) ctx->second_set = !ctx->second_set;
+}
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -174,7 +185,8 @@ vp_status vp_init(const vp_config* cfg, vp_ctx** out_ctx) {
     return st;
   }
   ctx->lay = vp::ws_layout(c.max_batch, c.num_q_heads, c.num_kv_heads, c.head_dim, c.max_visual, c.max_seq,
-                          ctx->num_sms);
+                          ctx->num_sms,
+                          vp::two_sets(c.max_batch, c.num_kv_heads, c.head_dim, c.max_seq, c.dtype == VP_BF16 ? 2 : 4));
   const vp::WsLayout& L = ctx->lay;
   const size_t off = L.total;
   ctx->ws_bytes = off;
@@ -261,7 +273,6 @@ vp_status vp_decode_step(vp_ctx* ctx, int32_t batch, const void* q,
   p.ratio_ppm = budget->ratio_ppm; p.fixed_k = budget->fixed_k;
   p.out = out; p.kept_idx = kept_idx; p.kept_cap = kept_cap; p.kept_count = kept_count;
   p.mass = mass; p.mass_stats = mass_stats;
-  p.z_ws = ctx->z_ws; p.split_st = ctx->split_st; p.split_o = ctx->split_o;
   p.gpart_o = ctx->gpart_o; p.gpart_st = ctx->gpart_st; p.tickets = ctx->tickets; p.err = ctx->err;
   p.hp = ctx->lay.hp;
   p.nsp_max = ctx->lay.nsp_max;
@@ -278,6 +289,7 @@ vp_status vp_decode_step(vp_ctx* ctx, int32_t batch, const void* q,
   }
   p.fused = vp::select_kind(p, kept_cap);
 
+  take_set(ctx, p);
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   cudaEvent_t* tev = nullptr;
   unsigned rec_flags = cudaEventRecordDefault;
@@ -355,7 +367,6 @@ vp_status vp_decode_gather(vp_ctx* ctx, int32_t batch, const void* q,
   p.kept_cap = kept_cap;
   p.kept_count = const_cast<int32_t*>(kept_count);
   p.out = out;
-  p.z_ws = ctx->z_ws; p.split_st = ctx->split_st; p.split_o = ctx->split_o;
   p.gpart_o = ctx->gpart_o; p.gpart_st = ctx->gpart_st; p.tickets = ctx->tickets; p.err = ctx->err;
   p.mt_o = ctx->mt_o; p.mt_st = ctx->mt_st; p.hmax = ctx->hmax;
   // Score splits as planned for the decode step; their weight covers the
@@ -372,6 +383,7 @@ vp_status vp_decode_gather(vp_ctx* ctx, int32_t batch, const void* q,
   if (!p.use_tma)
     return fail(ctx, VP_ERR_UNSUPPORTED, "vp_decode_gather: the cache layout needs the bulk-tensor path "
                 "(token axis not outermost, pages of at least 8 tokens)");
+  take_set(ctx, p);
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   cudaError_t e = vp::launch_score(p, st);
   if (e != cudaSuccess) return cuda_fail(ctx, "vp_decode_gather: score kernel launch", e);

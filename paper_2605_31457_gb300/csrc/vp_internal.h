@@ -88,6 +88,8 @@ struct StepParams {
   int act_words;
   unsigned* tickets;  // [max_batch][Hkv] (zero between calls)
   unsigned* err;      // device error word
+  int ws_free;        // 1: no kernel still running reads z_ws, split_st and split_o (two sets in turn): the score
+                      // kernel writes them at once and waits for the previous kernel only before it ends
   int hp;             // z_ws row stride (H rounded up to a multiple of 4)
   int ns, nsp_max;    // score splits (= text partials) per (sequence, kv-head); allocated
   int cl;             // CTAs in a select cluster
@@ -247,14 +249,34 @@ inline int split_floor(const Plan& pl, int batch, int Hkv, int num_sms, bool tc,
 
 // Workspace layout for up to `batch` sequences (offsets in bytes, 256-aligned).
 // The first `zero_bytes` (tickets, error word) must be zero before a call.
+// With two_sets, what the score kernel writes (logits, split statistics, text
+// partials) has a second set o_set2 bytes after the first; a context's calls
+// use the sets in turn, so that a score kernel does not wait for the previous
+// call's select and gather kernels before it writes.  Set n % 2 is free when
+// call n's score kernel starts: in such a context the last kernel of call
+// n - 1 lets it start only after that kernel's own wait, so the score kernel of
+// call n - 1 is complete, and every score kernel waits, before it ends, for the
+// last kernel of the call before it, here that of call n - 2.
+// Contexts whose calls span at most kSet2Cache bytes of cache use two sets:
+// their score kernel is shorter than the select kernel it then overlaps (B = 1,
+// 28 calls in a graph: 15.0 -> 12.1 us a call).  Larger calls keep one set and
+// the early start of the next score kernel, whose text tiles fill the drain of
+// the current one (8 sequences of 4096 + 16384 tokens: 51.8 us, two sets 55.4;
+// top-p on 16 of 6400 + 1024: 83.4 against 85.8).
+constexpr size_t kSet2Cache = (size_t)64 << 20;
+inline bool two_sets(int batch, int Hkv, int D, int max_seq, int esz) {
+  return (size_t)batch * Hkv * max_seq * D * esz * 2 <= kSet2Cache;
+}
 struct WsLayout {
   size_t o_tickets, o_err, zero_bytes, o_z, o_st, o_o, o_go, o_gs, o_mo, o_ms, o_hm, total;
+  size_t o_set2;  // 0: one set
   int hp, nsp_max, nk_max;
 };
 
 inline size_t ws_round(size_t x) { return (x + 255) / 256 * 256; }
 
-inline WsLayout ws_layout(int batch, int H, int Hkv, int D, int max_visual, int max_seq, int num_sms) {
+inline WsLayout ws_layout(int batch, int H, int Hkv, int D, int max_visual, int max_seq, int num_sms,
+                          bool second_set = false) {
   WsLayout w;
   w.hp = (H + 3) / 4 * 4;
   w.nk_max = kNkMax;
@@ -277,6 +299,11 @@ inline WsLayout ws_layout(int batch, int H, int Hkv, int D, int max_visual, int 
   w.o_mo = off; off = ws_round(off + B * H * (size_t)D * 4);
   w.o_ms = off; off = ws_round(off + B * H * 2 * 4);
   w.o_hm = off; off = ws_round(off + B * H * 4);
+  w.o_set2 = 0;
+  if (second_set) {
+    w.o_set2 = off - w.o_z;
+    off += w.o_go - w.o_z;
+  }
   w.total = off;
   return w;
 }

@@ -25,8 +25,10 @@
 // griddepcontrol.wait.  The slice gather kernel reads the call's inputs and
 // the score kernel's partials before its wait: the select kernel between them
 // lets its dependents start only after its own wait on the score kernel, so
-// both are complete by then.  Each kernel also lets its own dependent start
-// only after that wait, so the next call cannot overwrite the workspace early.
+// both are complete by then.  A score kernel waits for the previous kernel
+// before its first write; with two sets of the score kernels' outputs
+// (p.ws_free, see WsLayout) it writes at once and waits before it ends, and the
+// last kernel of a call lets the next one start only after its own wait.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -978,7 +980,7 @@ __global__ void __launch_bounds__(32 * NW, 1) k_score_tma(const __grid_constant_
   // The workspace (logits, partials) may still be read by the previous
   // kernel: each thread waits for it only before its first workspace write,
   // so splits of text tiles stream their whole range meanwhile.
-  bool ws_ok = ANCHOR;
+  bool ws_ok = ANCHOR || p.ws_free;
 
   for (int j = 0; j < nj; ++j) {
     const int t = warp + NW * j;
@@ -1180,6 +1182,7 @@ __global__ void __launch_bounds__(32 * NW, 1) k_score_tma(const __grid_constant_
   if (err) atomicOr(p.err, err);
   if (!ws_ok) pdl_wait();
   score_epilogue<GM, D, NW, C::THREADS>(p, b, g, s, wst, reinterpret_cast<const float*>(smem), GM * D, tail);
+  if (!ANCHOR && p.ws_free) pdl_wait();
 }
 
 // ---------------------------------------------------------------------------
@@ -1528,7 +1531,7 @@ __global__ void __launch_bounds__(kTcThreads, NS <= 3 ? 2 : 1) k_score_tc(const 
     // for it only before its first workspace write (visual logits, or the
     // split's partial), so splits of text tiles stream their whole range
     // meanwhile.
-    bool ws_ok = false;
+    bool ws_ok = p.ws_free;
     int j = 0;          // text tiles seen
     for (int i = 0; i < n; ++i) {
       const int u = tr.u0 + i, sb = i & 1;
@@ -1691,6 +1694,7 @@ __global__ void __launch_bounds__(kTcThreads, NS <= 3 ? 2 : 1) k_score_tc(const 
 #pragma unroll
     for (int h = 0; h < GM; ++h)
       if (h < G) p.split_o[(rec0 + (int64_t)h * p.nsp_max) * D + r] = o[h];
+    if (p.ws_free) pdl_wait();
     if (dead) timed_out = true;
   }
   if (timed_out) err |= ERR_TIMEOUT;
@@ -1888,7 +1892,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_score_f32(const __grid_constant
   const int s = blockIdx.x, g = blockIdx.y, b = blockIdx.z;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int l = lane % LPR, rs = lane / LPR;  // piece of the row, row slot of the warp
-  pdl_wait();
+  if (!p.ws_free) pdl_wait();
   const int G = p.G, H = p.H;
   const Seq sq = load_seq(p, b, s == 0 && g == 0);
   const float* qb = reinterpret_cast<const float*>(p.q) + ((int64_t)b * H + g * G) * D;
@@ -2052,6 +2056,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_score_f32(const __grid_constant
     if (rs == 0) *reinterpret_cast<float4*>(&sm.ow[warp][h][4 * l]) = acc[h];
   }
   score_epilogue<GM, D>(p, b, g, s, sm.wst, &sm.ow[0][0][0], GM * D, sm.tail);
+  if (p.ws_free) pdl_wait();
 }
 
 // ---------------------------------------------------------------------------
@@ -3178,10 +3183,11 @@ __global__ void __launch_bounds__(kMergeThreads) k_merge(const __grid_constant__
   constexpr int U = 10;                                 // splits of a group in flight
   __shared__ float4 acc_s[NG][LPR];
   __shared__ float2 st_s[NG];
-  // The next kernel is the next layer's score kernel, which waits for this one
-  // before it reads a kept set or writes the workspace: it may start now.
-  pdl_trigger();
+  // The next kernel is the next layer's score kernel: see WsLayout for when it
+  // may start.
+  if (!p.ws_free) pdl_trigger();
   pdl_wait();
+  if (p.ws_free) pdl_trigger();
   const int64_t row = (int64_t)blockIdx.y * p.H + blockIdx.x;
   const int sg = threadIdx.x / LPR, l = threadIdx.x % LPR, ns = p.ns;
   const float* st = p.split_st + row * p.nsp_max * ST_N;
@@ -3647,11 +3653,10 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
   const int d0 = GATHER ? (rank % rpg) * W : 0;
   const int64_t hrow0 = (int64_t)b * H + g * G;
   const int nsel = p.granularity ? p.Hkv : 1;
-  // Fused: the next kernel is the next call's score kernel, which reads only
-  // its inputs before its own wait, so it may start now.  Select only: the
-  // gather kernel reads the score partials before its wait, which this
-  // kernel's wait guarantees complete.
-  if constexpr (GATHER) pdl_trigger();
+  // Fused: the next kernel is the next call's score kernel, which with one set
+  // of outputs writes nothing before its own wait and may start now (with two:
+  // after this kernel's wait, see WsLayout).
+  if (GATHER && !p.ws_free) pdl_trigger();
   // While the score kernel finishes: the barrier that counts the keys in, the
   // histograms cleared, and the cluster's start (a CTA's shared memory may be
   // written once that CTA runs and its barrier is initialised; waited for here,
@@ -3674,8 +3679,10 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
   const float* stb = p.split_st + ((int64_t)b * H * p.nsp_max + l16) * ST_N;
   const float* st0 = stb + (int64_t)min(2 * warp + sub, H - 1) * p.nsp_max * ST_N;
   asm volatile("" : "+l"(st0));  // address in place before the wait
+  // Select only: the gather kernel reads the score partials before its wait,
+  // which this kernel's wait guarantees complete.
   pdl_wait();
-  if constexpr (!GATHER) pdl_trigger();
+  if (!GATHER || p.ws_free) pdl_trigger();
 
   // 1. Split statistics -> per-head max, normalisers and masses (Eq. 5,
   //    Eq. 6), and for this CTA's heads the text-only max and sum.  Sixteen

@@ -149,3 +149,68 @@ def test_anchor_gather_unsupported_configurations(vp):
             assert st == vp.VP_ERR_UNSUPPORTED, st
         finally:
             dev.close()
+
+
+@pytest.mark.parametrize("dtype", [W.BF16, W.FP32])
+def test_calls_in_turn_on_one_context(vp, dtype):
+    """Decode steps of different layers, and for bf16 gathers over their kept
+    sets between them, back to back on one small context (the score kernels'
+    outputs in two sets, used in turn): enqueued, and captured as three calls
+    in a graph replayed between enqueued ones, every output equals the call
+    run alone, bit for bit."""
+    r = small(layers=3, dtype=dtype, vis_len=(900, 577, 64), text_len=(517, 1070, 129))
+    devs = [Hn.Device(vp, Hn.make_inputs(r, i, t_cap=1700), r.budget, max_seq=1700) for i in range(3)]
+    ctx = devs[0].ctx
+
+    def new(d):
+        return [torch.full_like(d.out, float("nan")), torch.full_like(d.kept, -7), torch.full_like(d.count, -7),
+                torch.full_like(d.mass, float("nan")), torch.full_like(d.out, float("nan"))]
+
+    def call(d, o):
+        vp.vp_decode_step(ctx, d.B, d.q, d.kc, d.vc, d.span, d.tl, d.budget, o[0], o[1], d.kept_cap, o[2], o[3])
+
+    def gather(d, kept, count, o):
+        if dtype == W.BF16:
+            vp.vp_decode_gather(ctx, d.B, d.q, d.kc, d.vc, d.span, d.tl, kept, d.kept_cap, count, o[4])
+
+    def step(outs):
+        for i, d in enumerate(devs):
+            call(d, outs[i])
+            gather(devs[(i + 1) % 3], outs[i][1], outs[i][2], outs[i])
+
+    try:
+        want = []
+        for i, d in enumerate(devs):
+            o = new(d)
+            call(d, o)
+            torch.cuda.synchronize()
+            gather(devs[(i + 1) % 3], o[1], o[2], o)
+            torch.cuda.synchronize()
+            want.append([t.clone() for t in o])
+        runs = [[new(d) for d in devs] for _ in range(3)]
+        for outs in runs:
+            step(outs)
+        captured = [new(d) for d in devs]
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            for i, d in enumerate(devs):
+                call(d, captured[i])
+        mixed = [[new(d) for d in devs] for _ in range(2)]
+        graph.replay()
+        step(mixed[0])
+        graph.replay()
+        graph.replay()
+        step(mixed[1])
+        vp.vp_check_errors(ctx)
+        torch.cuda.synchronize()
+        for outs in runs + mixed:
+            for i in range(3):
+                for a, b in zip(outs[i], want[i]):
+                    assert torch.equal(a.view(torch.uint8), b.view(torch.uint8)), i
+        for i in range(3):
+            for a, b in zip(captured[i][:4], want[i][:4]):
+                assert torch.equal(a.view(torch.uint8), b.view(torch.uint8)), i
+    finally:
+        for d in devs:
+            d.close()
