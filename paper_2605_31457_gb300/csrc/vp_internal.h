@@ -38,14 +38,12 @@ struct KvView {
 };
 
 struct StepParams {
-  // bulk-tensor (TMA) descriptors of the K and V caches (bf16), when use_tma
+  // bulk-tensor (TMA) descriptors of the K and V caches (bf16), when use_tma:
+  // in boxes of up to 128 rows for the tensor-core score kernel (use_tc: decode
+  // step, bf16, D = 128, at most 16 query heads per kv-head), else of up to 32
   CUtensorMap tmk;  // 64-byte aligned type
   CUtensorMap tmv;
   int use_tma;
-  // the same caches in boxes of up to 128 rows, for the tensor-core score
-  // kernel (decode step, bf16, D = 128, at most 16 query heads per kv-head)
-  CUtensorMap tmk2;
-  CUtensorMap tmv2;
   int use_tc;
   int anchor;  // 1: a layer after the anchor layer -- text plus the given kept set, no selection
   int tpos, gpos, bpos;  // descriptor dimension (1..3) of the token, kv-head and sequence/page axes
@@ -337,8 +335,8 @@ cudaError_t configure_kernels(int max_visual, int H, int nsp_max);
 // Fills p.tmk / p.tmv / p.use_tma for a bf16 cache whose layout a 4-D tensor
 // descriptor can describe without reaching past the caller's memory; leaves
 // use_tma = 0 otherwise (the score kernel then copies rows one by one).
-// With p.use_tc set on entry (a plan made for the tensor-core kernel) it also
-// fills p.tmk2 / p.tmv2 and keeps use_tc only if that kernel can run.
+// With p.use_tc set on entry (a plan made for the tensor-core kernel) it keeps
+// use_tc only if that kernel can run, with descriptors for it.
 void encode_kv_maps(StepParams& p);
 // The tensor-core score kernel's shape conditions (decode step, bf16, D = 128,
 // at most 16 query heads per kv-head, pages of at least 8 rows).

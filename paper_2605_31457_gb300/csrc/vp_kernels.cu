@@ -1326,8 +1326,8 @@ __global__ void __launch_bounds__(kTcThreads, NS <= 3 ? 2 : 1) k_score_tc(const 
     }
     mbar_init(mma_done, 1);
     mbar_fence_init();
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&p.tmk2)) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&p.tmv2)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&p.tmk)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&p.tmv)) : "memory");
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 64;\n" ::"r"(smem_u32(tmem_slot))
@@ -1389,7 +1389,7 @@ __global__ void __launch_bounds__(kTcThreads, NS <= 3 ? 2 : 1) k_score_tc(const 
     __syncwarp();
     if (live) {
       auto crd = [&](int axis) { return axis == p.tpos ? row : axis == p.gpos ? g : base; };
-      tma_load_4d(smem_u32(smem + sl * C::SLOT) + hh * C::HALF + x * R * 128, part ? &p.tmv2 : &p.tmk2, 64 * hh,
+      tma_load_4d(smem_u32(smem + sl * C::SLOT) + hh * C::HALF + x * R * 128, part ? &p.tmv : &p.tmk, 64 * hh,
                   crd(1), crd(2), crd(3), full + sl);
     }
     ++qc;
@@ -4375,22 +4375,22 @@ void encode_kv_maps(StepParams& p) {
   p.use_tc = 0;
   if (p.dtype != 0 || (p.D != 64 && p.D != 128)) return;
   if (p.paged && p.page_size < 8) return;  // box origins must stay 1024-byte aligned in shared memory
-  const int R = p.paged ? (p.page_size < kTmaTile ? p.page_size : kTmaTile) : kTmaTile;
   int kt = 0, kg = 0, kb = 0, vt = 0, vg = 0, vb = 0;
-  if (!encode_one(p.k, p, &p.tmk, &kt, &kg, &kb, R) || !encode_one(p.v, p, &p.tmv, &vt, &vg, &vb, R)) return;
-  if (kt != vt || kg != vg || kb != vb) return;  // both caches must share an axis order
-  p.tpos = kt; p.gpos = kg; p.bpos = kb;
+  auto encode = [&](int rows) {
+    if (!encode_one(p.k, p, &p.tmk, &kt, &kg, &kb, rows) || !encode_one(p.v, p, &p.tmv, &vt, &vg, &vb, rows)) return false;
+    if (kt != vt || kg != vg || kb != vb) return false;  // both caches must share an axis order
+    p.tpos = kt; p.gpos = kg; p.bpos = kb;
+    return true;
+  };
   if (want_tc && tc_eligible(p.dtype, p.D, p.G, p.paged, p.page_size)) {
     // Page ids of a split's boxes are staged in shared memory: bound them.
     const int R2 = p.paged ? (p.page_size < kTcRows ? p.page_size : kTcRows) : kTcRows;
     const int64_t boxes = p.paged ? (int64_t)tc_max_split_tiles(p.max_seq, p.ns, p.split_w) * (kTcRows / R2) : 0;
-    if (boxes <= kTcMaxBoxes && encode_one(p.k, p, &p.tmk2, &kt, &kg, &kb, R2) &&
-        encode_one(p.v, p, &p.tmv2, &vt, &vg, &vb, R2) && kt == p.tpos && vt == p.tpos && kg == p.gpos &&
-        vg == p.gpos && kb == p.bpos && vb == p.bpos)
-      p.use_tc = 1;
-    p.use_tma = 1;
-    return;
+    if (boxes <= kTcMaxBoxes && encode(R2)) p.use_tc = p.use_tma = 1;
+    return;  // without the tensor-core kernel the caller plans for the others
   }
+  const int R = p.paged ? (p.page_size < kTmaTile ? p.page_size : kTmaTile) : kTmaTile;
+  if (!encode(R)) return;
   if (p.paged) {
     // Page ids of a CTA's boxes are staged in shared memory: bound them.
     const int64_t tiles = (p.max_seq + kTmaTile - 1) / kTmaTile;

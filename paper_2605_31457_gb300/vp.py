@@ -114,7 +114,20 @@ class VPError(RuntimeError):
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+def _stream(stream):
+    """Raw handle of a torch.cuda.Stream, of a raw handle, or (None) of torch's
+    current stream on the current device."""
+    if stream is None:
+        import torch
+        if not torch.cuda.is_initialized():
+            return torch.cuda.current_stream().cuda_stream
+        # torch.cuda.current_stream() builds a Stream object: 2.9 us a call
+        # against 0.3 us for the handle.
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return getattr(stream, "cuda_stream", stream)
 
 
 def _check(status, ctx):
@@ -137,15 +150,10 @@ def vp_decode_step(ctx, batch, q, k_cache: vp_kv, v_cache: vp_kv, visual_span: v
                    stream=None, check=True):
     """Enqueues one decode step.  Tensors are torch CUDA tensors; ``stream``
     is a torch.cuda.Stream or raw handle (default: torch's current stream)."""
-    if stream is None:
-        import torch
-        stream = torch.cuda.current_stream().cuda_stream
-    elif hasattr(stream, "cuda_stream"):
-        stream = stream.cuda_stream
     st = lib.vp_decode_step(ctx, int(batch), _ptr(q), ctypes.byref(k_cache), ctypes.byref(v_cache),
                             ctypes.byref(visual_span), _ptr(text_len), ctypes.byref(budget), _ptr(out),
                             _ptr(kept_idx), int(kept_cap), _ptr(kept_count), _ptr(mass),
-                            _ptr(mass_stats), ctypes.c_void_p(stream))
+                            _ptr(mass_stats), _stream(stream))
     return _check(st, ctx) if check else st
 
 
@@ -154,14 +162,9 @@ def vp_decode_gather(ctx, batch, q, k_cache: vp_kv, v_cache: vp_kv, visual_span:
     """Enqueues the attention of a layer after the anchor layer over every text
     token and the anchor's kept set (kept_idx / kept_count as vp_decode_step
     wrote them).  Tensors are torch CUDA tensors."""
-    if stream is None:
-        import torch
-        stream = torch.cuda.current_stream().cuda_stream
-    elif hasattr(stream, "cuda_stream"):
-        stream = stream.cuda_stream
     st = lib.vp_decode_gather(ctx, int(batch), _ptr(q), ctypes.byref(k_cache), ctypes.byref(v_cache),
                               ctypes.byref(visual_span), _ptr(text_len), _ptr(kept_idx), int(kept_cap),
-                              _ptr(kept_count), int(granularity), float(scale), _ptr(out), ctypes.c_void_p(stream))
+                              _ptr(kept_count), int(granularity), float(scale), _ptr(out), _stream(stream))
     return _check(st, ctx) if check else st
 
 
@@ -169,13 +172,8 @@ def vp_compact_kv(ctx, batch, src: vp_kv, dst: vp_kv, visual_span: vp_span, text
                   kept_count, stream=None, check=True):
     """Writes into ``dst`` (contiguous) the cache ``src`` with only the kept
     visual rows (FastV prefill pruning followed by VisionPulse)."""
-    if stream is None:
-        import torch
-        stream = torch.cuda.current_stream().cuda_stream
-    elif hasattr(stream, "cuda_stream"):
-        stream = stream.cuda_stream
     st = lib.vp_compact_kv(ctx, int(batch), ctypes.byref(src), ctypes.byref(dst), ctypes.byref(visual_span),
-                           _ptr(text_len), _ptr(kept_idx), int(kept_cap), _ptr(kept_count), ctypes.c_void_p(stream))
+                           _ptr(text_len), _ptr(kept_idx), int(kept_cap), _ptr(kept_count), _stream(stream))
     return _check(st, ctx) if check else st
 
 
@@ -209,12 +207,7 @@ def vp_last_error(ctx) -> str:
 
 
 def vp_check_errors(ctx, stream=None, check=True):
-    if stream is None:
-        import torch
-        stream = torch.cuda.current_stream().cuda_stream
-    elif hasattr(stream, "cuda_stream"):
-        stream = stream.cuda_stream
-    st = lib.vp_check_errors(ctx, ctypes.c_void_p(stream))
+    st = lib.vp_check_errors(ctx, _stream(stream))
     return _check(st, ctx) if check else st
 
 
@@ -240,15 +233,10 @@ def vp_decode_step_noalloc(cfg: vp_config, batch, q, k_cache: vp_kv, v_cache: vp
     """The decode step without a context or any device allocation (scratch in
     the library's fixed device array).  For callers that cannot allocate on
     their inference path.  Returns the raw vp_status (0 = VP_OK)."""
-    if stream is None:
-        import torch
-        stream = torch.cuda.current_stream().cuda_stream
-    elif hasattr(stream, "cuda_stream"):
-        stream = stream.cuda_stream
     return lib.vp_decode_step_noalloc(ctypes.byref(cfg), int(batch), _ptr(q), ctypes.byref(k_cache),
                                       ctypes.byref(v_cache), ctypes.byref(visual_span), _ptr(text_len),
                                       ctypes.byref(budget), _ptr(out), _ptr(kept_idx), int(kept_cap),
-                                      _ptr(kept_count), _ptr(mass), _ptr(mass_stats), ctypes.c_void_p(stream))
+                                      _ptr(kept_count), _ptr(mass), _ptr(mass_stats), _stream(stream))
 
 
 # ------------------------------------------------------- marshalling helpers
