@@ -51,6 +51,10 @@ constexpr int64_t kPpm = 1000000;
 constexpr int kMaxVisual = 32768;  // score keys of one sequence fit in shared memory
 constexpr int kMaxHeads = 128;
 constexpr int kMaxGroup = 16;
+// Splits of a layer after the anchor layer, at most: the merge kernel's groups
+// take up to eight each in one round trip (B = 1 decode, 27 such layers: 37
+// splits 234 us, 32 230, 24 241).
+constexpr int kGatherSplits = 32;
 
 vp_status fail(vp_ctx* ctx, vp_status st, const std::string& msg) {
   if (ctx) ctx->last_error = msg;
@@ -277,7 +281,7 @@ vp_status vp_decode_step(vp_ctx* ctx, int32_t batch, const void* q,
   p.hp = ctx->lay.hp;
   p.nsp_max = ctx->lay.nsp_max;
   p.nk_max = ctx->lay.nk_max;
-  if (!vp::plan_step(p, ctx->num_sms, kept_cap, budget->granularity, ctx->score_path))
+  if (!vp::plan_step(p, ctx->num_sms, kept_cap, budget->granularity, ctx->score_path, ctx->lay.o_set2 != 0))
     return fail(ctx, VP_ERR_UNSUPPORTED, "vp_decode_step: the tcgen05 score kernel (VP_SCORE_TC) cannot serve this "
                 "call (needs bf16, head_dim 128, G <= 16, pages of >= 8 tokens, a tensor-descriptor layout)");
   p.mt_o = ctx->mt_o; p.mt_st = ctx->mt_st; p.hmax = ctx->hmax;
@@ -371,7 +375,8 @@ vp_status vp_decode_gather(vp_ctx* ctx, int32_t batch, const void* q,
   p.mt_o = ctx->mt_o; p.mt_st = ctx->mt_st; p.hmax = ctx->hmax;
   // Score splits as planned for the decode step; their weight covers the
   // cache outside the visual span plus the kept rows.
-  const vp::Plan pl = vp::make_plan(batch, Hkv, D, ctx->num_sms, c.max_visual, c.max_seq, 0, granularity);
+  vp::Plan pl = vp::make_plan(batch, Hkv, D, ctx->num_sms, c.max_visual, c.max_seq, 0, granularity);
+  pl.ns = std::min(pl.ns, kGatherSplits);
   p.hp = ctx->lay.hp;
   p.ns = pl.ns; p.nsp_max = ctx->lay.nsp_max; p.cl = 1;
   {

@@ -171,8 +171,17 @@ struct Plan {
 };
 
 // tc: the score splits are for the tensor-core kernel (128-row tiles).
+// beside: the score kernel runs beside the previous call's select kernel (a
+// context with two sets of its outputs).  It then has that kernel's time to
+// itself, on the other SMs, while every split lengthens the select kernel's
+// merges: at most kBesideSplits splits, or as many as keep kBesideTiles tiles a
+// CTA, on the SMs the select clusters leave.  Measured, B = 1, 28/4 heads,
+// 3857 tokens, 28 calls in a graph: 37 splits 344 us, 32 337, 24 308, 20 312,
+// 16 303, 12 312; 4 fp32 sequences of up to 2796 tokens (32 select CTAs): 19
+// splits 22.9 us a call, 16 22.8, 15 (one wave beside them) 14.9.
+constexpr int kBesideSplits = 16, kBesideTiles = 18;
 inline Plan make_plan(int batch, int Hkv, int D, int num_sms, int max_visual, int max_seq, int kept_cap,
-                      int granularity, bool tc = false) {
+                      int granularity, bool tc = false, bool beside = false) {
   const long long units = (long long)batch * Hkv;
   const int TR = tc ? kTcRows : 32;
   // Fixed-weight splits sized for the longest sequence (tiles wholly inside
@@ -186,7 +195,11 @@ inline Plan make_plan(int batch, int Hkv, int D, int num_sms, int max_visual, in
   // the visual span counted once more).  Score CTAs are small enough that
   // two fit on an SM.
   const long long tiles = tc ? w_max : (max_visual + 31) / 32 + 2LL * ((max_seq + 31) / 32);
+  const long long sel = (long long)batch * (granularity ? Hkv : 1);
+  int cl = 1;
+  while (cl < 8 && sel * cl * 2 <= num_sms) cl *= 2;
   const long long slots = 2LL * num_sms;
+  const long long score_slots = beside && sel * cl <= num_sms / 2 ? slots - 2 * sel * cl : slots;
   // Split count: minimise (waves of CTAs) x (tiles per CTA + a fixed cost per
   // CTA for its start, its pipeline fill and its partial), keeping a minimum
   // of work per CTA; the smaller count wins a tie.  The costs were measured
@@ -194,18 +207,21 @@ inline Plan make_plan(int batch, int Hkv, int D, int num_sms, int max_visual, in
   // kernel, about 6 weight units of 128 rows for the tensor-core kernel.
   long long ns_hi = tiles / (tc ? 2 * kTcWv : 8);
   if (ns_hi > kNsMax) ns_hi = kNsMax;
+  if (beside) {
+    const long long units_per = tc ? 2 * kTcWv * kBesideTiles / 8 : kBesideTiles;  // as 8 tiles to 2 K-only ones above
+    const long long least = (tiles + units_per - 1) / units_per;
+    const long long cap = least > kBesideSplits ? least : kBesideSplits;
+    if (ns_hi > cap) ns_hi = cap;
+  }
   if (ns_hi < 1) ns_hi = 1;
   const double fixed = tc ? 6.0 * kTcWv : 12.0;
   long long ns = 1;
   double best = 0.0;
   for (long long c = 1; c <= ns_hi; ++c) {
-    const double waves = (double)((units * c + slots - 1) / slots);
+    const double waves = (double)((units * c + score_slots - 1) / score_slots);
     const double cost = waves * ((double)tiles / (double)c + fixed);
     if (c == 1 || cost < best * (1.0 - 1e-9)) { best = cost; ns = c; }
   }
-  const long long sel = (long long)batch * (granularity ? Hkv : 1);
-  int cl = 1;
-  while (cl < 8 && sel * cl * 2 <= num_sms) cl *= 2;
   // Kept chunks of about 2048 rows, smaller (down to 256) while the gather
   // grid would not fill the GPU once (measured against 1024-row chunks and a
   // twice-filled grid: the chunk gather 5% to 22% faster across the sweep).
@@ -255,15 +271,18 @@ inline int split_floor(const Plan& pl, int batch, int Hkv, int num_sms, bool tc,
 // n - 1 lets it start only after that kernel's own wait, so the score kernel of
 // call n - 1 is complete, and every score kernel waits, before it ends, for the
 // last kernel of the call before it, here that of call n - 2.
-// Contexts whose calls span at most kSet2Cache bytes of cache use two sets:
-// their score kernel is shorter than the select kernel it then overlaps (B = 1,
-// 28 calls in a graph: 15.0 -> 12.1 us a call).  Larger calls keep one set and
-// the early start of the next score kernel, whose text tiles fill the drain of
-// the current one (8 sequences of 4096 + 16384 tokens: 51.8 us, two sets 55.4;
-// top-p on 16 of 6400 + 1024: 83.4 against 85.8).
-constexpr size_t kSet2Cache = (size_t)64 << 20;
+// Contexts whose calls span at most kSet2Cache bytes of cache (fp32:
+// kSet2CacheF32, its score kernel fills the SMs' registers) use two sets: score
+// and select kernel then take turns on fewer SMs each (see make_plan's
+// `beside`).  Measured, one set against two, us a call back to back: 28/4 heads,
+// B = 1 of 3857 tokens 15.0 / 10.9; 4 x 8192 29.6 / 19.7; 2 x 17296 25.2 / 18.3;
+// 16 x 3857 37.7 / 31.1; 6 x 20480 (252 MB) 46.5 / 39.9; fp32, 4 x 2796 (47 MB)
+// 23.4 / 14.9, 8 x 2796 35.1 / 38.2.  Larger calls are bound by HBM: they keep
+// one set and the early start of the next score kernel, whose text tiles fill
+// the drain of the current one (8 x 20480 51.5 / 55.2).
+constexpr size_t kSet2Cache = (size_t)256 << 20, kSet2CacheF32 = (size_t)64 << 20;
 inline bool two_sets(int batch, int Hkv, int D, int max_seq, int esz) {
-  return (size_t)batch * Hkv * max_seq * D * esz * 2 <= kSet2Cache;
+  return (size_t)batch * Hkv * max_seq * D * esz * 2 <= (esz == 2 ? kSet2Cache : kSet2CacheF32);
 }
 struct WsLayout {
   size_t o_tickets, o_err, zero_bytes, o_z, o_st, o_o, o_go, o_gs, o_mo, o_ms, o_hm, total;
@@ -390,7 +409,7 @@ inline int select_kind(const StepParams& p, int kept_cap) {
 // kernel was faster, above both the tensor-core kernel).
 // path: 0 the choice above, 1 never the tensor-core kernel, 2 only it
 // (false when it cannot serve the call).
-inline bool plan_step(StepParams& p, int num_sms, int kept_cap, int granularity, int path = 0) {
+inline bool plan_step(StepParams& p, int num_sms, int kept_cap, int granularity, int path = 0, bool beside = false) {
   p.num_sms = num_sms;
   const long long w_tc = 2LL * ((p.max_seq + kTcRows - 1) / kTcRows) - p.max_visual / kTcRows;
   const bool eligible = tc_eligible(p.dtype, p.D, p.G, p.paged, p.page_size);
@@ -399,7 +418,7 @@ inline bool plan_step(StepParams& p, int num_sms, int kept_cap, int granularity,
   if (path == 2 && !tc) return false;
   for (int pass = 0; pass < 2; ++pass) {
     const bool want = tc && pass == 0;
-    const Plan pl = make_plan(p.B, p.Hkv, p.D, num_sms, p.max_visual, p.max_seq, kept_cap, granularity, want);
+    const Plan pl = make_plan(p.B, p.Hkv, p.D, num_sms, p.max_visual, p.max_seq, kept_cap, granularity, want, beside);
     p.ns = pl.ns; p.cl = pl.cl; p.nk = pl.nk; p.nm = pl.nm; p.nc = pl.nc; p.gslice = pl.gslice;
     p.split_w = split_floor(pl, p.B, p.Hkv, num_sms, want, pl.split_w);
     p.use_tc = want ? 1 : 0;
