@@ -2126,12 +2126,15 @@ struct RadixCut {
 // ppm / 10^6 of all n scores.  A radix select over score mass, 4 bits a pass
 // from the top: every thread adds the candidates it owns to its own column of
 // col[16][NTH] (plain loads and stores, one bank per lane), warp d sums digit
-// d's row, and every thread takes the digit in which the mass is reached.
-// Bound by latency: eight passes of two barriers each.  The digit sums were
-// shared float atomics before, which retry while lanes meet on one address,
-// and scores fall into few digits: N_v = 6400, 16 sequences, 32 heads, the whole
-// call took 187 us (131 us of it this kernel), now 89 us.  The columns also make the sums (and with
-// them K_t) the same on every run.
+// d's row, and every thread takes the digit in which the mass is reached.  Once
+// at most 32 candidates are left (after three passes, usually), one warp takes
+// them in descending order.  Bound by latency: a pass is two barriers and a
+// walk over the keys.  The digit sums were shared float atomics before, which
+// retry while lanes meet on one address, and scores fall into few digits: 16
+// sequences of N_v = 6400, 32 heads, this kernel 131 us, with the columns 32,
+// and 22 with the list and with logit rows shared by a warp's lanes also in
+// the 512-thread form (the call 187, 83 and 73 us).  The columns also make the
+// sums (and with them K_t) the same on every run.
 // wsum: 32 floats, wcnt: 2 x NTH / 32 ints.  Returns K (before the capacity
 // clamp); theta, krem and n_theta as in RadixCut (unset when K >= n).
 constexpr int kTopPDigits = 16;
@@ -2146,6 +2149,55 @@ __device__ __forceinline__ int top_p_cut(const uint32_t* key_s, int n, int ppm, 
   uint32_t prefix = 0, mask = 0;
   float need = 0.f;  // score mass still to cover
   for (int shift = 28; shift >= 0; shift -= 4) {
+    if (shift == 16 || shift == 8) {
+      // Few candidates left (usual after three passes): list them, and one
+      // warp takes them in descending order until they reach the mass.
+      unsigned* n_list = reinterpret_cast<unsigned*>(wcnt);  // read after the passes only
+      uint32_t* list = reinterpret_cast<uint32_t*>(col);     // every digit sum is read
+      if (tid == 0) *n_list = 0;
+      __syncthreads();
+      for (int i = tid; i < n; i += NTH) {
+        const uint32_t k = key_s[i];
+        if ((k & mask) == prefix) {
+          const unsigned pos = atomicAdd(n_list, 1u);
+          if (pos < 32) list[pos] = k;
+        }
+      }
+      __syncthreads();
+      const unsigned nl = *n_list;
+      if (nl <= 32) {
+        if (warp == 0) {
+          const uint32_t mine = lane < (int)nl ? list[lane] : 0u;
+          int rank = 0;  // place in descending order, equal keys in list order
+          for (int i = 0; i < (int)nl; ++i) {
+            const uint32_t o = __shfl_sync(0xffffffffu, mine, i);
+            rank += o > mine || (o == mine && i < lane);
+          }
+          __syncwarp();
+          if (lane < (int)nl) list[rank] = mine;
+          __syncwarp();
+          const uint32_t key = lane < (int)nl ? list[lane] : 0u;
+          float sum = __uint_as_float(key);
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const float x = __shfl_up_sync(0xffffffffu, sum, o);
+            if (lane >= o) sum += x;
+          }
+          // The first that reaches the mass; the last when rounding falls short.
+          const unsigned hit = __ballot_sync(0xffffffffu, lane < (int)nl && sum >= need);
+          const int at = hit ? __ffs(hit) - 1 : (int)nl - 1;
+          const uint32_t cut = __shfl_sync(0xffffffffu, key, at);
+          float above = key > cut ? __uint_as_float(key) : 0.f;
+          above = warp_sum(above);
+          if (lane == 0) { wsum[0] = __uint_as_float(cut); wsum[1] = need - above; }
+        }
+        __syncthreads();
+        prefix = __float_as_uint(wsum[0]);
+        need = wsum[1];
+        __syncthreads();  // wcnt and col are free again
+        break;
+      }
+    }
 #pragma unroll
     for (int d = 0; d < kTopPDigits; ++d) col[d * NTH + tid] = 0.f;
     for (int i = tid; i < n; i += NTH) {
@@ -2252,28 +2304,14 @@ __global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepPara
   fetch(warp, lane, cx0, cy0);
   fetch(warp, lane + 32, cx1, cy1);
   const int nv = sq.nv;
-  // This rank's slice of the visual tokens; its first logit row is requested
-  // now so that it arrives while the statistics are merged (heads up to 32;
-  // at 1024 threads the registers are too few for it).
-  // Slices of whole 32-token words, so that a warp owns its activity words.
+  // This rank's slice of the visual tokens, in whole 32-token words, so that a warp owns its activity words.
   const int per = ((nv + ncl - 1) / ncl + 31) & ~31;
   const int i0 = min(nv, rank * per), i1 = min(nv, i0 + per);
   const int hbeg = p.granularity ? gsel * p.G : 0;
   const int hcnt = p.granularity ? p.G : H;
   const bool vec = (hbeg & 3) == 0 && (hcnt & 3) == 0;
-  // Long slices (the 1024-thread form, slices above kSelSliceSmall) take the
-  // row-shared importance loop below; short ones (the B = 1 decode) request
-  // each thread's first row now.  The 512-thread form is compiled without the
-  // row-shared loop: its launches are latency-bound, and the larger code
-  // measured slower there.
-  const bool wide = NTH >= 1024 && vec && hcnt >= 4 && hcnt <= 32 && (i1 - i0) > 2 * NTH;
-  const bool pre = !wide && NTH <= 512 && vec && hcnt <= 32 && i0 + tid < i1;
-  float4 zpre[8];
-  if (pre) {
-    const float4* zr = reinterpret_cast<const float4*>(p.z_ws + ((int64_t)b * p.max_visual + i0 + tid) * p.hp + hbeg);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) zpre[q] = 4 * q < hcnt ? __ldcg(zr + q) : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
+  // Logit rows on 16-byte boundaries take the row-shared importance loop below.
+  const bool wide = vec && hcnt >= 4 && hcnt <= 32;
   for (int h = warp; h < H; h += NW) {
     float4 nx0, ny0, nx1, ny1;
     fetch(h + NW, lane, nx0, ny0);
@@ -2424,47 +2462,20 @@ __global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepPara
       }
     }
   };
-  bool done = false;
-  if constexpr (NTH >= 1024) {
-    if (wide) {
-      const int Q = hcnt / 4;
-      if (Q <= 1) wide_loop(std::integral_constant<int, 1>{});
-      else if (Q <= 2) wide_loop(std::integral_constant<int, 2>{});
-      else if (Q <= 4) wide_loop(std::integral_constant<int, 4>{});
-      else wide_loop(std::integral_constant<int, 8>{});
-      done = true;
-    }
-  }
-  if (!done) {
+  if (wide) {
+    const int Q = hcnt / 4;
+    if (Q <= 1) wide_loop(std::integral_constant<int, 1>{});
+    else if (Q <= 2) wide_loop(std::integral_constant<int, 2>{});
+    else if (Q <= 4) wide_loop(std::integral_constant<int, 4>{});
+    else wide_loop(std::integral_constant<int, 8>{});
+  } else {
     for (int wb = i0 + 32 * warp; wb < i1; wb += NTH) {  // one word of tokens per warp
       const int i = wb + lane;
       const float* zr = p.z_ws + ((int64_t)b * p.max_visual + i) * p.hp + hbeg;
       float a = 0.f;
-      if (i >= i1) {
-      } else if (pre && i == i0 + tid) {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          if (4 * q < hcnt) {
-            const int h = hbeg + 4 * q;
-            a = fmaf(fexp2_rel(zpre[q].x, hM_s[h]), hInv_s[h], a);
-            a = fmaf(fexp2_rel(zpre[q].y, hM_s[h + 1]), hInv_s[h + 1], a);
-            a = fmaf(fexp2_rel(zpre[q].z, hM_s[h + 2]), hInv_s[h + 2], a);
-            a = fmaf(fexp2_rel(zpre[q].w, hM_s[h + 3]), hInv_s[h + 3], a);
-          }
-        }
-      } else if (vec) {
-        for (int hh = 0; hh < hcnt; hh += 4) {
-          const float4 z4 = __ldcg(reinterpret_cast<const float4*>(zr + hh));
-          const int h = hbeg + hh;
-          a = fmaf(fexp2_rel(z4.x, hM_s[h]), hInv_s[h], a);
-          a = fmaf(fexp2_rel(z4.y, hM_s[h + 1]), hInv_s[h + 1], a);
-          a = fmaf(fexp2_rel(z4.z, hM_s[h + 2]), hInv_s[h + 2], a);
-          a = fmaf(fexp2_rel(z4.w, hM_s[h + 3]), hInv_s[h + 3], a);
-        }
-      } else {
+      if (i < i1)
         for (int hh = 0; hh < hcnt; ++hh)
           a = fmaf(fexp2_rel(__ldcg(zr + hh), hM_s[hbeg + hh]), hInv_s[hbeg + hh], a);
-      }
       const bool on = i < i1 && emit(i, a);
       if (act_row) {
         const unsigned m = __ballot_sync(0xffffffffu, on);
