@@ -3466,6 +3466,10 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather_slice(const __grid_co
 //      cluster; one launch and one dependency replace two, and only the
 //      selection itself lies between the score kernel and the kept rows'
 //      loads.
+// Every instruction runs about once per launch, so the code is kept short: the
+// unroll depths (three logit rows, two records, four text partials in flight)
+// were swept on the fused form; 8, 4 and 10 cost the B = 1 step of 28 calls
+// 305 us, these 276 to 282 (2 or 4 rows 285 and 291, one record 296).
 // Bound by latency: the records, the exchange of the keys, the cut and the
 // kept rows follow one another, each at the cost of its slowest warp's
 // instructions and one trip to L2, HBM or a neighbour's shared memory.  B = 1,
@@ -3627,7 +3631,7 @@ struct SgSmem {
   float fin[GM][2];              // kept max, kept sum
 };
 
-constexpr int kSgTextSplits = 10;  // text split partials a thread requests ahead
+constexpr int kSgTextSplits = 4;  // text split partials a thread requests ahead
 
 // Byte offset of 16-byte piece c of row j in a stage of 128-byte rows, the
 // pieces XOR-swizzled by the row so that ldmatrix reads hit distinct banks.
@@ -3698,12 +3702,13 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
   // 1. Split statistics -> per-head max, normalisers and masses (Eq. 5,
   //    Eq. 6), and for this CTA's heads the text-only max and sum.  Sixteen
   //    lanes per head (two heads per warp); lane l16 folds splits l16,
-  //    l16 + 16, ..., four records requested at a time (one round trip for
-  //    up to 64 splits).  The first round's records are requested before
+  //    l16 + 16, ..., MR records requested at a time (one round trip for
+  //    up to 16 MR splits).  The first round's records are requested before
   //    anything else: they are on the critical path.
-  auto fetch4 = [&](const float* st, int s0, bool live, float4 (&x)[4], float4 (&y)[4]) {  // s0: first split of the round
+  constexpr int MR = GATHER ? 2 : 1;
+  auto fetch4 = [&](const float* st, int s0, bool live, float4 (&x)[MR], float4 (&y)[MR]) {  // s0: first split of the round
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < MR; ++k) {
       if (k > 0 && s0 + 16 * k >= ns) break;  // uniform
       const int s = s0 + 16 * k;
       if (live && s + l16 < ns) {
@@ -3715,7 +3720,7 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
       }
     }
   };
-  float4 rx[4], ry[4];
+  float4 rx[MR], ry[MR];
   fetch4(st0, 0, 2 * warp + sub < H, rx, ry);
 
   // This CTA's slice of the visual tokens.  A group of 2^rsh lanes shares a
@@ -3723,7 +3728,7 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
   // end on 16-byte boundaries), so that loads cover whole rows and all warps
   // share the exponentials.  The first kZPre rounds of rows are requested next,
   // so that they arrive while the statistics are merged.
-  constexpr int kZPre = 8;
+  constexpr int kZPre = GATHER ? 3 : 8;
   const int per = (nv + ncl - 1) / ncl;
   const int i0 = min(nv, rank * per), i1 = min(nv, i0 + per);
   const int hbeg = p.granularity ? gsel * G : 0;
@@ -3754,11 +3759,11 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
     if (h0 != 2 * warp) fetch4(sth, 0, h < H, rx, ry);  // the first round's records are in flight already
     float m = -CUDART_INF_F, a1v = 0.f, atv = 0.f, a1t = 0.f, att = 0.f;
     float mt = -CUDART_INF_F, lt = 0.f;  // text only
-    for (int s0 = 0;; s0 += 64) {
+    for (int s0 = 0;; s0 += 16 * MR) {
       if (s0) fetch4(sth, s0, h < H, rx, ry);
       float mn = m, mtn = mt;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
+      for (int k = 0; k < MR; ++k) {
         if (k > 0 && s0 + 16 * k >= ns) break;  // uniform
         mn = fmaxf(mn, fmaxf(rx[k].x, ry[k].x));
         mtn = fmaxf(mtn, rx[k].x);
@@ -3771,7 +3776,7 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
       m = mn;
       mt = mtn;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
+      for (int k = 0; k < MR; ++k) {
         if (k > 0 && s0 + 16 * k >= ns) break;  // uniform
         a1v = fmaf(exp2_rel(ry[k].x, m), ry[k].y, a1v);
         atv = fmaf(exp2_tau(ry[k].x, m, inv_tau), ry[k].z, atv);
@@ -3779,7 +3784,7 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
         att = fmaf(exp2_tau(rx[k].x, m, inv_tau), rx[k].z, att);
         lt = fmaf(exp2_rel(rx[k].x, mt), rx[k].y, lt);
       }
-      if (s0 + 64 >= ns) break;
+      if (s0 + 16 * MR >= ns) break;
     }
     float M = m, Mt = mt;
 #pragma unroll
@@ -3877,10 +3882,17 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
         for (int r = zq; r < (GATHER ? ncl : 1); r += lpt) st_async_u32(key_a + 4 * i, key, bar_a, r);
       }
     };
+#pragma unroll 1
+    for (int r = 0; i0 + r * zstep < i1; r += kZPre) {
+      if (r > 0) {
 #pragma unroll
-    for (int q = 0; q < kZPre; ++q)
-      if (i0 + q * zstep < i1) score(zi0 + q * zstep, zpre[q]);  // uniform
-    for (int q = kZPre; i0 + q * zstep < i1; ++q) score(zi0 + q * zstep, zload(zi0 + q * zstep));
+        for (int q = 0; q < kZPre; ++q)
+          if (i0 + (r + q) * zstep < i1) zpre[q] = zload(zi0 + (r + q) * zstep);  // uniform
+      }
+#pragma unroll
+      for (int q = 0; q < kZPre; ++q)
+        if (i0 + (r + q) * zstep < i1) score(zi0 + (r + q) * zstep, zpre[q]);  // uniform
+    }
   }
   if (bad) atomicOr(p.err, ERR_NONFINITE);
 
