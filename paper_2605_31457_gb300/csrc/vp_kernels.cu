@@ -2925,8 +2925,9 @@ struct GmCfg {
   static constexpr size_t smem(bool paged) { return (size_t)OFF_ENT + kGmMaxChunk * (paged ? 8 : 4); }
 };
 
-template <int D, int NT, int NW, bool PAGED>
-__global__ void __launch_bounds__(32 * NW, (NT == 1 ? 20 : 12) / NW) k_gather_mma(const __grid_constant__ StepParams p) {
+// MB: CTAs per SM.
+template <int D, int NT, int NW, int MB, bool PAGED>
+__global__ void __launch_bounds__(32 * NW, MB) k_gather_mma(const __grid_constant__ StepParams p) {
   using C = GmCfg<D, NT, NW>;
   constexpr int GM = C::GM;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -4164,9 +4165,9 @@ template <int GM>
 size_t slice_smem() { return sizeof(SliceSmem<GM>); }
 
 constexpr int kGmWide = 512;
-template <int D, int NT, int NW>
+template <int D, int NT, int NW, int MB>
 cudaError_t launch_gather_mma(const StepParams& p, dim3 grid, cudaStream_t st) {
-  return launch_ex(p.paged ? k_gather_mma<D, NT, NW, true> : k_gather_mma<D, NT, NW, false>, grid, dim3(32 * NW),
+  return launch_ex(p.paged ? k_gather_mma<D, NT, NW, MB, true> : k_gather_mma<D, NT, NW, MB, false>, grid, dim3(32 * NW),
                    GmCfg<D, NT, NW>::smem(p.paged), st, 1, p);
 }
 
@@ -4187,9 +4188,16 @@ cudaError_t launch_gather_td(const StepParams& p, cudaStream_t st) {
     // though the gather alone takes 43 against 42 us).  Chunked lists run
     // several waves (8192 of 16384: 212 us with four warps, 230 with eight),
     // short ones one or two steps per warp (29 of 576: 6.1 against 9.2 us).
-    if (p.nk == 1 && p.kept_cap >= kGmWide)
-      return p.G <= 8 ? launch_gather_mma<D, 1, 8>(p, grid, st) : launch_gather_mma<D, 2, 8>(p, grid, st);
-    return p.G <= 8 ? launch_gather_mma<D, 1, 4>(p, grid, st) : launch_gather_mma<D, 2, 4>(p, grid, st);
+    // Three CTAs per SM (fewer registers) where that saves a wave (40 sequences,
+    // 1250 of 5000: 144 us, two per SM 153; 1280 of 6400 runs two waves either
+    // way: 227 us, three per SM 242).
+    if (p.nk == 1 && p.kept_cap >= kGmWide) {
+      const long long n = (long long)p.nc * p.Hkv * p.B, two = 2LL * p.num_sms, three = 3LL * p.num_sms;
+      if (p.G > 8) return launch_gather_mma<D, 2, 8, 1>(p, grid, st);
+      return (n + three - 1) / three < (n + two - 1) / two ? launch_gather_mma<D, 1, 8, 3>(p, grid, st)
+                                                           : launch_gather_mma<D, 1, 8, 2>(p, grid, st);
+    }
+    return p.G <= 8 ? launch_gather_mma<D, 1, 4, 5>(p, grid, st) : launch_gather_mma<D, 2, 4, 3>(p, grid, st);
   }
   if (p.G <= 4) return launch_ex(k_gather<T, D, 4>, grid, dim3(kGatherThreads), gather_smem<T, D, 4>(), st, 1, p);
   if (p.G <= 8) return launch_ex(k_gather<T, D, 8>, grid, dim3(kGatherThreads), gather_smem<T, D, 8>(), st, 1, p);
@@ -4206,15 +4214,19 @@ cudaError_t configure_fixed_kernels() {
 #define VP_SET(kernel, bytes) if (e == cudaSuccess) e = set_smem(kernel, bytes)
   VP_SET((k_score_tc<8>), (TcCfg::SMEM));
   VP_SET((k_score_tc<16>), (TcCfg::SMEM));
-#define VP_SET_GM(D, NT)                                                          \
-  VP_SET((k_gather_mma<D, NT, 4, false>), (GmCfg<D, NT, 4>::smem(false)));          \
-  VP_SET((k_gather_mma<D, NT, 4, true>), (GmCfg<D, NT, 4>::smem(true)));            \
-  VP_SET((k_gather_mma<D, NT, 8, false>), (GmCfg<D, NT, 8>::smem(false)));          \
-  VP_SET((k_gather_mma<D, NT, 8, true>), (GmCfg<D, NT, 8>::smem(true)))
-  VP_SET_GM(128, 1);
-  VP_SET_GM(128, 2);
-  VP_SET_GM(64, 1);
-  VP_SET_GM(64, 2);
+#define VP_SET_GM(D, NT, NW, MB)                                                            \
+  VP_SET((k_gather_mma<D, NT, NW, MB, false>), (GmCfg<D, NT, NW>::smem(false)));            \
+  VP_SET((k_gather_mma<D, NT, NW, MB, true>), (GmCfg<D, NT, NW>::smem(true)))
+  VP_SET_GM(128, 1, 4, 5);
+  VP_SET_GM(128, 1, 8, 2);
+  VP_SET_GM(128, 1, 8, 3);
+  VP_SET_GM(128, 2, 4, 3);
+  VP_SET_GM(128, 2, 8, 1);
+  VP_SET_GM(64, 1, 4, 5);
+  VP_SET_GM(64, 1, 8, 2);
+  VP_SET_GM(64, 1, 8, 3);
+  VP_SET_GM(64, 2, 4, 3);
+  VP_SET_GM(64, 2, 8, 1);
 #undef VP_SET_GM
   VP_SET((k_score_tma<128, 1, kTmaWarps, tma_slots<128>(), false>), (tma_smem<128, 1>()));
   VP_SET((k_score_tma<128, 2, kTmaWarps, tma_slots<128>(), false>), (tma_smem<128, 2>()));

@@ -148,13 +148,15 @@ def test_kept_row_steps(vp, H, Hkv, D, paged, k):
 @pytest.mark.parametrize("paged", [False, True])
 def test_chunk_gather_long_lists(vp, paged):
     """One CTA per (sequence, kv-head) with a list of more than 512 rows (the
-    eight-warp form), ragged spans."""
-    vis = tuple(640 + 3 * i for i in range(40))
-    r = small(heads=16, kv_heads=8, head_dim=64, batch=40, vis_len=vis, vis_start=(1,) * 40, text_len=(20,) * 40,
-              paged=paged, page_size=16)
-    inp = Hn.make_inputs(r)
-    budget = dict(mode=O.FIXED_RATIO, tau=0.1, ratio_ppm=850_000)
-    Hn.check_all(vp, inp, budget, seqs=(0, 7, 39))
+    eight-warp forms: 320 CTAs fill one wave at three per SM, 480 take two
+    either way), ragged spans."""
+    for batch in (40, 60):
+        vis = tuple(640 + 3 * i for i in range(batch))
+        r = small(heads=16, kv_heads=8, head_dim=64, batch=batch, vis_len=vis, vis_start=(1,) * batch,
+                  text_len=(20,) * batch, paged=paged, page_size=16)
+        inp = Hn.make_inputs(r)
+        budget = dict(mode=O.FIXED_RATIO, tau=0.1, ratio_ppm=850_000)
+        Hn.check_all(vp, inp, budget, seqs=(0, 7, batch - 1))
 
 
 @pytest.mark.parametrize("H,Hkv,batch,gran", [(28, 4, 1, 0), (14, 2, 3, 0), (8, 2, 5, 1), (28, 4, 20, 1), (28, 4, 80, 0),
