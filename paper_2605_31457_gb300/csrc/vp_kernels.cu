@@ -4164,7 +4164,7 @@ cudaError_t launch_score_d(const StepParams& p, cudaStream_t st) {
 template <int GM>
 size_t slice_smem() { return sizeof(SliceSmem<GM>); }
 
-constexpr int kGmWide = 512;
+constexpr int kGmWide = 100, kGmWideChunk = 1024;
 template <int D, int NT, int NW, int MB>
 cudaError_t launch_gather_mma(const StepParams& p, dim3 grid, cudaStream_t st) {
   return launch_ex(p.paged ? k_gather_mma<D, NT, NW, MB, true> : k_gather_mma<D, NT, NW, MB, false>, grid, dim3(32 * NW),
@@ -4181,21 +4181,32 @@ cudaError_t launch_gather_td(const StepParams& p, cudaStream_t st) {
   }
   const dim3 grid(p.nc, p.Hkv, p.B);
   if (sizeof(T) == 2) {
-    // Eight warps where one CTA per (sequence, kv-head) has a long list to
-    // itself: such a grid is about one wave, and at two CTAs per SM its last
-    // third leaves room, CTA by CTA, for the next call's score kernel (1280 of
-    // 6400, 64 sequences, 8 kv-heads: the call 229 us, with four warps 241,
-    // though the gather alone takes 43 against 42 us).  Chunked lists run
-    // several waves (8192 of 16384: 212 us with four warps, 230 with eight),
-    // short ones one or two steps per warp (29 of 576: 6.1 against 9.2 us).
-    // Three CTAs per SM (fewer registers) where that saves a wave (40 sequences,
-    // 1250 of 5000: 144 us, two per SM 153; 1280 of 6400 runs two waves either
-    // way: 227 us, three per SM 242).
+    // Eight warps where one CTA per (sequence, kv-head) has a list of kGmWide
+    // rows or more to itself: such a grid is about one wave, and at two CTAs per
+    // SM its last third leaves room, CTA by CTA, for the next call's score
+    // kernel, which four-warp CTAs, all resident and ending together, do not (64
+    // sequences, 8 kv-heads, the call with eight / four warps: 1280 of 6400 229 /
+    // 241 us, 460 of 2304 122 / 134, 288 of 576 85 / 90, 115 of 576 74.4 / 76.8;
+    // one or two steps per warp, 29 of 576: 71.4 / 69.3).  Three CTAs per SM
+    // (fewer registers) where that saves a wave (40 sequences, 1250 of 5000: 144
+    // us, two per SM 153; 1280 of 6400 runs two waves either way: 227 us, three
+    // per SM 242).
+    // Several chunks: four warps take about a tenth less time a byte (2048 CTAs,
+    // 8192 of 16384: 616 us, eight warps 632), and a grid that the SMs hold at
+    // once stays with them (320 CTAs, 6000 of 12000: 114, 120; 640, 3000 of
+    // 10000: 241, 255); so eight only in several waves that are that much
+    // fuller, two CTAs per SM against five (1024 CTAs, 3200 of 6400: 282 us,
+    // four warps 295; 1536, 5734 of 16384: 568, 575).  Measured at D = 128 only.
+    const long long n = (long long)p.nc * p.Hkv * p.B, two = 2LL * p.num_sms, three = 3LL * p.num_sms;
     if (p.nk == 1 && p.kept_cap >= kGmWide) {
-      const long long n = (long long)p.nc * p.Hkv * p.B, two = 2LL * p.num_sms, three = 3LL * p.num_sms;
       if (p.G > 8) return launch_gather_mma<D, 2, 8, 1>(p, grid, st);
       return (n + three - 1) / three < (n + two - 1) / two ? launch_gather_mma<D, 1, 8, 3>(p, grid, st)
                                                            : launch_gather_mma<D, 1, 8, 2>(p, grid, st);
+    }
+    if (D == 128 && p.G <= 8 && p.nk > 1 && p.kept_cap >= (long long)kGmWideChunk * p.nk) {
+      const long long five = 5LL * p.num_sms;
+      if (n > five && 11 * two * ((n + two - 1) / two) < 10 * five * ((n + five - 1) / five))
+        return launch_gather_mma<D, 1, 8, 2>(p, grid, st);
     }
     return p.G <= 8 ? launch_gather_mma<D, 1, 4, 5>(p, grid, st) : launch_gather_mma<D, 2, 4, 3>(p, grid, st);
   }

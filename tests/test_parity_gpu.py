@@ -147,7 +147,7 @@ def test_kept_row_steps(vp, H, Hkv, D, paged, k):
 
 @pytest.mark.parametrize("paged", [False, True])
 def test_chunk_gather_long_lists(vp, paged):
-    """One CTA per (sequence, kv-head) with a list of more than 512 rows (the
+    """One CTA per (sequence, kv-head) with a long list (the
     eight-warp forms: 320 CTAs fill one wave at three per SM, 480 take two
     either way), ragged spans."""
     for batch in (40, 60):
@@ -157,6 +157,14 @@ def test_chunk_gather_long_lists(vp, paged):
         inp = Hn.make_inputs(r)
         budget = dict(mode=O.FIXED_RATIO, tau=0.1, ratio_ppm=850_000)
         Hn.check_all(vp, inp, budget, seqs=(0, 7, batch - 1))
+
+
+def test_chunk_gather_two_long_chunks(vp):
+    """Two chunks of more than 1024 rows (768 CTAs: the eight-warp form, its
+    waves fuller than the four-warp ones), the last sequences' spans shorter."""
+    vis = tuple(2470 if i < 2 else 64 if i < 45 else 900 * (i - 44) - 899 for i in range(48))
+    r = small(heads=8, kv_heads=8, head_dim=128, batch=48, vis_len=vis, vis_start=(1,) * 48, text_len=(20,) * 48)
+    Hn.check_all(vp, Hn.make_inputs(r), dict(mode=O.FIXED_RATIO, tau=0.1, ratio_ppm=850_000), seqs=(0, 1, 44, 45, 46, 47))
 
 
 @pytest.mark.parametrize("H,Hkv,batch,gran", [(28, 4, 1, 0), (14, 2, 3, 0), (8, 2, 5, 1), (28, 4, 20, 1), (28, 4, 80, 0),
