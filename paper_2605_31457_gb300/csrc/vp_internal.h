@@ -298,11 +298,15 @@ inline WsLayout ws_layout(int batch, int H, int Hkv, int D, int max_visual, int 
   w.hp = (H + 3) / 4 * 4;
   w.nk_max = kNkMax;
   w.nsp_max = 1;
+  // Every plan a call may get: a plan beside the select clusters (second_set)
+  // has fewer slots, which can make more splits the better count.
   for (int bb = 1; bb <= batch; ++bb)
-    for (int tc = 0; tc < 2; ++tc) {
-      const Plan pl = make_plan(bb, Hkv, D, num_sms, max_visual, max_seq, 0, 0, tc != 0);
-      if (pl.ns > w.nsp_max) w.nsp_max = pl.ns;
-    }
+    for (int tc = 0; tc < 2; ++tc)
+      for (int gran = 0; gran < (second_set ? 2 : 1); ++gran)
+        for (int beside = 0; beside < (second_set ? 2 : 1); ++beside) {
+          const Plan pl = make_plan(bb, Hkv, D, num_sms, max_visual, max_seq, 0, gran, tc != 0, beside != 0);
+          if (pl.ns > w.nsp_max) w.nsp_max = pl.ns;
+        }
   const size_t B = (size_t)batch, G = (size_t)(H / Hkv);
   size_t off = 0;
   w.o_tickets = off; off = ws_round(off + B * Hkv * 4);

@@ -108,6 +108,38 @@ int check_chunks() {
   return bad;
 }
 
+// Contexts with two sets of the score kernels' outputs plan with `beside`: their
+// splits must fit the workspace too, for every batch up to max_batch, both
+// granularities and any kv-head count a context accepts (H <= 128).
+int check_beside() {
+  using namespace vp;
+  const int before = fails;
+  long long plans = 0;
+  for (int Hkv : {1, 2, 3, 4, 5, 8, 12, 16, 28, 40, 48, 56, 64, 96, 128})
+    for (int D : {64, 128})
+      for (int sms : {152, 132})
+        for (int max_batch : {1, 2, 3, 4, 7, 16, 64})
+          for (int mv : {0, 256, 2304, 16384, 32767})
+            for (int ex : {1, 64, 257, 1975, 2561, 3513, 4869, 7173, 11772, 30000}) {
+              const int ms = mv + ex, H = Hkv;
+              if (!two_sets(max_batch, Hkv, D, ms, 2)) continue;
+              const WsLayout ws = ws_layout(max_batch, H, Hkv, D, mv, ms, sms, true);
+              for (int B = 1; B <= max_batch; ++B)
+                for (int tc = 0; tc < 2; ++tc)
+                  for (int gran = 0; gran < 2; ++gran) {
+                    const Plan pl = make_plan(B, Hkv, D, sms, mv, ms, 64, gran, tc != 0, true);
+                    ++plans;
+                    check(pl.ns >= 1 && pl.ns <= kNsMax && pl.ns <= ws.nsp_max, "beside: ns within the workspace", B, Hkv,
+                          D, sms, mv, ms, 64, tc, gran);
+                    const int w = split_floor(pl, B, Hkv, sms, tc != 0, pl.split_w);
+                    check(w >= 1 && w <= pl.split_w, "split_floor within the planned weight", B, Hkv, D, sms, mv, ms, 64,
+                          tc, gran);
+                  }
+            }
+  std::printf("%lld plans beside a select kernel, %d violations\n", plans, fails - before);
+  return 0;
+}
+
 }  // namespace
 
 int main() {
@@ -174,6 +206,7 @@ int main() {
                   }
             }
   std::printf("%lld plans, %d violations\n", plans, fails);
+  fails += check_beside();
   fails += check_forms();
   fails += check_chunks();
   return fails ? 1 : 0;
