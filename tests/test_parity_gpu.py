@@ -187,6 +187,21 @@ def test_selection_cut(vp, H, Hkv, batch, gran, nv):
         assert all(np.array_equal(row[:k], np.arange(k)) for row in gpu["kept"][-1])
 
 
+@pytest.mark.parametrize("H,Hkv", [(33, 33), (35, 5), (42, 6), (70, 10), (99, 33), (127, 127)])
+@pytest.mark.parametrize("batch", [1, 160])
+def test_selection_head_counts(vp, H, Hkv, batch):
+    """Selection over more than 32 heads whose logit rows are not whole 16-byte
+    pieces, in clusters and (batch 160) without one: every head counts in the
+    scores.  Every second sequence has one visual token that only the last
+    kv-head's queries attend to."""
+    r = small(heads=H, kv_heads=Hkv, head_dim=64, batch=batch, vis_len=67, vis_start=2, text_len=9, seed=H + batch)
+    inp = Hn.make_inputs(r)
+    for b in range(0, batch, 2):
+        inp.k[b, :, 2 + 41] = 0
+        inp.k[b, -1, 2 + 41] = 30 * inp.q[b, -1] / inp.q[b, -1].float().norm()
+    Hn.check_all(vp, inp, dict(mode=O.FIXED_RATIO, tau=0.1, ratio_ppm=60_000), seqs=sorted({0, 1 % batch, batch - 1}))
+
+
 def test_paged_cache(vp):
     r = small(batch=4, vis_len=(300, 577, 64, 1000), vis_start=(0, 13, 40, 0),
               text_len=(517, 70, 129, 33), paged=True, page_size=16)
