@@ -2996,7 +2996,7 @@ __global__ void __launch_bounds__(32 * NW, MB) k_gather_mma(const __grid_constan
         if (i < n && (e[u] < 0 || e[u] >= sq.nv)) { err |= ERR_KEPT; e[u] = -1; }
         if constexpr (PAGED) {
           const int lp = (sq.vs + e[u]) >> p.page_shift;
-          pg[u] = e[u] >= 0 && lp < p.v.max_pages ? __ldg(p.v.block_table + (int64_t)b * p.v.max_pages + lp) : 0;
+          pg[u] = e[u] < 0 ? 0 : lp < p.v.max_pages ? __ldg(p.v.block_table + (int64_t)b * p.v.max_pages + lp) : -1;
         }
       }
 #pragma unroll

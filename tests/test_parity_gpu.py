@@ -202,6 +202,32 @@ def test_selection_head_counts(vp, H, Hkv, batch):
     Hn.check_all(vp, inp, dict(mode=O.FIXED_RATIO, tau=0.1, ratio_ppm=60_000), seqs=sorted({0, 1 % batch, batch - 1}))
 
 
+@pytest.mark.parametrize("H,Hkv,batch", [(28, 4, 1), (16, 8, 45), (32, 2, 3)])
+def test_chunk_gather_short_value_table(vp, H, Hkv, batch):
+    """Kept rows past the end of V's block table (K's is longer) are skipped and
+    flagged: the output is the attention over the text and the other kept rows."""
+    vs, nv, rows = 128, 896, 512
+    r = small(heads=H, kv_heads=Hkv, head_dim=64, batch=batch, vis_len=nv, vis_start=vs, text_len=vs, paged=True,
+              page_size=16)
+    inp = Hn.make_inputs(r)
+    dev = Hn.Device(vp, inp, dict(mode=O.DENSE, tau=0.1))
+    try:
+        short = dev.bt[:, :(vs + rows) // 16].contiguous()
+        dev.vc = vp.kv_paged(dev.v_t, short)
+        out = dev.run(check_errors=False)["out"]
+        with pytest.raises(vp.VPError, match="block table"):
+            vp.vp_check_errors(dev.ctx)
+    finally:
+        dev.close()
+    keep = np.arange(vs + nv) < vs + rows
+    for b in sorted({0, batch - 1}):
+        z = Hn.oracle_seq(inp, b, dev.budget_dict)["z"]
+        v = inp.v[b, :, :vs + nv].double().numpy()
+        for h in range(H):
+            want = O.pruned_attention(z[h:h + 1], v[h * Hkv // H][None], keep)[0]
+            np.testing.assert_allclose(out[b][h], want, rtol=0, atol=2e-2)
+
+
 def test_paged_cache(vp):
     r = small(batch=4, vis_len=(300, 577, 64, 1000), vis_start=(0, 13, 40, 0),
               text_len=(517, 70, 129, 33), paged=True, page_size=16)
