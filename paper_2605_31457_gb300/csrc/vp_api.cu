@@ -41,7 +41,7 @@ struct vp_ctx {
   int64_t tcalls = 0;
   int32_t last_score_path = 0;  // vp_last_launch: score kernel and kernel count of the last call
   int32_t last_kernels = 0;
-  bool second_set = false;  // which set of the score kernel's outputs the next call uses
+  vp::SetTurn turn;  // which set of the score kernel's outputs the next call uses
 };
 
 namespace {
@@ -69,13 +69,30 @@ vp_status cuda_fail(vp_ctx* ctx, const char* what, cudaError_t e) {
 int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 // The set of the score kernel's outputs for a call about to be enqueued.
-void take_set(vp_ctx* ctx, vp::StepParams& p) {
-  const size_t off = ctx->second_set ? ctx->lay.o_set2 / sizeof(float) : 0;
+void take_set(vp_ctx* ctx, vp::StepParams& p, cudaStream_t st) {
+  const size_t off = ctx->turn.second ? ctx->lay.o_set2 / sizeof(float) : 0;
   p.z_ws = ctx->z_ws + off;
   p.split_st = ctx->split_st + off;
   p.split_o = ctx->split_o + off;
   p.ws_free = ctx->lay.o_set2 != 0;
-  if (p.ws_free) ctx->second_set = !ctx->second_set;
+  if (!p.ws_free) return;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(st, &cs, &id) != cudaSuccess) {
+    cudaGetLastError();
+    ctx->turn.chained = false;
+  }
+  p.ordered = ctx->turn.begin(st, cs == cudaStreamCaptureStatusNone ? 0 : id + 1);
+}
+// Enqueues the score kernel of the call that took its set.
+cudaError_t enqueue_score(vp::StepParams& p, cudaStream_t st) {
+  const cudaError_t e = vp::launch_score(p, st);
+  p.ordered = 0;
+  return e;
+}
+// Every kernel of the call is enqueued.
+void set_taken(vp_ctx* ctx) {
+  if (ctx->lay.o_set2) ctx->turn.end();
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -293,8 +310,8 @@ vp_status vp_decode_step(vp_ctx* ctx, int32_t batch, const void* q,
   }
   p.fused = vp::select_kind(p, kept_cap);
 
-  take_set(ctx, p);
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  take_set(ctx, p, st);
   cudaEvent_t* tev = nullptr;
   unsigned rec_flags = cudaEventRecordDefault;
   if (ctx->tslots > 0) {
@@ -305,7 +322,7 @@ vp_status vp_decode_step(vp_ctx* ctx, int32_t batch, const void* q,
   }
   cudaError_t e = cudaSuccess;
   if (tev) e = cudaEventRecordWithFlags(tev[0], st, rec_flags);
-  if (e == cudaSuccess) e = vp::launch_score(p, st);
+  if (e == cudaSuccess) e = enqueue_score(p, st);
   if (e != cudaSuccess) return cuda_fail(ctx, "vp_decode_step: score kernel launch", e);
   if (tev) e = cudaEventRecordWithFlags(tev[1], st, rec_flags);
   if (e == cudaSuccess) e = vp::launch_select(p, st);
@@ -313,6 +330,7 @@ vp_status vp_decode_step(vp_ctx* ctx, int32_t batch, const void* q,
   if (tev) e = cudaEventRecordWithFlags(tev[2], st, rec_flags);
   if (e == cudaSuccess) e = vp::launch_gather(p, st);
   if (e != cudaSuccess) return cuda_fail(ctx, "vp_decode_step: gather kernel launch", e);
+  set_taken(ctx);
   if (tev) e = cudaEventRecordWithFlags(tev[3], st, rec_flags);
   if (e != cudaSuccess) return cuda_fail(ctx, "vp_decode_step: timing event", e);
   ctx->last_score_path = p.use_tc ? VP_SCORE_TC : VP_SCORE_MMA;
@@ -388,12 +406,13 @@ vp_status vp_decode_gather(vp_ctx* ctx, int32_t batch, const void* q,
   if (!p.use_tma)
     return fail(ctx, VP_ERR_UNSUPPORTED, "vp_decode_gather: the cache layout needs the bulk-tensor path "
                 "(token axis not outermost, pages of at least 8 tokens)");
-  take_set(ctx, p);
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  cudaError_t e = vp::launch_score(p, st);
+  take_set(ctx, p, st);
+  cudaError_t e = enqueue_score(p, st);
   if (e != cudaSuccess) return cuda_fail(ctx, "vp_decode_gather: score kernel launch", e);
   e = vp::launch_merge(p, st);
   if (e != cudaSuccess) return cuda_fail(ctx, "vp_decode_gather: merge kernel launch", e);
+  set_taken(ctx);
   ctx->last_score_path = VP_SCORE_MMA;
   ctx->last_kernels = 2;
   return VP_OK;

@@ -99,6 +99,7 @@ struct StepParams {
                       // 2 k_selgat selecting only (fast_select_ok)
   int split_w;        // weight of one score split (bulk-tensor kernel)
   int num_sms;        // SMs of the device (launch shapes chosen per call)
+  int ordered;        // launch only: 1 while the next kernel must wait for everything before it on the stream
 };
 
 // ---------------------------------------------------------------- host planning
@@ -284,6 +285,30 @@ constexpr size_t kSet2Cache = (size_t)256 << 20, kSet2CacheF32 = (size_t)64 << 2
 inline bool two_sets(int batch, int Hkv, int D, int max_seq, int esz) {
   return (size_t)batch * Hkv * max_seq * D * esz * 2 <= (esz == 2 ? kSet2Cache : kSet2CacheF32);
 }
+// That needs calls that are adjacent on the device to use different sets, which
+// the order of the host's calls alone does not give: a captured call runs when
+// its graph does, or never, and a call whose launches failed leaves no last
+// kernel.  So a call that does not follow a complete call of the same context
+// on the same stream and in the same capture (0: none) is `ordered`: its score
+// kernel is launched without the programmatic overlap, after everything before
+// it on the stream, when no kernel reads either set.
+struct SetTurn {
+  bool second = false;  // set of the next call
+  bool chained = false;
+  const void* stream = nullptr;
+  unsigned long long capture = 0;
+  bool begin(const void* st, unsigned long long cap) {  // returns whether the call is ordered
+    const bool ordered = !chained || st != stream || cap != capture;
+    stream = st;
+    capture = cap;
+    chained = false;
+    return ordered;
+  }
+  void end() {  // every kernel of the call was enqueued
+    second = !second;
+    chained = true;
+  }
+};
 struct WsLayout {
   size_t o_tickets, o_err, zero_bytes, o_z, o_st, o_o, o_go, o_gs, o_mo, o_ms, o_hm, total;
   size_t o_set2;  // 0: one set

@@ -6,7 +6,9 @@
 // picks the slice gather only for kept sets it holds; a table of call shapes
 // gets its expected select form, and a table of the chunk gather's call
 // shapes its chunk count, CTAs per (sequence, kv-head) and whether the lone
-// CTA combines in place.  Prints one line per violation and exits non-zero if
+// CTA combines in place; the plans of contexts with two sets of the
+// score kernels' outputs fit the workspace as well, and their calls never take
+// the set of the call before them on the device (SetTurn).  Prints one line per violation and exits non-zero if
 // there was any.
 #include <cstdio>
 
@@ -140,6 +142,39 @@ int check_beside() {
   return 0;
 }
 
+// The sets that calls take, whatever mix of streams, captures and failed
+// launches the host's calls come in: of two calls adjacent on the device (in
+// one stream, or in one capture of it), the later uses the other set or is
+// ordered, and it is ordered after a call that failed.
+int check_turns() {
+  using namespace vp;
+  struct Last { int set = -1; bool complete = true; };
+  unsigned rnd = 12345;
+  auto draw = [&](unsigned n) { rnd = rnd * 1664525u + 1013904223u; return (rnd >> 16) % n; };
+  int bad = 0, free_calls = 0;
+  for (int trial = 0; trial < 2000; ++trial) {
+    SetTurn turn;
+    Last last[3][3];
+    const unsigned n_st = 1 + draw(2), n_cap = 1 + draw(3), fail_pct = trial % 2 ? 10 : 0;
+    static const int streams[3] = {};
+    unsigned st = 0, cap = 0;
+    for (int call = 0; call < 40; ++call) {
+      if (draw(4) == 0) st = draw(n_st);
+      if (draw(4) == 0) cap = draw(n_cap);
+      Last& l = last[st][cap];
+      const bool ordered = turn.begin(&streams[st], cap);
+      const int set = turn.second;
+      if (!ordered && (set == l.set || !l.complete)) ++bad;
+      free_calls += !ordered;
+      l = Last{set, draw(100) >= fail_pct};
+      if (l.complete) turn.end();
+    }
+  }
+  if (bad || free_calls < 10000)
+    std::printf("FAIL turns of the output sets: %d calls on a set in use, %d calls not ordered\n", bad, free_calls);
+  return bad || free_calls < 10000;
+}
+
 }  // namespace
 
 int main() {
@@ -207,6 +242,7 @@ int main() {
             }
   std::printf("%lld plans, %d violations\n", plans, fails);
   fails += check_beside();
+  fails += check_turns();
   fails += check_forms();
   fails += check_chunks();
   return fails ? 1 : 0;

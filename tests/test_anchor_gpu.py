@@ -214,3 +214,54 @@ def test_calls_in_turn_on_one_context(vp, dtype):
     finally:
         for d in devs:
             d.close()
+
+
+def test_captured_calls_between_enqueued_ones(vp):
+    """Calls captured on another stream, and not launched, between calls that
+    are enqueued back to back: the enqueued ones still use the score kernels'
+    output sets in turn, and equal the call run alone, bit for bit; so do the
+    captured ones when their graph runs."""
+    r = small(layers=2, vis_len=(900, 577, 64), text_len=(517, 1070, 129))
+    devs = [Hn.Device(vp, Hn.make_inputs(r, i, t_cap=1700), r.budget, max_seq=1700) for i in range(2)]
+    ctx = devs[0].ctx
+
+    def new(d):
+        return [torch.full_like(d.out, float("nan")), torch.full_like(d.kept, -7), torch.full_like(d.count, -7),
+                torch.full_like(d.mass, float("nan"))]
+
+    def call(d, o, stream):
+        vp.vp_decode_step(ctx, d.B, d.q, d.kc, d.vc, d.span, d.tl, d.budget, o[0], o[1], d.kept_cap, o[2], o[3],
+                          stream=stream)
+
+    try:
+        want = []
+        for d in devs:
+            o = new(d)
+            call(d, o, None)
+            torch.cuda.synchronize()
+            want.append(o)
+        run, side = torch.cuda.Stream(), torch.cuda.Stream()
+        n = 24
+        outs = [new(devs[i % 2]) for i in range(n)]
+        captured = [[new(devs[(i + j) % 2]) for j in range(1 + i % 2)] for i in range(n)]
+        graphs = [torch.cuda.CUDAGraph() for _ in range(n)]
+        torch.cuda.synchronize()
+        for i in range(n):
+            call(devs[i % 2], outs[i], run)
+            with torch.cuda.stream(side):
+                graphs[i].capture_begin(capture_error_mode="relaxed")
+                for j, o in enumerate(captured[i]):
+                    call(devs[(i + j) % 2], o, side)
+                graphs[i].capture_end()
+        torch.cuda.synchronize()
+        for g in graphs:
+            g.replay()
+        vp.vp_check_errors(ctx)
+        torch.cuda.synchronize()
+        for i in range(n):
+            for j, o in [(i, outs[i])] + [(i + j, o) for j, o in enumerate(captured[i])]:
+                for a, b in zip(o, want[j % 2]):
+                    assert torch.equal(a.view(torch.uint8), b.view(torch.uint8)), i
+    finally:
+        for d in devs:
+            d.close()

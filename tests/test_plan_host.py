@@ -6,7 +6,9 @@ the chunk kernel's limit, the slice gather is chosen only for kept sets it
 can hold, every benchmarked call shape gets the expected select form
 (fused select + gather and its slice width, select only, or the
 shared-memory select), and the chunk gather's benchmarked shapes get their
-expected chunk count, text-merge slices and CTAs per (sequence, kv-head)
+expected chunk count, text-merge slices and CTAs per (sequence, kv-head); the
+splits of plans beside a select kernel fit the workspace, and calls never take
+the output set of the call before them on the device
 (tests/plan_invariants.cpp)."""
 
 import os
