@@ -51,10 +51,6 @@ constexpr int64_t kPpm = 1000000;
 constexpr int kMaxVisual = 32768;  // score keys of one sequence fit in shared memory
 constexpr int kMaxHeads = 128;
 constexpr int kMaxGroup = 16;
-// Splits of a layer after the anchor layer, at most: the merge kernel's groups
-// take up to eight each in one round trip (B = 1 decode, 27 such layers: 37
-// splits 234 us, 32 230, 24 241).
-constexpr int kGatherSplits = 32;
 
 vp_status fail(vp_ctx* ctx, vp_status st, const std::string& msg) {
   if (ctx) ctx->last_error = msg;
@@ -391,17 +387,11 @@ vp_status vp_decode_gather(vp_ctx* ctx, int32_t batch, const void* q,
   p.out = out;
   p.gpart_o = ctx->gpart_o; p.gpart_st = ctx->gpart_st; p.tickets = ctx->tickets; p.err = ctx->err;
   p.mt_o = ctx->mt_o; p.mt_st = ctx->mt_st; p.hmax = ctx->hmax;
-  // Score splits as planned for the decode step; their weight covers the
-  // cache outside the visual span plus the kept rows.
-  vp::Plan pl = vp::make_plan(batch, Hkv, D, ctx->num_sms, c.max_visual, c.max_seq, 0, granularity);
-  pl.ns = std::min(pl.ns, kGatherSplits);
+  const vp::Plan pl = vp::gather_plan(batch, Hkv, D, ctx->num_sms, c.max_visual, c.max_seq, kept_cap, granularity,
+                                      p.paged, p.page_size);
   p.hp = ctx->lay.hp;
   p.ns = pl.ns; p.nsp_max = ctx->lay.nsp_max; p.cl = 1;
-  {
-    long long w = 2LL * ((c.max_seq + 31) / 32 - c.max_visual / 32 + (kept_cap + 31) / 32);
-    if (w < 1) w = 1;
-    p.split_w = vp::split_floor(pl, batch, Hkv, ctx->num_sms, false, (int)((w + pl.ns - 1) / pl.ns));
-  }
+  p.split_w = pl.split_w;
   vp::encode_kv_maps(p);
   if (!p.use_tma)
     return fail(ctx, VP_ERR_UNSUPPORTED, "vp_decode_gather: the cache layout needs the bulk-tensor path "

@@ -160,6 +160,21 @@ inline int tc_max_split_tiles(int max_seq, int ns, int split_w) {
   const long long per = split_w > fair ? split_w : fair;
   return (int)(per / kTcWv + 1);
 }
+constexpr int kTmaTile = 32;         // rows of a tile of the mma.sync score kernel
+constexpr int kTmaMaxBoxes = 1024;   // page ids per cache one of its CTAs stages
+// Whether the page ids of a score CTA's boxes fit its staging, for any sequence
+// of at most max_seq tokens in ns splits of weight split_w (bf16 caches; the
+// boxes of a CTA grow as its splits get fewer).
+inline bool page_ids_fit(int paged, int page_size, int max_seq, int ns, int split_w, bool tc) {
+  if (!paged) return true;
+  if (tc) {
+    const int rows = page_size < kTcRows ? page_size : kTcRows;
+    return (int64_t)tc_max_split_tiles(max_seq, ns, split_w) * (kTcRows / rows) <= kTcMaxBoxes;
+  }
+  const int rows = page_size < kTmaTile ? page_size : kTmaTile;
+  const int64_t tiles = (max_seq + kTmaTile - 1) / kTmaTile;
+  return ((2 * tiles + ns - 1) / ns + 1) * (kTmaTile / rows) <= kTmaMaxBoxes;
+}
 constexpr int kNsMax = 256;   // score splits per (sequence, kv-head)
 constexpr int kMaxMerge = 8;  // gather CTAs merging slices of the text partials
 
@@ -260,6 +275,38 @@ inline int split_floor(const Plan& pl, int batch, int Hkv, int num_sms, bool tc,
   if ((long long)batch * Hkv * pl.ns > 2LL * num_sms) return planned_w;
   const int least = tc ? 2 * kTcWv : 8;
   return planned_w < least ? planned_w : least;
+}
+
+// Score splits and select clusters of a decode step.  Fewer splits beside a
+// select kernel hold more page ids each: where those no longer fit, the call
+// keeps the splits it has on the whole GPU (paged, 8-token pages, 8 sequences
+// of 65536 tokens, one kv-head: 22 splits of 33 tiles, 38 of 19 fit).
+inline Plan step_plan(int batch, int Hkv, int D, int num_sms, int max_visual, int max_seq, int kept_cap,
+                      int granularity, bool tc, bool beside, int paged, int page_size) {
+  for (;; beside = false) {
+    Plan pl = make_plan(batch, Hkv, D, num_sms, max_visual, max_seq, kept_cap, granularity, tc, beside);
+    pl.split_w = split_floor(pl, batch, Hkv, num_sms, tc, pl.split_w);
+    if (!beside || page_ids_fit(paged, page_size, max_seq, pl.ns, pl.split_w, tc)) return pl;
+  }
+}
+
+// Splits of a layer after the anchor layer, at most: the merge kernel's groups
+// take up to eight each in one round trip (B = 1 decode, 27 such layers: 37
+// splits 234 us, 32 230, 24 241).
+constexpr int kGatherSplits = 32;
+// Score splits of a layer after the anchor layer: as planned for the decode
+// step, at most kGatherSplits unless their page ids need more.  Their weight
+// covers the cache outside the visual span plus the kept rows.
+inline Plan gather_plan(int batch, int Hkv, int D, int num_sms, int max_visual, int max_seq, int kept_cap,
+                        int granularity, int paged, int page_size) {
+  Plan pl = make_plan(batch, Hkv, D, num_sms, max_visual, max_seq, 0, granularity);
+  long long w = 2LL * ((max_seq + 31) / 32 - max_visual / 32 + (kept_cap + 31) / 32);
+  if (w < 1) w = 1;
+  const int ns = pl.ns;
+  for (pl.ns = ns < kGatherSplits ? ns : kGatherSplits;; pl.ns = ns) {
+    pl.split_w = split_floor(pl, batch, Hkv, num_sms, false, (int)((w + pl.ns - 1) / pl.ns));
+    if (pl.ns == ns || page_ids_fit(paged, page_size, max_seq, pl.ns, pl.split_w, false)) return pl;
+  }
 }
 
 // Workspace layout for up to `batch` sequences (offsets in bytes, 256-aligned).
@@ -447,9 +494,10 @@ inline bool plan_step(StepParams& p, int num_sms, int kept_cap, int granularity,
   if (path == 2 && !tc) return false;
   for (int pass = 0; pass < 2; ++pass) {
     const bool want = tc && pass == 0;
-    const Plan pl = make_plan(p.B, p.Hkv, p.D, num_sms, p.max_visual, p.max_seq, kept_cap, granularity, want, beside);
+    const Plan pl = step_plan(p.B, p.Hkv, p.D, num_sms, p.max_visual, p.max_seq, kept_cap, granularity, want, beside,
+                              p.dtype == 0 && p.paged, p.page_size);
     p.ns = pl.ns; p.cl = pl.cl; p.nk = pl.nk; p.nm = pl.nm; p.nc = pl.nc; p.gslice = pl.gslice;
-    p.split_w = split_floor(pl, p.B, p.Hkv, num_sms, want, pl.split_w);
+    p.split_w = pl.split_w;
     p.use_tc = want ? 1 : 0;
     encode_kv_maps(p);
     if (p.use_tc || !want) return true;

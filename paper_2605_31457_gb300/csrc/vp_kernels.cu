@@ -663,8 +663,6 @@ __global__ void __launch_bounds__(kThreads) k_score_mma(const __grid_constant__ 
 // the slot.  For paged caches the page ids of the CTA's boxes are read into
 // shared memory once, before the first copy.
 // ---------------------------------------------------------------------------
-constexpr int kTmaTile = 32;
-constexpr int kTmaMaxBoxes = 1024;  // page-id entries per cache a CTA may hold
 
 template <int D, int NT, int NW, int S>
 struct TmaCfg {
@@ -4445,22 +4443,12 @@ void encode_kv_maps(StepParams& p) {
     return true;
   };
   if (want_tc && tc_eligible(p.dtype, p.D, p.G, p.paged, p.page_size)) {
-    // Page ids of a split's boxes are staged in shared memory: bound them.
     const int R2 = p.paged ? (p.page_size < kTcRows ? p.page_size : kTcRows) : kTcRows;
-    const int64_t boxes = p.paged ? (int64_t)tc_max_split_tiles(p.max_seq, p.ns, p.split_w) * (kTcRows / R2) : 0;
-    if (boxes <= kTcMaxBoxes && encode(R2)) p.use_tc = p.use_tma = 1;
+    if (page_ids_fit(p.paged, p.page_size, p.max_seq, p.ns, p.split_w, true) && encode(R2)) p.use_tc = p.use_tma = 1;
     return;  // without the tensor-core kernel the caller plans for the others
   }
   const int R = p.paged ? (p.page_size < kTmaTile ? p.page_size : kTmaTile) : kTmaTile;
-  if (!encode(R)) return;
-  if (p.paged) {
-    // Page ids of a CTA's boxes are staged in shared memory: bound them.
-    const int64_t tiles = (p.max_seq + kTmaTile - 1) / kTmaTile;
-    const int64_t per_cta = (2 * tiles + p.ns - 1) / p.ns + 1;
-    const int64_t boxes = per_cta * (kTmaTile / R);
-    if (boxes > kTmaMaxBoxes) return;
-  }
-  p.use_tma = 1;
+  if (page_ids_fit(p.paged, p.page_size, p.max_seq, p.ns, p.split_w, false) && encode(R)) p.use_tma = 1;
 }
 
 cudaError_t configure_kernels(int max_visual, int H, int nsp_max) {

@@ -8,7 +8,8 @@
 // shapes its chunk count, CTAs per (sequence, kv-head) and whether the lone
 // CTA combines in place; the plans of contexts with two sets of the
 // score kernels' outputs fit the workspace as well, and their calls never take
-// the set of the call before them on the device (SetTurn).  Prints one line per violation and exits non-zero if
+// the set of the call before them on the device (SetTurn); plans of fewer
+// splits keep the page ids of a paged call within the kernels' staging.  Prints one line per violation and exits non-zero if
 // there was any.
 #include <cstdio>
 
@@ -175,6 +176,42 @@ int check_turns() {
   return bad || free_calls < 10000;
 }
 
+// A call whose page ids fit in the splits of the whole GPU's plan is served by
+// the same score kernel, whatever fewer splits its own plan would rather have:
+// decode steps beside a select kernel, and layers after the anchor layer.
+int check_page_ids() {
+  using namespace vp;
+  int bad = 0, fewer = 0;
+  for (int Hkv : {1, 2, 4, 8, 16})
+    for (int D : {64, 128})
+      for (int B : {1, 2, 4, 8, 16})
+        for (int page : {8, 16, 32, 64, 128})
+          for (int mv : {0, 1296, 16384})
+            for (long long ms = 2 * mv + 1000; ms <= 1 << 20; ms += ms / 7) {
+              const int bsz = B, T = (int)ms;
+              if (two_sets(B, Hkv, D, T, 2))
+                for (int gran = 0; gran < 2; ++gran)
+                  for (int tc = 0; tc < 2; ++tc) {
+                    const Plan whole = step_plan(bsz, Hkv, D, 152, mv, T, 64, gran, tc != 0, false, 1, page);
+                    const Plan pl = step_plan(bsz, Hkv, D, 152, mv, T, 64, gran, tc != 0, true, 1, page);
+                    fewer += pl.ns < whole.ns;
+                    if (page_ids_fit(1, page, T, whole.ns, whole.split_w, tc != 0) &&
+                        !page_ids_fit(1, page, T, pl.ns, pl.split_w, tc != 0) && ++bad <= 10)
+                      std::printf("FAIL page ids of a decode step: B=%d Hkv=%d D=%d page=%d max_visual=%d max_seq=%d "
+                                  "tc=%d gran=%d: %d splits, %d before\n", B, Hkv, D, page, mv, T, tc, gran, pl.ns, whole.ns);
+                  }
+              const Plan whole = make_plan(bsz, Hkv, D, 152, mv, T, 0, 0);
+              const Plan pl = gather_plan(bsz, Hkv, D, 152, mv, T, 64, 0, 1, page);
+              fewer += pl.ns < whole.ns;
+              if ((pl.ns > whole.ns || (page_ids_fit(1, page, T, whole.ns, whole.split_w, false) &&
+                                        !page_ids_fit(1, page, T, pl.ns, pl.split_w, false))) && ++bad <= 10)
+                std::printf("FAIL page ids after the anchor: B=%d Hkv=%d D=%d page=%d max_visual=%d max_seq=%d: %d "
+                            "splits, %d before\n", B, Hkv, D, page, mv, T, pl.ns, whole.ns);
+            }
+  if (bad || fewer < 100) std::printf("FAIL page ids: %d calls lose their kernel, %d plans of fewer splits\n", bad, fewer);
+  return bad || fewer < 100;
+}
+
 }  // namespace
 
 int main() {
@@ -243,6 +280,7 @@ int main() {
   std::printf("%lld plans, %d violations\n", plans, fails);
   fails += check_beside();
   fails += check_turns();
+  fails += check_page_ids();
   fails += check_forms();
   fails += check_chunks();
   return fails ? 1 : 0;

@@ -265,3 +265,26 @@ def test_captured_calls_between_enqueued_ones(vp):
     finally:
         for d in devs:
             d.close()
+
+
+@pytest.mark.parametrize("H,Hkv,D,batch,max_seq,path", [(7, 1, 64, 1, 140_000, 0), (28, 4, 128, 1, 140_000, 0),
+                                                        (7, 1, 128, 8, 65_536, 2)])
+def test_small_pages_in_long_contexts(vp, H, Hkv, D, batch, max_seq, path):
+    """Contexts for long sequences over 8-token pages: calls whose page ids fit
+    only in the splits of the whole GPU's plan are served (decode steps on the
+    tensor-core kernel, layers after the anchor)."""
+    r = small(heads=H, kv_heads=Hkv, head_dim=D, batch=batch, vis_len=(300,) * batch, vis_start=(13,) * batch,
+              text_len=tuple(150 + i for i in range(batch)), paged=True, page_size=8)
+    inp = Hn.make_inputs(r, t_cap=512)
+    dev = Hn.Device(vp, inp, r.budget, max_seq=max_seq, score_path=path)
+    try:
+        gpu = dev.run()
+        vp.vp_decode_gather(dev.ctx, dev.B, dev.q, dev.kc, dev.vc, dev.span, dev.tl, dev.kept, dev.kept_cap, dev.count,
+                            dev.out)  # the anchor's set on the anchor's inputs: the same attention
+        vp.vp_check_errors(dev.ctx)
+        again = dev.out.float().cpu().numpy()
+    finally:
+        dev.close()
+    for b in range(batch):
+        Hn.compare_seq(inp, gpu, b, r.budget)
+    np.testing.assert_allclose(again, gpu["out"], rtol=0, atol=2e-2)
