@@ -290,12 +290,17 @@ inline Plan step_plan(int batch, int Hkv, int D, int num_sms, int max_visual, in
   }
 }
 
-// Splits of a layer after the anchor layer, at most: the merge kernel's groups
-// take up to eight each in one round trip (B = 1 decode, 27 such layers: 37
-// splits 234 us, 32 230, 24 241).
-constexpr int kGatherSplits = 32;
+// Splits of a layer after the anchor layer, at most, while a split's weight
+// stays below kGatherSplitW (nine tiles): the merge kernel's groups take up to
+// eight each in one round trip (B = 1 decode, 27 such layers: 37 splits 234 us,
+// 32 230, 24 241), and longer sequences need the CTAs.  Measured, one sequence
+// of 16384 / 32768 / 65536 / 131072 tokens, us a call with 32 splits and with
+// this rule: 4 kv-heads 11.6 / 17.2 / 32 / 58 and 12.1 / 14.8 / 26.6 / 47,
+// 2 kv-heads 11.3 / 16.7 / 27.7 / 49.7 and 10.7 / 14.1 / 18.0 / 27.9; weights of
+// 6 and 10 are up to a sixth slower at 8192 tokens.
+constexpr int kGatherSplits = 32, kGatherSplitW = 18;
 // Score splits of a layer after the anchor layer: as planned for the decode
-// step, at most kGatherSplits unless their page ids need more.  Their weight
+// step within that limit, unless their page ids need more.  Their weight
 // covers the cache outside the visual span plus the kept rows.
 inline Plan gather_plan(int batch, int Hkv, int D, int num_sms, int max_visual, int max_seq, int kept_cap,
                         int granularity, int paged, int page_size) {
@@ -303,7 +308,8 @@ inline Plan gather_plan(int batch, int Hkv, int D, int num_sms, int max_visual, 
   long long w = 2LL * ((max_seq + 31) / 32 - max_visual / 32 + (kept_cap + 31) / 32);
   if (w < 1) w = 1;
   const int ns = pl.ns;
-  for (pl.ns = ns < kGatherSplits ? ns : kGatherSplits;; pl.ns = ns) {
+  const long long by_w = (w + kGatherSplitW - 1) / kGatherSplitW, most = by_w > kGatherSplits ? by_w : kGatherSplits;
+  for (pl.ns = ns < most ? ns : (int)most;; pl.ns = ns) {
     pl.split_w = split_floor(pl, batch, Hkv, num_sms, false, (int)((w + pl.ns - 1) / pl.ns));
     if (pl.ns == ns || page_ids_fit(paged, page_size, max_seq, pl.ns, pl.split_w, false)) return pl;
   }

@@ -208,6 +208,15 @@ int check_page_ids() {
                 std::printf("FAIL page ids after the anchor: B=%d Hkv=%d D=%d page=%d max_visual=%d max_seq=%d: %d "
                             "splits, %d before\n", B, Hkv, D, page, mv, T, pl.ns, whole.ns);
             }
+  // After the anchor, one long sequence gets every split of the whole GPU's plan.
+  for (int Hkv : {1, 2, 4, 8}) {
+    const Plan whole = make_plan(1, Hkv, 128, 152, 1296, 131072, 0, 0);
+    const Plan pl = gather_plan(1, Hkv, 128, 152, 1296, 131072, 64, 0, 0, 1);
+    if (pl.ns != whole.ns) {
+      std::printf("FAIL splits after the anchor: Hkv=%d: %d of %d\n", Hkv, pl.ns, whole.ns);
+      ++bad;
+    }
+  }
   if (bad || fewer < 100) std::printf("FAIL page ids: %d calls lose their kernel, %d plans of fewer splits\n", bad, fewer);
   return bad || fewer < 100;
 }
