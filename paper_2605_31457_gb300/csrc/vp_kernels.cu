@@ -2263,7 +2263,8 @@ template <int NTH>
 __global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepParams p) {
   constexpr int NW = NTH / 32;
   extern __shared__ __align__(16) uint32_t key_s[];  // [max_visual] score keys (rank 0's copy is used)
-  __shared__ float hM_s[kMaxHeads], hInv_s[kMaxHeads], hMass_s[kMaxHeads], hMass1_s[kMaxHeads];
+  __shared__ __align__(16) float hM_s[kMaxHeads], hInv_s[kMaxHeads];
+  __shared__ float hMass_s[kMaxHeads], hMass1_s[kMaxHeads];
   __shared__ unsigned hist_s[3][256];  // one per radix pass, used in turn
   __shared__ int wsum_s[32];
   __shared__ int sh_i[4];
@@ -2309,7 +2310,7 @@ __global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepPara
   const int hcnt = p.granularity ? p.G : H;
   const bool vec = (hbeg & 3) == 0 && (hcnt & 3) == 0;
   // Logit rows on 16-byte boundaries take the row-shared importance loop below.
-  const bool wide = vec && hcnt >= 4 && hcnt <= 32;
+  const bool wide = vec && hcnt >= 4;
   for (int h = warp; h < H; h += NW) {
     float4 nx0, ny0, nx1, ny1;
     fetch(h + NW, lane, nx0, ny0);
@@ -2400,9 +2401,13 @@ __global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepPara
   // Long slices: LPT lanes share a token row, each reading one float4 of its
   // heads, so that a warp's load covers consecutive rows; eight loads per
   // lane are in flight, and a reduce-scatter over the LPT lanes leaves every
-  // lane whole-token sums to emit.
-  auto wide_loop = [&](auto lpt_tag) {
+  // lane whole-token sums to emit.  More than 32 heads (MORE): further rounds of
+  // 32, a form of its own (40 / 64 heads, the call with one word per load and
+  // now: 32 sequences of N_v = 6400, 158 / 171 and 126 / 116 us; 8 sequences
+  // 68 / 78 and 53 / 55).
+  auto wide_loop = [&](auto lpt_tag, auto more_tag) {
     constexpr int LPT = decltype(lpt_tag)::value, TPI = 32 / LPT, V = 8;
+    constexpr bool MORE = decltype(more_tag)::value;
     const int Q = hcnt / 4, lq = lane % LPT;
     const bool qok = lq < Q;
     float m4[4], i4[4];
@@ -2433,6 +2438,24 @@ __global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepPara
         a = fmaf(fexp2_rel(zz[j].z, m4[2]), i4[2], a);
         v[j] = fmaf(fexp2_rel(zz[j].w, m4[3]), i4[3], a);
       }
+      if constexpr (MORE) {
+        for (int q = LPT + lq; q < Q; q += LPT) {
+          const float4 mq = reinterpret_cast<const float4*>(hM_s + hbeg)[q], iq = reinterpret_cast<const float4*>(hInv_s + hbeg)[q];
+#pragma unroll
+          for (int j = 0; j < V; ++j) {
+            const int tok = base + j * TPI + lane / LPT;
+            if (tok < i1) zz[j] = __ldcg(reinterpret_cast<const float4*>(zb + (int64_t)tok * p.hp) + (q - lq));
+          }
+#pragma unroll
+          for (int j = 0; j < V; ++j) {
+            v[j] = fmaf(fexp2_rel(zz[j].x, mq.x), iq.x, v[j]);
+            v[j] = fmaf(fexp2_rel(zz[j].y, mq.y), iq.y, v[j]);
+            v[j] = fmaf(fexp2_rel(zz[j].z, mq.z), iq.z, v[j]);
+            v[j] = fmaf(fexp2_rel(zz[j].w, mq.w), iq.w, v[j]);
+          }
+        }
+        __syncwarp();
+      }
 #pragma unroll
       for (int s_ = 0; s_ < 3; ++s_) {
         const int o = LPT >> (s_ + 1), half = V >> (s_ + 1);
@@ -2462,10 +2485,11 @@ __global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepPara
   };
   if (wide) {
     const int Q = hcnt / 4;
-    if (Q <= 1) wide_loop(std::integral_constant<int, 1>{});
-    else if (Q <= 2) wide_loop(std::integral_constant<int, 2>{});
-    else if (Q <= 4) wide_loop(std::integral_constant<int, 4>{});
-    else wide_loop(std::integral_constant<int, 8>{});
+    if (Q <= 1) wide_loop(std::integral_constant<int, 1>{}, std::false_type{});
+    else if (Q <= 2) wide_loop(std::integral_constant<int, 2>{}, std::false_type{});
+    else if (Q <= 4) wide_loop(std::integral_constant<int, 4>{}, std::false_type{});
+    else if (Q <= 8) wide_loop(std::integral_constant<int, 8>{}, std::false_type{});
+    else wide_loop(std::integral_constant<int, 8>{}, std::true_type{});
   } else {
     for (int wb = i0 + 32 * warp; wb < i1; wb += NTH) {  // one word of tokens per warp
       const int i = wb + lane;

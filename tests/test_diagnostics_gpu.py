@@ -140,3 +140,28 @@ def test_top_p_cut_and_bits_at_slice_edges(vp, nv, batch, ppm):
     for b in range(batch):
         ref = Hn.compare_seq(inp, gpu, b, budget)
         _compare(ref["s"], delta, n_act.cpu().numpy()[b], flags[b])
+
+
+@pytest.mark.parametrize("heads,kv_heads", [(36, 4), (40, 8), (64, 8), (100, 20), (128, 16), (42, 6)])
+@pytest.mark.parametrize("nv,batch", [(2305, 2), (5001, 2)])
+def test_many_heads(vp, heads, kv_heads, nv, batch):
+    """Importance over more than 32 heads (logit rows of further rounds of 32, and
+    a head count that is no multiple of 4), with top-p budgets and activity bits,
+    in the 512-thread kernel, against the oracle."""
+    r = W.shrink(W.QWEN7B, layers=1, batch=batch, heads=heads, kv_heads=kv_heads, head_dim=64, vis_len=nv, vis_start=3,
+                 text_len=37, steps=1)
+    inp = Hn.make_inputs(r)
+    budget = dict(mode=O.TOP_P, tau=0.1, ratio_ppm=100_000)
+    delta = 1.0 / (nv + 37)
+    bits = torch.zeros((batch, (nv + 31) // 32), dtype=torch.int32, device="cuda")
+    n_act = torch.zeros((batch,), dtype=torch.int32, device="cuda")
+    dev = Hn.Device(vp, inp, budget)
+    try:
+        vp.vp_set_diagnostics(dev.ctx, delta, n_act, bits)
+        gpu = dev.run()
+    finally:
+        dev.close()
+    flags = _bits_to_flags(bits.cpu().numpy().view(np.uint32), nv)
+    for b in range(batch):
+        ref = Hn.compare_seq(inp, gpu, b, budget)
+        _compare(ref["s"], delta, n_act.cpu().numpy()[b], flags[b])
