@@ -2259,8 +2259,10 @@ __device__ __forceinline__ int top_p_cut(const uint32_t* key_s, int n, int ppm, 
   return above + (int)m_eq;
 }
 
+// One CTA per SM is asked for so that the 512-thread form gets the registers
+// for eight logit rows in flight (left to itself the compiler stops at 64).
 template <int NTH>
-__global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepParams p) {
+__global__ void __launch_bounds__(NTH, 1) k_select(const __grid_constant__ StepParams p) {
   constexpr int NW = NTH / 32;
   extern __shared__ __align__(16) uint32_t key_s[];  // [max_visual] score keys (rank 0's copy is used)
   __shared__ __align__(16) float hM_s[kMaxHeads], hInv_s[kMaxHeads];
@@ -2390,22 +2392,25 @@ __global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepPara
   int n_on = 0;
   uint32_t* act_row = p.act_bits ? p.act_bits + ((int64_t)b * nsel + gsel) * p.act_words : nullptr;
   // Stores the key of token i; returns whether S_i > delta (Sec. 4.3).
-  auto emit = [&](int i, float a) {  // a: sum over the heads of exp2(z - M_h) / L_h
+  auto emit = [&](int i, float a, bool act) {  // a: sum over the heads of exp2(z - M_h) / L_h
     const float sc = a * inv_cnt;
     if (!isfinite(sc)) bad = 1;
     key0[i] = __float_as_uint(sc);
-    const bool on = diag && __float_as_uint(sc) > p.act_delta_bits;
+    if (!act) return false;
+    const bool on = __float_as_uint(sc) > p.act_delta_bits;
     n_on += on;
     return on;
   };
   // Long slices: LPT lanes share a token row, each reading one float4 of its
   // heads, so that a warp's load covers consecutive rows; eight loads per
   // lane are in flight, and a reduce-scatter over the LPT lanes leaves every
-  // lane whole-token sums to emit.  More than 32 heads (MORE): further rounds of
+  // lane whole-token sums to emit.  The activity words are in the loop only with
+  // diagnostics on (tested per token instead, the 1024-thread form took 24.6 us
+  // at N_v = 6400 and 43.0 at 16384, B = 64; now 22.5 and 38.9).  More than 32 heads (MORE): further rounds of
   // 32, a form of its own (40 / 64 heads, the call with one word per load and
   // now: 32 sequences of N_v = 6400, 158 / 171 and 126 / 116 us; 8 sequences
   // 68 / 78 and 53 / 55).
-  auto wide_loop = [&](auto lpt_tag, auto more_tag) {
+  auto wide_loop = [&](auto lpt_tag, auto more_tag, auto diag_tag) {
     constexpr int LPT = decltype(lpt_tag)::value, TPI = 32 / LPT, V = 8;
     constexpr bool MORE = decltype(more_tag)::value;
     const int Q = hcnt / 4, lq = lane % LPT;
@@ -2423,38 +2428,48 @@ __global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepPara
     for (int s_ = 0; s_ < 3; ++s_)
       if ((LPT >> (s_ + 1)) > 0 && (lane & (LPT >> (s_ + 1)))) off += V >> (s_ + 1);
     for (int base = i0 + warp * V * TPI; base < i1; base += NW * V * TPI) {
-      float4 zz[V];
-#pragma unroll
-      for (int j = 0; j < V; ++j) {
-        const int tok = base + j * TPI + lane / LPT;
-        zz[j] = (qok && tok < i1) ? __ldcg(reinterpret_cast<const float4*>(zb + (int64_t)tok * p.hp))
-                                  : make_float4(-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F);
-      }
       float v[V];
-#pragma unroll
-      for (int j = 0; j < V; ++j) {
-        float a = fexp2_rel(zz[j].x, m4[0]) * i4[0];
-        a = fmaf(fexp2_rel(zz[j].y, m4[1]), i4[1], a);
-        a = fmaf(fexp2_rel(zz[j].z, m4[2]), i4[2], a);
-        v[j] = fmaf(fexp2_rel(zz[j].w, m4[3]), i4[3], a);
-      }
       if constexpr (MORE) {
-        for (int q = LPT + lq; q < Q; q += LPT) {
-          const float4 mq = reinterpret_cast<const float4*>(hM_s + hbeg)[q], iq = reinterpret_cast<const float4*>(hInv_s + hbeg)[q];
+        constexpr int F = NTH >= 1024 ? 4 : 8;  // loads in flight: the 1024-thread form has 64 registers
 #pragma unroll
-          for (int j = 0; j < V; ++j) {
-            const int tok = base + j * TPI + lane / LPT;
-            if (tok < i1) zz[j] = __ldcg(reinterpret_cast<const float4*>(zb + (int64_t)tok * p.hp) + (q - lq));
-          }
+        for (int j = 0; j < V; ++j) v[j] = 0.f;
+#pragma unroll 1
+        for (int q = 0; q < Q - lq; q += LPT) {
+          const float4 mq = reinterpret_cast<const float4*>(hM_s + hbeg)[q + lq];
+          const float4 iq = reinterpret_cast<const float4*>(hInv_s + hbeg)[q + lq];
 #pragma unroll
-          for (int j = 0; j < V; ++j) {
-            v[j] = fmaf(fexp2_rel(zz[j].x, mq.x), iq.x, v[j]);
-            v[j] = fmaf(fexp2_rel(zz[j].y, mq.y), iq.y, v[j]);
-            v[j] = fmaf(fexp2_rel(zz[j].z, mq.z), iq.z, v[j]);
-            v[j] = fmaf(fexp2_rel(zz[j].w, mq.w), iq.w, v[j]);
+          for (int j0 = 0; j0 < V; j0 += F) {
+            float4 zz[F];
+#pragma unroll
+            for (int j = 0; j < F; ++j) {
+              const int tok = min(base + (j0 + j) * TPI + lane / LPT, i1 - 1);  // past the slice: not emitted
+              zz[j] = __ldcg(reinterpret_cast<const float4*>(zb + (int64_t)tok * p.hp) + q);
+            }
+#pragma unroll
+            for (int j = 0; j < F; ++j) {
+              float a = fmaf(fexp2_rel(zz[j].x, mq.x), iq.x, v[j0 + j]);
+              a = fmaf(fexp2_rel(zz[j].y, mq.y), iq.y, a);
+              a = fmaf(fexp2_rel(zz[j].z, mq.z), iq.z, a);
+              v[j0 + j] = fmaf(fexp2_rel(zz[j].w, mq.w), iq.w, a);
+            }
           }
         }
         __syncwarp();
+      } else {
+        float4 zz[V];
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+          const int tok = base + j * TPI + lane / LPT;
+          zz[j] = (qok && tok < i1) ? __ldcg(reinterpret_cast<const float4*>(zb + (int64_t)tok * p.hp))
+                                    : make_float4(-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F);
+        }
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+          float a = fexp2_rel(zz[j].x, m4[0]) * i4[0];
+          a = fmaf(fexp2_rel(zz[j].y, m4[1]), i4[1], a);
+          a = fmaf(fexp2_rel(zz[j].z, m4[2]), i4[2], a);
+          v[j] = fmaf(fexp2_rel(zz[j].w, m4[3]), i4[3], a);
+        }
       }
 #pragma unroll
       for (int s_ = 0; s_ < 3; ++s_) {
@@ -2471,25 +2486,31 @@ __global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepPara
 #pragma unroll
       for (int k = 0; k < V / LPT; ++k) {
         const int tok = base + (k + off) * TPI + lane / LPT;
-        const bool on = tok < i1 && emit(tok, v[k]);
-        if (act_row && __any_sync(0xffffffffu, on)) {
-          // The lanes' tokens of one k span at most V * TPI / 32 words.
+        const bool on = tok < i1 && emit(tok, v[k], decltype(diag_tag)::value);
+        if constexpr (decltype(diag_tag)::value) {
+          if (act_row && __any_sync(0xffffffffu, on)) {
+            // The lanes' tokens of one k span at most V * TPI / 32 words.
 #pragma unroll
-          for (int w = 0; w < V * TPI / 32; ++w) {
-            const unsigned m = __reduce_or_sync(0xffffffffu, on && ((tok - base) >> 5) == w ? 1u << (tok & 31) : 0u);
-            if (m && lane == 0) atomicOr(act_row + (base >> 5) + w, m);
+            for (int w = 0; w < V * TPI / 32; ++w) {
+              const unsigned m = __reduce_or_sync(0xffffffffu, on && ((tok - base) >> 5) == w ? 1u << (tok & 31) : 0u);
+              if (m && lane == 0) atomicOr(act_row + (base >> 5) + w, m);
+            }
           }
         }
       }
     }
   };
   if (wide) {
-    const int Q = hcnt / 4;
-    if (Q <= 1) wide_loop(std::integral_constant<int, 1>{}, std::false_type{});
-    else if (Q <= 2) wide_loop(std::integral_constant<int, 2>{}, std::false_type{});
-    else if (Q <= 4) wide_loop(std::integral_constant<int, 4>{}, std::false_type{});
-    else if (Q <= 8) wide_loop(std::integral_constant<int, 8>{}, std::false_type{});
-    else wide_loop(std::integral_constant<int, 8>{}, std::true_type{});
+    auto any_width = [&](auto diag_tag) {
+      const int Q = hcnt / 4;
+      if (Q <= 1) wide_loop(std::integral_constant<int, 1>{}, std::false_type{}, diag_tag);
+      else if (Q <= 2) wide_loop(std::integral_constant<int, 2>{}, std::false_type{}, diag_tag);
+      else if (Q <= 4) wide_loop(std::integral_constant<int, 4>{}, std::false_type{}, diag_tag);
+      else if (Q <= 8) wide_loop(std::integral_constant<int, 8>{}, std::false_type{}, diag_tag);
+      else wide_loop(std::integral_constant<int, 8>{}, std::true_type{}, diag_tag);
+    };
+    if (diag) any_width(std::true_type{});
+    else any_width(std::false_type{});
   } else {
     for (int wb = i0 + 32 * warp; wb < i1; wb += NTH) {  // one word of tokens per warp
       const int i = wb + lane;
@@ -2498,7 +2519,7 @@ __global__ void __launch_bounds__(NTH) k_select(const __grid_constant__ StepPara
       if (i < i1)
         for (int hh = 0; hh < hcnt; ++hh)
           a = fmaf(fexp2_rel(__ldcg(zr + hh), hM_s[hbeg + hh]), hInv_s[hbeg + hh], a);
-      const bool on = i < i1 && emit(i, a);
+      const bool on = i < i1 && emit(i, a, diag);
       if (act_row) {
         const unsigned m = __ballot_sync(0xffffffffu, on);
         if (m && lane == 0) atomicOr(act_row + (wb >> 5), m);
