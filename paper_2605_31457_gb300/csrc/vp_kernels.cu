@@ -3768,10 +3768,9 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
   fetch4(st0, 0, 2 * warp + sub < H, rx, ry);
 
   // This CTA's slice of the visual tokens.  A group of 2^rsh lanes shares a
-  // token, each lane four of its heads (where they do not start and end on
-  // 16-byte boundaries: head zq, and above 32 heads also zq + 32, zq + 64 and
-  // zq + 96), so that loads cover whole rows and all warps share the
-  // exponentials.  The first kZPre rounds of rows are requested next,
+  // token, each lane four of its heads (one load, or one per head where they do
+  // not start and end on 16-byte boundaries), so that loads cover whole rows and
+  // all warps share the exponentials.  The first kZPre rounds of rows are requested next,
   // so that they arrive while the statistics are merged.
   constexpr int kZPre = GATHER ? 3 : 8;
   const int per = (nv + ncl - 1) / ncl;
@@ -3779,23 +3778,21 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
   const int hbeg = p.granularity ? gsel * G : 0;
   const int hcnt = p.granularity ? G : H;
   const bool vec = (hbeg & 3) == 0 && (hcnt & 3) == 0;
-  const int nq = vec ? hcnt >> 2 : hcnt;  // lanes a token needs, one per piece or head; a group has at most 32
-  // Fused, single heads are at most 16: the cluster's ranks split into the
-  // kv-heads, so more than two of them make H a multiple of 4.
-  const bool rounds = !GATHER && !vec && nq > 32;
-  const int rsh = nq <= 1 ? 0 : 32 - __clz(nq - 1), lpt = 1 << min(rsh, 5);
+  const int nq = (hcnt + 3) >> 2;  // lanes a token needs (at most 128 heads: 32)
+  const int rsh = nq <= 1 ? 0 : 32 - __clz(nq - 1), lpt = 1 << rsh;
   const int zq = tid & (lpt - 1), zstep = NTH / lpt;
   const bool zlane = zq < nq;
   auto zload = [&](int i) {
     float4 z = make_float4(-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F);
     if (zlane && i < i1) {
-      const float* zr = p.z_ws + ((int64_t)b * p.max_visual + i) * p.hp + hbeg;
-      if (vec) z = __ldcg(reinterpret_cast<const float4*>(zr) + zq);
-      else z.x = __ldcg(zr + zq);
-      if (rounds) {
-        if (zq + 32 < nq) z.y = __ldcg(zr + zq + 32);
-        if (zq + 64 < nq) z.z = __ldcg(zr + zq + 64);
-        if (zq + 96 < nq) z.w = __ldcg(zr + zq + 96);
+      const float* zr = p.z_ws + ((int64_t)b * p.max_visual + i) * p.hp + hbeg + 4 * zq;
+      if (vec) {
+        z = __ldcg(reinterpret_cast<const float4*>(zr));
+      } else {
+        z.x = __ldcg(zr);
+        if (4 * zq + 1 < hcnt) z.y = __ldcg(zr + 1);
+        if (4 * zq + 2 < hcnt) z.z = __ldcg(zr + 2);
+        if (4 * zq + 3 < hcnt) z.w = __ldcg(zr + 3);
       }
     }
     return z;
@@ -3908,13 +3905,12 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
         m4 = reinterpret_cast<const float4*>(sm.hM + hbeg)[zq];
         r4 = reinterpret_cast<const float4*>(sm.hInv + hbeg)[zq];
       } else {
-        m4.x = sm.hM[hbeg + zq];
-        r4.x = sm.hInv[hbeg + zq];
-        if (rounds) {  // heads past nq: weight 0
-          if (zq + 32 < nq) { m4.y = sm.hM[zq + 32]; r4.y = sm.hInv[zq + 32]; }
-          if (zq + 64 < nq) { m4.z = sm.hM[zq + 64]; r4.z = sm.hInv[zq + 64]; }
-          if (zq + 96 < nq) { m4.w = sm.hM[zq + 96]; r4.w = sm.hInv[zq + 96]; }
-        }
+        const float* hm = sm.hM + hbeg + 4 * zq;
+        const float* hi = sm.hInv + hbeg + 4 * zq;
+        m4.x = hm[0]; r4.x = hi[0];  // heads past hcnt: logit -inf, weight 0
+        if (4 * zq + 1 < hcnt) { m4.y = hm[1]; r4.y = hi[1]; }
+        if (4 * zq + 2 < hcnt) { m4.z = hm[2]; r4.z = hi[2]; }
+        if (4 * zq + 3 < hcnt) { m4.w = hm[3]; r4.w = hi[3]; }
       }
     }
     // Every lane of the group gets the token's score; lane r sends it to CTA
@@ -3924,11 +3920,9 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
     const unsigned key_a = smem_u32(key_s), bar_a = smem_u32(&sm.bar);
     auto score = [&](int i, const float4& z) {
       float a = fexp2_rel(z.x, m4.x) * r4.x;
-      if (vec || rounds) {
-        a = fmaf(fexp2_rel(z.y, m4.y), r4.y, a);
-        a = fmaf(fexp2_rel(z.z, m4.z), r4.z, a);
-        a = fmaf(fexp2_rel(z.w, m4.w), r4.w, a);
-      }
+      a = fmaf(fexp2_rel(z.y, m4.y), r4.y, a);
+      a = fmaf(fexp2_rel(z.z, m4.z), r4.z, a);
+      a = fmaf(fexp2_rel(z.w, m4.w), r4.w, a);
       for (int o = 1; o < lpt; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
       if (i >= i1) return;
       const float sc = a * inv_cnt;
