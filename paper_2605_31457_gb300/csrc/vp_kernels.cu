@@ -4047,10 +4047,23 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
       const float w = exp2_rel(tmx[k], tmh);
       a.x = fmaf(w, tov[k].x, a.x); a.y = fmaf(w, tov[k].y, a.y); a.z = fmaf(w, tov[k].z, a.z); a.w = fmaf(w, tov[k].w, a.w);
     }
-    for (int k = kSgTextSplits; tlive && tsg + TSG * k < ns; ++k) {
-      const float w = exp2_rel(__ldcg(tst + (int64_t)(TSG * k) * ST_N), tmh);
-      const float4 v = __ldcg(reinterpret_cast<const float4*>(tso + (int64_t)(TSG * k) * D));
-      a.x = fmaf(w, v.x, a.x); a.y = fmaf(w, v.y, a.y); a.z = fmaf(w, v.z, a.z); a.w = fmaf(w, v.w, a.w);
+#pragma unroll 1
+    for (int k0 = kSgTextSplits; TSG * k0 < ns; k0 += kSgTextSplits) {  // more splits: as many in flight again
+#pragma unroll
+      for (int k = 0; k < kSgTextSplits; ++k) {
+        const int o = TSG * (k0 + k);
+        tmx[k] = -CUDART_INF_F;
+        tov[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (tlive && tsg + o < ns) {
+          tmx[k] = __ldcg(tst + (int64_t)o * ST_N);
+          tov[k] = __ldcg(reinterpret_cast<const float4*>(tso + (int64_t)o * D));
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < kSgTextSplits; ++k) {
+        const float w = exp2_rel(tmx[k], tmh);
+        a.x = fmaf(w, tov[k].x, a.x); a.y = fmaf(w, tov[k].y, a.y); a.z = fmaf(w, tov[k].z, a.z); a.w = fmaf(w, tov[k].w, a.w);
+      }
     }
     for (int o = 1; o < TSG; o <<= 1) {
       a.x += __shfl_xor_sync(0xffffffffu, a.x, o);

@@ -228,6 +228,15 @@ def test_chunk_gather_short_value_table(vp, H, Hkv, batch):
             np.testing.assert_allclose(out[b][h], want, rtol=0, atol=2e-2)
 
 
+@pytest.mark.parametrize("H,Hkv,D", [(14, 2, 64), (28, 4, 128)])
+@pytest.mark.parametrize("text", [9000, 17000])
+def test_many_text_splits(vp, H, Hkv, D, text):
+    """One long text: more score splits than the fused kernel requests text
+    partials of at once."""
+    r = small(heads=H, kv_heads=Hkv, head_dim=D, batch=1, vis_len=(300,), vis_start=(13,), text_len=(text,))
+    Hn.check_all(vp, Hn.make_inputs(r), r.budget)
+
+
 def test_paged_cache(vp):
     r = small(batch=4, vis_len=(300, 577, 64, 1000), vis_start=(0, 13, 40, 0),
               text_len=(517, 70, 129, 33), paged=True, page_size=16)
