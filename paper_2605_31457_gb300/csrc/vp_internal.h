@@ -195,7 +195,16 @@ struct Plan {
 // 3857 tokens, 28 calls in a graph: 37 splits 344 us, 32 337, 24 308, 20 312,
 // 16 303, 12 312; 4 fp32 sequences of up to 2796 tokens (32 select CTAs): 19
 // splits 22.9 us a call, 16 22.8, 15 (one wave beside them) 14.9.
+// A call that runs by itself (a kernel of the caller's between two calls) pays
+// for the SMs left out: where the plan costs more than kBesideCost times the
+// whole GPU's by the costs below, it takes the whole GPU.  us a call, back to
+// back / by itself, on the SMs left and on all: 8 x 3857 tokens, 28/4 heads
+// 22.7 / 29.9 and 21.4 / 24.2; 9 x 4000 24.9 / 32.6 and 23.2 / 24.4; 8 x 7424,
+// 32/8 heads 46.9 / 58.2 and 43.5 / 50.5.  Below that the overlap is worth more:
+// 6 x 5000 (1.37) 17.9 / 27.6 and 23.2 / 24.0; 6 x 20480 (1.37) 39.5 / 52.4 and
+// 46.4 / 51.9; 5 x 9000 22.0 / 34.4 and 31.7 / 32.4.
 constexpr int kBesideSplits = 16, kBesideTiles = 18;
+constexpr double kBesideCost = 1.5;
 inline Plan make_plan(int batch, int Hkv, int D, int num_sms, int max_visual, int max_seq, int kept_cap,
                       int granularity, bool tc = false, bool beside = false) {
   const long long units = (long long)batch * Hkv;
@@ -231,12 +240,19 @@ inline Plan make_plan(int batch, int Hkv, int D, int num_sms, int max_visual, in
   }
   if (ns_hi < 1) ns_hi = 1;
   const double fixed = tc ? 6.0 * kTcWv : 12.0;
-  long long ns = 1;
-  double best = 0.0;
-  for (long long c = 1; c <= ns_hi; ++c) {
-    const double waves = (double)((units * c + score_slots - 1) / score_slots);
-    const double cost = waves * ((double)tiles / (double)c + fixed);
-    if (c == 1 || cost < best * (1.0 - 1e-9)) { best = cost; ns = c; }
+  auto cost = [&](long long c, long long on) {
+    return (double)((units * c + on - 1) / on) * ((double)tiles / (double)c + fixed);
+  };
+  auto best_of = [&](long long on) {
+    long long n = 1;
+    for (long long c = 2; c <= ns_hi; ++c)
+      if (cost(c, on) < cost(n, on) * (1.0 - 1e-9)) n = c;
+    return n;
+  };
+  long long ns = best_of(score_slots);
+  if (score_slots < slots) {
+    const long long whole = best_of(slots);
+    if (cost(ns, slots) > kBesideCost * cost(whole, slots)) ns = whole;
   }
   // Kept chunks of about 2048 rows, smaller (down to 256) while the gather
   // grid would not fill the GPU once (measured against 1024-row chunks and a

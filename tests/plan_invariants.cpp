@@ -140,7 +140,22 @@ int check_beside() {
                   }
             }
   std::printf("%lld plans beside a select kernel, %d violations\n", plans, fails - before);
-  return 0;
+  // Splits of such plans: on the SMs the select clusters leave, unless that
+  // would cost a call that runs by itself too much.
+  struct { int B, Hkv, D, mv, ms, tc, want; } cases[] = {
+      {1, 4, 128, 1296, 3920, 0, 16}, {4, 4, 128, 4096, 8255, 0, 15}, {6, 4, 128, 4096, 20543, 1, 8},
+      {8, 4, 128, 1296, 3920, 0, 9}, {9, 4, 128, 1296, 4059, 0, 8}, {8, 8, 64, 1296, 5059, 0, 4}, {8, 8, 128, 6400, 7487, 1, 4},
+  };
+  int bad = 0;
+  for (const auto& c : cases) {
+    const Plan pl = make_plan(c.B, c.Hkv, c.D, 152, c.mv, c.ms, 64, 0, c.tc != 0, true);
+    if (pl.ns != c.want) {
+      std::printf("FAIL splits beside a select kernel: B=%d Hkv=%d D=%d max_visual=%d max_seq=%d tc=%d: %d (want %d)\n", c.B,
+                  c.Hkv, c.D, c.mv, c.ms, c.tc, pl.ns, c.want);
+      ++bad;
+    }
+  }
+  return bad;
 }
 
 // The sets that calls take, whatever mix of streams, captures and failed
