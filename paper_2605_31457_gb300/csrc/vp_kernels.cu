@@ -1528,8 +1528,11 @@ __global__ void __launch_bounds__(kTcThreads, NS <= 3 ? 2 : 1) k_score_tc(const 
     // The workspace may still be read by the previous kernel: a thread waits
     // for it only before its first workspace write (visual logits, or the
     // split's partial), so splits of text tiles stream their whole range
-    // meanwhile.
-    bool ws_ok = p.ws_free;
+    // meanwhile.  (Two sets of outputs: no wait here, one at the end.  ws_ok
+    // starts as a constant: started from p.ws_free, the 16-head form's registers
+    // fall out so that it takes 70 us in place of 55, 64 sequences of N_v = 2304,
+    // 32/2 heads.)
+    bool ws_ok = false;
     int j = 0;          // text tiles seen
     for (int i = 0; i < n; ++i) {
       const int u = tr.u0 + i, sb = i & 1;
@@ -1547,7 +1550,7 @@ __global__ void __launch_bounds__(kTcThreads, NS <= 3 ? 2 : 1) k_score_tc(const 
       // A tile with visual rows writes logits: wait for the workspace first
       // (the same decision for every softmax thread).
       if (!ws_ok && u * kTcRows < sq.vs + sq.nv && u * kTcRows + kTcRows > sq.vs) {
-        pdl_wait();
+        if (!p.ws_free) pdl_wait();
         ws_ok = true;
       }
       const int pos = u * kTcRows + r;
@@ -1666,7 +1669,7 @@ __global__ void __launch_bounds__(kTcThreads, NS <= 3 ? 2 : 1) k_score_tc(const 
       }
     }
     wg_sync();
-    if (!ws_ok) pdl_wait();
+    if (!ws_ok && !p.ws_free) pdl_wait();
     const int64_t rec0 = ((int64_t)b * H + g * G) * p.nsp_max + s;  // split slot of head 0
     if (r < G) {
       const int h = r;
