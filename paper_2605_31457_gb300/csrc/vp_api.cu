@@ -294,17 +294,16 @@ vp_status vp_decode_step(vp_ctx* ctx, int32_t batch, const void* q,
   p.hp = ctx->lay.hp;
   p.nsp_max = ctx->lay.nsp_max;
   p.nk_max = ctx->lay.nk_max;
-  if (!vp::plan_step(p, ctx->num_sms, kept_cap, budget->granularity, ctx->score_path, ctx->lay.o_set2 != 0))
-    return fail(ctx, VP_ERR_UNSUPPORTED, "vp_decode_step: the tcgen05 score kernel (VP_SCORE_TC) cannot serve this "
-                "call (needs bf16, head_dim 128, G <= 16, pages of >= 8 tokens, a tensor-descriptor layout)");
-  p.mt_o = ctx->mt_o; p.mt_st = ctx->mt_st; p.hmax = ctx->hmax;
   if (ctx->diag_n_act || ctx->diag_bits) {
     memcpy(&p.act_delta_bits, &ctx->diag_delta, sizeof(float));
     p.n_act = ctx->diag_n_act;
     p.act_bits = ctx->diag_bits;
     p.act_words = (c.max_visual + 31) / 32;
   }
-  p.fused = vp::select_kind(p, kept_cap);
+  if (!vp::plan_step(p, ctx->num_sms, kept_cap, budget->granularity, ctx->score_path, ctx->lay.o_set2 != 0))
+    return fail(ctx, VP_ERR_UNSUPPORTED, "vp_decode_step: the tcgen05 score kernel (VP_SCORE_TC) cannot serve this "
+                "call (needs bf16, head_dim 128, G <= 16, pages of >= 8 tokens, a tensor-descriptor layout)");
+  p.mt_o = ctx->mt_o; p.mt_st = ctx->mt_st; p.hmax = ctx->hmax;
 
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   take_set(ctx, p, st);

@@ -188,7 +188,7 @@ struct Plan {
 
 // tc: the score splits are for the tensor-core kernel (128-row tiles).
 // beside: the score kernel runs beside the previous call's select kernel (a
-// context with two sets of its outputs).  It then has that kernel's time to
+// context with two sets of its outputs); 0 if not.  It then has that kernel's time to
 // itself, on the other SMs, while every split lengthens the select kernel's
 // merges: at most kBesideSplits splits, or as many as keep kBesideTiles tiles a
 // CTA, on the SMs the select clusters leave.  Measured, B = 1, 28/4 heads,
@@ -196,17 +196,20 @@ struct Plan {
 // 16 303, 12 312; 4 fp32 sequences of up to 2796 tokens (32 select CTAs): 19
 // splits 22.9 us a call, 16 22.8, 15 (one wave beside them) 14.9.
 // A call that runs by itself (a kernel of the caller's between two calls) pays
-// for the SMs left out: where the plan costs more than kBesideCost times the
+// for the SMs left out: where the plan costs more than `beside` times the
 // whole GPU's by the costs below, it takes the whole GPU.  us a call, back to
 // back / by itself, on the SMs left and on all: 8 x 3857 tokens, 28/4 heads
 // 22.7 / 29.9 and 21.4 / 24.2; 9 x 4000 24.9 / 32.6 and 23.2 / 24.4; 8 x 7424,
 // 32/8 heads 46.9 / 58.2 and 43.5 / 50.5.  Below that the overlap is worth more:
 // 6 x 5000 (1.37) 17.9 / 27.6 and 23.2 / 24.0; 6 x 20480 (1.37) 39.5 / 52.4 and
-// 46.4 / 51.9; 5 x 9000 22.0 / 34.4 and 31.7 / 32.4.
+// 46.4 / 51.9; 5 x 9000 22.0 / 34.4 and 31.7 / 32.4.  A call of three kernels has
+// less to gain, its gather kernel takes the whole GPU in between: 4 x 4352 at 20%
+// (1.16) 18.3 / 27.0 and 24.3 / 25.9, but 6 x 6400 with diagnostics (1.36) 37.8 /
+// 39.7 and 32.5 / 33.7, with a top-p budget 36.1 / 42.6 and 34.6 / 37.1.
 constexpr int kBesideSplits = 16, kBesideTiles = 18;
-constexpr double kBesideCost = 1.5;
+constexpr double kBesideCost = 1.5, kBesideCost3 = 1.25;  // calls of two and of three kernels
 inline Plan make_plan(int batch, int Hkv, int D, int num_sms, int max_visual, int max_seq, int kept_cap,
-                      int granularity, bool tc = false, bool beside = false) {
+                      int granularity, bool tc = false, double beside = 0.0) {
   const long long units = (long long)batch * Hkv;
   const int TR = tc ? kTcRows : 32;
   // Fixed-weight splits sized for the longest sequence (tiles wholly inside
@@ -224,7 +227,7 @@ inline Plan make_plan(int batch, int Hkv, int D, int num_sms, int max_visual, in
   int cl = 1;
   while (cl < 8 && sel * cl * 2 <= num_sms) cl *= 2;
   const long long slots = 2LL * num_sms;
-  const long long score_slots = beside && sel * cl <= num_sms / 2 ? slots - 2 * sel * cl : slots;
+  const long long score_slots = beside > 0.0 && sel * cl <= num_sms / 2 ? slots - 2 * sel * cl : slots;
   // Split count: minimise (waves of CTAs) x (tiles per CTA + a fixed cost per
   // CTA for its start, its pipeline fill and its partial), keeping a minimum
   // of work per CTA; the smaller count wins a tie.  The costs were measured
@@ -232,7 +235,7 @@ inline Plan make_plan(int batch, int Hkv, int D, int num_sms, int max_visual, in
   // kernel, about 6 weight units of 128 rows for the tensor-core kernel.
   long long ns_hi = tiles / (tc ? 2 * kTcWv : 8);
   if (ns_hi > kNsMax) ns_hi = kNsMax;
-  if (beside) {
+  if (beside > 0.0) {
     const long long units_per = tc ? 2 * kTcWv * kBesideTiles / 8 : kBesideTiles;  // as 8 tiles to 2 K-only ones above
     const long long least = (tiles + units_per - 1) / units_per;
     const long long cap = least > kBesideSplits ? least : kBesideSplits;
@@ -252,7 +255,7 @@ inline Plan make_plan(int batch, int Hkv, int D, int num_sms, int max_visual, in
   long long ns = best_of(score_slots);
   if (score_slots < slots) {
     const long long whole = best_of(slots);
-    if (cost(ns, slots) > kBesideCost * cost(whole, slots)) ns = whole;
+    if (cost(ns, slots) > beside * cost(whole, slots)) ns = whole;
   }
   // Kept chunks of about 2048 rows, smaller (down to 256) while the gather
   // grid would not fill the GPU once (measured against 1024-row chunks and a
@@ -298,11 +301,11 @@ inline int split_floor(const Plan& pl, int batch, int Hkv, int num_sms, bool tc,
 // keeps the splits it has on the whole GPU (paged, 8-token pages, 8 sequences
 // of 65536 tokens, one kv-head: 22 splits of 33 tiles, 38 of 19 fit).
 inline Plan step_plan(int batch, int Hkv, int D, int num_sms, int max_visual, int max_seq, int kept_cap,
-                      int granularity, bool tc, bool beside, int paged, int page_size) {
-  for (;; beside = false) {
+                      int granularity, bool tc, double beside, int paged, int page_size) {
+  for (;; beside = 0.0) {
     Plan pl = make_plan(batch, Hkv, D, num_sms, max_visual, max_seq, kept_cap, granularity, tc, beside);
     pl.split_w = split_floor(pl, batch, Hkv, num_sms, tc, pl.split_w);
-    if (!beside || page_ids_fit(paged, page_size, max_seq, pl.ns, pl.split_w, tc)) return pl;
+    if (beside == 0.0 || page_ids_fit(paged, page_size, max_seq, pl.ns, pl.split_w, tc)) return pl;
   }
 }
 
@@ -397,8 +400,9 @@ inline WsLayout ws_layout(int batch, int H, int Hkv, int D, int max_visual, int 
   for (int bb = 1; bb <= batch; ++bb)
     for (int tc = 0; tc < 2; ++tc)
       for (int gran = 0; gran < (second_set ? 2 : 1); ++gran)
-        for (int beside = 0; beside < (second_set ? 2 : 1); ++beside) {
-          const Plan pl = make_plan(bb, Hkv, D, num_sms, max_visual, max_seq, 0, gran, tc != 0, beside != 0);
+        for (double beside : {0.0, kBesideCost, kBesideCost3}) {
+          if (beside > 0.0 && !second_set) continue;
+          const Plan pl = make_plan(bb, Hkv, D, num_sms, max_visual, max_seq, 0, gran, tc != 0, beside);
           if (pl.ns > w.nsp_max) w.nsp_max = pl.ns;
         }
   const size_t B = (size_t)batch, G = (size_t)(H / Hkv);
@@ -507,8 +511,12 @@ inline int select_kind(const StepParams& p, int kept_cap) {
 // kernel was faster, above both the tensor-core kernel).
 // path: 0 the choice above, 1 never the tensor-core kernel, 2 only it
 // (false when it cannot serve the call).
-inline bool plan_step(StepParams& p, int num_sms, int kept_cap, int granularity, int path = 0, bool beside = false) {
+// two_sets: the context has two sets of the score kernels' outputs.
+inline bool plan_step(StepParams& p, int num_sms, int kept_cap, int granularity, int path = 0, bool two_sets = false) {
   p.num_sms = num_sms;
+  p.cl = make_plan(p.B, p.Hkv, p.D, num_sms, p.max_visual, p.max_seq, kept_cap, granularity).cl;
+  p.fused = select_kind(p, kept_cap);
+  const double beside = !two_sets ? 0.0 : p.fused == 1 ? kBesideCost : kBesideCost3;
   const long long w_tc = 2LL * ((p.max_seq + kTcRows - 1) / kTcRows) - p.max_visual / kTcRows;
   const bool eligible = tc_eligible(p.dtype, p.D, p.G, p.paged, p.page_size);
   const bool tc = path == 2 ? eligible
