@@ -1720,9 +1720,13 @@ __global__ void __launch_bounds__(kTcThreads, NS <= 3 ? 2 : 1) k_score_tc(const 
 // a thread keeps eight rows in flight: the indices of its next eight
 // rows, then their pages, then their data, then the stores (one row at a time
 // before).  8 x 4 x 2561 rows of 256 bytes, read and written: 12.5 -> 11.1 us.
+// Rows of 128 bytes are four to a thread (U): with eight the empty half cost
+// more than the rest gained, 32 x 8 x 2561 rows 41.2 -> 47.7 us, with four 36.3.
 // ---------------------------------------------------------------------------
 constexpr int kCompactRows = 128;  // destination rows per CTA
 
+// U: rows of a thread in flight (kCompactRows * 16-byte pieces per row / 256, at most 8).
+template <int U>
 __global__ void __launch_bounds__(256) k_compact(const __grid_constant__ CompactParams c) {
   // kept_idx / kept_count may come from the previous kernel.  No early
   // trigger: the next call may read the caches written here before its own
@@ -1744,7 +1748,6 @@ __global__ void __launch_bounds__(256) k_compact(const __grid_constant__ Compact
   const char* src = static_cast<const char*>(c.src.data);
   char* dst = static_cast<char*>(c.dst);
   const int piece = threadIdx.x % ppr;
-  constexpr int U = 8;  // rows of a thread in flight
   for (int t0 = r0 + threadIdx.x / ppr; t0 < r1; t0 += U * rpi) {
     int pos[U], page[U];
 #pragma unroll
@@ -4387,7 +4390,7 @@ cudaError_t launch_compact(const CompactParams& c, cudaStream_t st) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_compact, c);
+  return cudaLaunchKernelEx(&cfg, c.D * c.esz <= 128 ? k_compact<4> : k_compact<8>, c);
 }
 
 // Dynamic shared memory of k_selgat: the score keys and the cut's two
