@@ -4260,9 +4260,15 @@ cudaError_t launch_gather_td(const StepParams& p, cudaStream_t st) {
     // sequences, 8 kv-heads, the call with eight / four warps: 1280 of 6400 229 /
     // 241 us, 460 of 2304 122 / 134, 288 of 576 85 / 90, 115 of 576 74.4 / 76.8;
     // one or two steps per warp, 29 of 576: 71.4 / 69.3).  Three CTAs per SM
-    // (fewer registers) where that saves a wave (40 sequences, 1250 of 5000: 144
-    // us, two per SM 153; 1280 of 6400 runs two waves either way: 227 us, three
-    // per SM 242).
+    // (80 registers, a few words spilled) where that saves a wave (40 sequences,
+    // 1250 of 5000: 144 us, two per SM 153; 1280 of 6400 runs two waves either
+    // way: 227 us, three per SM 242).  64 dimensions, eight / four warps: 152
+    // sequences, 1152 of 2304 236 / 241 us, 40 of 461 77.0 / 77.9, 64 of 461
+    // 112.2 / 109.7; 16 heads per kv-head 91.8 / 104.
+    // More than 8 heads per kv-head, 128 dimensions: eight warps (160 registers)
+    // are one CTA per SM, so only where four-warp CTAs would all be resident
+    // (1152 of 2304, 304 CTAs 144 / 157 us; 608: 282 / 264) and its waves are
+    // full to three quarters (115 of 2304, 160 CTAs 100 / 93.5).
     // Several chunks: four warps take about a tenth less time a byte (2048 CTAs,
     // 8192 of 16384: 616 us, eight warps 632), and a grid that the SMs hold at
     // once stays with them (320 CTAs, 6000 of 12000: 114, 120; 640, 3000 of
@@ -4271,7 +4277,10 @@ cudaError_t launch_gather_td(const StepParams& p, cudaStream_t st) {
     // four warps 295; 1536, 5734 of 16384: 568, 575).  Measured at D = 128 only.
     const long long n = (long long)p.nc * p.Hkv * p.B, two = 2LL * p.num_sms, three = 3LL * p.num_sms;
     if (p.nk == 1 && p.kept_cap >= kGmWide) {
-      if (p.G > 8) return launch_gather_mma<D, 2, 8, 1>(p, grid, st);
+      const long long one = p.num_sms;
+      if (p.G > 8)
+        return D == 64 || (n <= three && 4 * n >= 3 * one * ((n + one - 1) / one)) ? launch_gather_mma<D, 2, 8, 1>(p, grid, st)
+                                                                                   : launch_gather_mma<D, 2, 4, 3>(p, grid, st);
       return (n + three - 1) / three < (n + two - 1) / two ? launch_gather_mma<D, 1, 8, 3>(p, grid, st)
                                                            : launch_gather_mma<D, 1, 8, 2>(p, grid, st);
     }

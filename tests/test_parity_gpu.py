@@ -159,6 +159,17 @@ def test_chunk_gather_long_lists(vp, paged):
         Hn.check_all(vp, inp, budget, seqs=(0, 7, batch - 1))
 
 
+@pytest.mark.parametrize("batch", [100, 152, 153])
+def test_chunk_gather_many_heads(vp, batch):
+    """16 query heads per kv-head, one CTA per (sequence, kv-head): the four-warp
+    form where one eight-warp CTA per SM leaves a wave half empty (200 CTAs) or
+    the grid does not fit once (459), the eight-warp form between (304)."""
+    kv = 3 if batch == 153 else 2
+    vis = tuple(130 + i for i in range(batch))
+    r = small(heads=16 * kv, kv_heads=kv, batch=batch, vis_len=vis, vis_start=(1,) * batch, text_len=(20,) * batch)
+    Hn.check_all(vp, Hn.make_inputs(r), dict(mode=O.FIXED_RATIO, tau=0.1, ratio_ppm=950_000), seqs=(0, 7, batch - 1))
+
+
 def test_chunk_gather_two_long_chunks(vp):
     """Two chunks of more than 1024 rows (768 CTAs: the eight-warp form, its
     waves fuller than the four-warp ones), the last sequences' spans shorter."""
