@@ -204,10 +204,11 @@ struct Plan {
 // 6 x 5000 (1.37) 17.9 / 27.6 and 23.2 / 24.0; 6 x 20480 (1.37) 39.5 / 52.4 and
 // 46.4 / 51.9; 5 x 9000 22.0 / 34.4 and 31.7 / 32.4.  A call of three kernels has
 // less to gain, its gather kernel takes the whole GPU in between: 4 x 4352 at 20%
-// (1.16) 18.3 / 27.0 and 24.3 / 25.9, but 6 x 6400 with diagnostics (1.36) 37.8 /
-// 39.7 and 32.5 / 33.7, with a top-p budget 36.1 / 42.6 and 34.6 / 37.1.
+// (1.16) 18.3 / 26.7 and 24.4 / 26.2, but 4 x 8192 with diagnostics (1.20) 32.6 /
+// 36.0 and 32.1 / 34.3, 4 x 3328, 32/8 heads (1.21) 26.9 / 29.4 and 25.7 / 27.9,
+// 6 x 6400 (1.36) 37.8 / 39.7 and 32.5 / 33.7.
 constexpr int kBesideSplits = 16, kBesideTiles = 18;
-constexpr double kBesideCost = 1.5, kBesideCost3 = 1.25;  // calls of two and of three kernels
+constexpr double kBesideCost = 1.5, kBesideCost3 = 1.18;  // calls of two and of three kernels
 inline Plan make_plan(int batch, int Hkv, int D, int num_sms, int max_visual, int max_seq, int kept_cap,
                       int granularity, bool tc = false, double beside = 0.0) {
   const long long units = (long long)batch * Hkv;
