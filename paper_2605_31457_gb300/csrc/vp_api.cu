@@ -384,8 +384,7 @@ vp_status vp_decode_gather(vp_ctx* ctx, int32_t batch, const void* q,
   p.kept_cap = kept_cap;
   p.kept_count = const_cast<int32_t*>(kept_count);
   p.out = out;
-  p.gpart_o = ctx->gpart_o; p.gpart_st = ctx->gpart_st; p.tickets = ctx->tickets; p.err = ctx->err;
-  p.mt_o = ctx->mt_o; p.mt_st = ctx->mt_st; p.hmax = ctx->hmax;
+  p.err = ctx->err;
   const vp::Plan pl = vp::gather_plan(batch, Hkv, D, ctx->num_sms, c.max_visual, c.max_seq, kept_cap, granularity,
                                       p.paged, p.page_size);
   p.hp = ctx->lay.hp;

@@ -5,25 +5,32 @@
 //             go to the workspace; visual and text tokens keep separate online
 //             softmax statistics at tau = 1 and at tau (the two sums of Eq. 6);
 //             text tokens also accumulate their unnormalised attention output.
-//   k_select  per sequence (or per kv-head), a cluster of up to 8 CTAs: merges
+//   k_selgat  per sequence (or per kv-head), a cluster of up to 8 CTAs: merges
 //             the split statistics into the visual mass per head (Eq. 5) and
 //             its head-max (Sec. 4.3) and the budget K_t (Eq. 7 + clamp of
 //             Sec. 5.2); every CTA computes the importance score S_i (Eq. 2) of
-//             a slice of the visual tokens into rank 0's shared memory, which
-//             then finds the Top-K_t set (Eq. 3) by radix select, ties to the
-//             lower index, emitted in ascending order.
-//   k_gather  per (sequence, kv-head): CTA c attends over chunk c of the kept
-//             visual tokens, reading V only for them, and merges slice c of the
-//             text partials; the last CTA to finish combines everything in
-//             log-sum-exp form and writes the output (Sec. 4.2, Sec. 5.7).
+//             a slice of the visual tokens into every CTA's shared memory and
+//             finds the Top-K_t set (Eq. 3) by radix select, ties to the lower
+//             index, emitted in ascending order.  For short kept sets each CTA
+//             then attends over its slice of the output dimensions and the call
+//             ends here; otherwise only rank 0 cuts and a gather kernel follows.
+//   k_select  the same selection for the calls that kernel does not serve (more
+//             than 4096 visual tokens, top-p budgets, diagnostics); rank 0 cuts.
+//   k_gather, k_gather_mma, k_gather_slice
+//             per (sequence, kv-head): CTA c attends over chunk c (or slice c of
+//             the dimensions) of the kept visual tokens, reading V only for
+//             them, and merges a slice of the text partials; the chunks' last
+//             CTA to finish combines everything in log-sum-exp form and writes
+//             the output (Sec. 4.2, Sec. 5.7).
+//   k_merge   layers after the anchor layer: combines the score splits.
 //
 // Logits are carried in log2 units (z * log2 e) so that every exponential is
 // one exp2f: exp(z - m) = exp2(z2 - m2), exp((z - m) / tau) = exp2((z2 - m2) / tau).
 //
 // Every kernel may be launched as a programmatic dependent of the preceding
 // kernel on the stream: it reads nothing that kernel writes before
-// griddepcontrol.wait.  The slice gather kernel reads the call's inputs and
-// the score kernel's partials before its wait: the select kernel between them
+// griddepcontrol.wait.  The gather kernels read the call's inputs and may read
+// the score kernel's partials before their wait: the select kernel between them
 // lets its dependents start only after its own wait on the score kernel, so
 // both are complete by then.  A score kernel waits for the previous kernel
 // before its first write; with two sets of the score kernels' outputs
@@ -178,8 +185,8 @@ __device__ __forceinline__ void ldsm_x4_t(unsigned addr, uint32_t& r0, uint32_t&
 }
 
 // Asynchronous 4-byte store to the shared memory of CTA `rank` of the cluster
-// (only in a launch with a cluster), counted by that CTA's mbarrier; addr and bar are this CTA's own addresses of
-// the same variables.
+// (only in a launch with a cluster), counted by that CTA's mbarrier; addr and
+// bar are this CTA's own addresses of the same variables.
 __device__ __forceinline__ void st_async_u32(unsigned addr, uint32_t v, unsigned bar, int rank) {
   asm volatile(
       "{\n .reg .b32 a, m;\n mapa.shared::cluster.u32 a, %0, %3;\n mapa.shared::cluster.u32 m, %2, %3;\n"
@@ -2412,10 +2419,10 @@ __global__ void __launch_bounds__(NTH, 1) k_select(const __grid_constant__ StepP
   // lane are in flight, and a reduce-scatter over the LPT lanes leaves every
   // lane whole-token sums to emit.  The activity words are in the loop only with
   // diagnostics on (tested per token instead, the 1024-thread form took 24.6 us
-  // at N_v = 6400 and 43.0 at 16384, B = 64; now 22.5 and 38.9).  More than 32 heads (MORE): further rounds of
-  // 32, a form of its own (40 / 64 heads, the call with one word per load and
-  // now: 32 sequences of N_v = 6400, 158 / 171 and 126 / 116 us; 8 sequences
-  // 68 / 78 and 53 / 55).
+  // at N_v = 6400 and 43.0 at 16384, B = 64; now 22.5 and 38.9).  More than 32
+  // heads (MORE): further rounds of 32, a form of its own (40 / 64 heads, the call
+  // with one word per load and now: 32 sequences of N_v = 6400, 158 / 171 and
+  // 124 / 116 us).
   auto wide_loop = [&](auto lpt_tag, auto more_tag, auto diag_tag) {
     constexpr int LPT = decltype(lpt_tag)::value, TPI = 32 / LPT, V = 8;
     constexpr bool MORE = decltype(more_tag)::value;
@@ -2554,9 +2561,7 @@ __global__ void __launch_bounds__(NTH, 1) k_select(const __grid_constant__ StepP
   // 4. Radix select of the K-th largest key, 8 bits per pass from the top;
   //    lanes holding the same digit add to the histogram once per warp.  One
   //    barrier per pass: every warp scans the finished histogram itself, and
-  //    pass p clears the buffer of pass p - 2 for pass p + 1.  (The same cut
-  //    as radix_cut, written out here: at 1024 threads this kernel runs at the
-  //    64-register limit, and with the shared routine it spilled more.)
+  //    pass p clears the buffer of pass p - 2 for pass p + 1.
   uint32_t theta = 0;
   unsigned krem = 0, n_theta = 0;  // keys equal to theta: to keep, in total
   if (topp) {
@@ -4042,8 +4047,8 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
     else *reinterpret_cast<uint4*>(vst + off) = make_uint4(0u, 0u, 0u, 0u);
   }
   asm volatile("cp.async.commit_group;\n" ::: "memory");
-  // The text part, while the copies are in flight: sum exp2(m_s - m_text) * o_s over the splits, then over
-  //     the element's four split groups.
+  // The text part, while the copies are in flight: sum exp2(m_s - m_text) * o_s
+  // over the splits, then over the element's split groups.
   if constexpr (GATHER) {
     const float tmh = sm.hMt[th];
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
