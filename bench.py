@@ -8,17 +8,19 @@ step.  A step is one vp_decode_step call per layer (each layer acting as its
 own anchor layer), i.e. the whole five-stage hot path over every layer and
 sequence.  This is the largest of the synthetic workloads shaped like the
 paper's Qwen decoders (Sec. 5.1, App. B.1); the others are measured too and
-reported under `configs`.
+reported in a table of their own on the standard error.
 
 Prints one JSON line (rank 0).  `value` is decode steps per second with the
 caches resident in HBM (per-step CUDA graphs of the layer calls, timed with
 CUDA events); `e2e` is the same metric through the C ABI with the step's
 queries and appended K/V copied in from pinned host memory and the results
 copied back; `roofline` is the score kernel's (it moves the step's bytes);
-`configs` holds the same figures for the tiny fp32 reference, the B = 1
-Qwen2.5-VL-7B-shaped decode, the batched paged serving batch and the 20
-points of the visual-length / retention sweep, each with its own clocks;
-`cpu_baseline` is the CPU oracle on the host cores over a bounded sample.
+`cpu_baseline` is the CPU oracle on the host cores over a bounded sample.  The
+line stays short enough to be read from the end of a log; one JSON line on the
+standard error, {"configs": ...}, holds the same figures for the tiny fp32
+reference, the B = 1 Qwen2.5-VL-7B-shaped decode, the batched paged serving
+batch and the 20 points of the visual-length / retention sweep, each with its
+own clocks.
 `--impl reference` times the CPU oracle instead (rank 0, host cores).
 """
 
@@ -919,8 +921,7 @@ def run_ours(args, rank, world, local):
             line[k] = res[k]
     if "pipeline" in line:
         line["config"]["pipeline"] = line.pop("pipeline")
-    if not args.no_configs and world == 1:
-        line["configs"] = run_configs(args, dev, world)
+    table = run_configs(args, dev, world) if not args.no_configs and world == 1 else None
     if not args.no_cpu_baseline and rank == 0 and world == 1:
         pool = OraclePool(r, S, cpu_caches(r, nbuf), args.cpu_workers)
         try:
@@ -934,8 +935,16 @@ def run_ours(args, rank, world, local):
         finally:
             pool.close()
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        report(line, table)
     return 0
+
+
+def report(line, table):
+    """The result: one line on the standard output, the table of the other
+    workloads (if measured) before it on the standard error."""
+    if table is not None:
+        print(json.dumps({"configs": table}), file=sys.stderr, flush=True)
+    print(json.dumps(line), flush=True)
 
 
 def run_layer_calls(args):

@@ -1,5 +1,8 @@
 """Host logic of bench.py on the CPU: the algorithmic byte count of a layer
-call, the workload table and the clock summary.  No GPU work runs here."""
+call, the workload table, the clock summary and the printed result.  No GPU
+work runs here."""
+
+import json
 
 import pytest
 
@@ -114,3 +117,11 @@ def test_oracle_pool_times_whole_steps():
         assert small.step(0) > 0
     finally:
         small.close()
+
+
+def test_report_prints_one_line_and_the_table_apart(capsys):
+    bench.report({"metric": "m", "value": 1.5}, {"tiny": {"steps_per_s": 2.0}})
+    bench.report({"metric": "m", "value": 2.5}, None)
+    got = capsys.readouterr()
+    assert [json.loads(x) for x in got.out.splitlines()] == [{"metric": "m", "value": 1.5}, {"metric": "m", "value": 2.5}]
+    assert [json.loads(x) for x in got.err.splitlines()] == [{"configs": {"tiny": {"steps_per_s": 2.0}}}]
