@@ -3701,7 +3701,11 @@ __device__ __forceinline__ unsigned sg_voff(int j, int c) {
 // GATHER = false: the selection alone (steps 1, 2b and 3), for calls whose
 // gather runs as its own kernel; it also writes every head's largest logit
 // (p.hmax) for that kernel.
-template <typename T, int D, int GM, bool GATHER = true>
+// VEC: the selection's heads start and end on 16-byte pieces of a logit row; a
+// form of its own, as the other form's loads would lengthen the code that every
+// launch runs about once (28-call step of the B = 1 decode 286 us, with them
+// apart 277).
+template <typename T, int D, int GM, bool VEC, bool GATHER = true>
 __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ StepParams p) {
   constexpr int NTH = kSgThreads, NW = kSgWarps;
   constexpr bool BF = sizeof(T) == 2;
@@ -3788,7 +3792,6 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
   const int i0 = min(nv, rank * per), i1 = min(nv, i0 + per);
   const int hbeg = p.granularity ? gsel * G : 0;
   const int hcnt = p.granularity ? G : H;
-  const bool vec = (hbeg & 3) == 0 && (hcnt & 3) == 0;
   const int nq = (hcnt + 3) >> 2;  // lanes a token needs (at most 128 heads: 32)
   const int rsh = nq <= 1 ? 0 : 32 - __clz(nq - 1), lpt = 1 << rsh;
   const int zq = tid & (lpt - 1), zstep = NTH / lpt;
@@ -3797,7 +3800,7 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
     float4 z = make_float4(-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F);
     if (zlane && i < i1) {
       const float* zr = p.z_ws + ((int64_t)b * p.max_visual + i) * p.hp + hbeg + 4 * zq;
-      if (vec) {
+      if constexpr (VEC) {
         z = __ldcg(reinterpret_cast<const float4*>(zr));
       } else {
         z.x = __ldcg(zr);
@@ -3912,7 +3915,7 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
   {
     float4 m4 = make_float4(0.f, 0.f, 0.f, 0.f), r4 = m4;  // this lane's heads: maxima, 1 / normalisers
     if (zlane) {
-      if (vec) {
+      if constexpr (VEC) {
         m4 = reinterpret_cast<const float4*>(sm.hM + hbeg)[zq];
         r4 = reinterpret_cast<const float4*>(sm.hInv + hbeg)[zq];
       } else {
@@ -4052,28 +4055,23 @@ __global__ void __launch_bounds__(kSgThreads) k_selgat(const __grid_constant__ S
   if constexpr (GATHER) {
     const float tmh = sm.hMt[th];
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int k = 0; k < kSgTextSplits; ++k) {
-      if (TSG * k >= ns) break;  // uniform
-      const float w = exp2_rel(tmx[k], tmh);
-      a.x = fmaf(w, tov[k].x, a.x); a.y = fmaf(w, tov[k].y, a.y); a.z = fmaf(w, tov[k].z, a.z); a.w = fmaf(w, tov[k].w, a.w);
-    }
 #pragma unroll 1
-    for (int k0 = kSgTextSplits; TSG * k0 < ns; k0 += kSgTextSplits) {  // more splits: as many in flight again
-#pragma unroll
-      for (int k = 0; k < kSgTextSplits; ++k) {
-        const int o = TSG * (k0 + k);
-        tmx[k] = -CUDART_INF_F;
-        tov[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (tlive && tsg + o < ns) {
-          tmx[k] = __ldcg(tst + (int64_t)o * ST_N);
-          tov[k] = __ldcg(reinterpret_cast<const float4*>(tso + (int64_t)o * D));
-        }
-      }
+    for (int k0 = 0;;) {
 #pragma unroll
       for (int k = 0; k < kSgTextSplits; ++k) {
         const float w = exp2_rel(tmx[k], tmh);
         a.x = fmaf(w, tov[k].x, a.x); a.y = fmaf(w, tov[k].y, a.y); a.z = fmaf(w, tov[k].z, a.z); a.w = fmaf(w, tov[k].w, a.w);
+      }
+      k0 += kSgTextSplits;
+      if (TSG * k0 >= ns) break;  // uniform
+#pragma unroll
+      for (int k = 0; k < kSgTextSplits; ++k) {  // more splits: as many in flight again
+        const int o = TSG * (k0 + k);
+        tmx[k] = -CUDART_INF_F;
+        if (tlive && tsg + o < ns) {
+          tmx[k] = __ldcg(tst + (int64_t)o * ST_N);
+          tov[k] = __ldcg(reinterpret_cast<const float4*>(tso + (int64_t)o * D));
+        }
       }
     }
     for (int o = 1; o < TSG; o <<= 1) {
@@ -4416,16 +4414,22 @@ size_t selgat_smem_bytes(int max_visual, int dtype, int W = 64) {
   return keys > stage ? keys : stage;
 }
 
+// k_selgat's VEC: every selection's heads are whole 16-byte pieces.
+bool selgat_vec(const StepParams& p) { return ((p.granularity ? p.G : p.H) & 3) == 0; }
+
 template <typename T, int D>
 cudaError_t launch_selgat_td(const StepParams& p, dim3 grid, size_t smem, cudaStream_t st) {
-  if (p.G <= 4) return launch_ex(k_selgat<T, D, 4>, grid, dim3(kSgThreads), smem, st, p.cl, p);
-  return launch_ex(k_selgat<T, D, 8>, grid, dim3(kSgThreads), smem, st, p.cl, p);
+  const bool vec = selgat_vec(p);
+  if (p.G <= 4)
+    return launch_ex(vec ? k_selgat<T, D, 4, true> : k_selgat<T, D, 4, false>, grid, dim3(kSgThreads), smem, st, p.cl, p);
+  return launch_ex(vec ? k_selgat<T, D, 8, true> : k_selgat<T, D, 8, false>, grid, dim3(kSgThreads), smem, st, p.cl, p);
 }
 
 cudaError_t launch_select(const StepParams& p, cudaStream_t st) {
   const dim3 grid(p.cl, p.granularity ? p.Hkv : 1, p.B);
   if (p.fused == 2)
-    return launch_ex(k_selgat<__nv_bfloat16, 128, 8, false>, grid, dim3(kSgThreads),
+    return launch_ex(selgat_vec(p) ? k_selgat<__nv_bfloat16, 128, 8, true, false>
+                                   : k_selgat<__nv_bfloat16, 128, 8, false, false>, grid, dim3(kSgThreads),
                      selgat_smem_bytes(p.max_visual, 0), st, p.cl, p);
   if (p.fused == 1) {
     const size_t smem = selgat_smem_bytes(p.max_visual, p.dtype, selgat_slice_dims(p));
@@ -4534,24 +4538,22 @@ cudaError_t configure_kernels(int max_visual, int H, int nsp_max) {
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&attr, k);
     if (e == cudaSuccess && attr.maxDynamicSharedSizeBytes < need) e = set_smem(k, need);
   }
-  {
+  auto raise = [&](void (*k)(StepParams), int need) {
     cudaFuncAttributes attr;
-    const int need = (int)selgat_smem_bytes(max_visual, 0);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&attr, k_selgat<__nv_bfloat16, 128, 8, false>);
-    if (e == cudaSuccess && attr.maxDynamicSharedSizeBytes < need) e = set_smem(k_selgat<__nv_bfloat16, 128, 8, false>, need);
-  }
-  void (*const selgat[2][4])(StepParams) = {
-      {k_selgat<__nv_bfloat16, 128, 4>, k_selgat<__nv_bfloat16, 128, 8>, k_selgat<__nv_bfloat16, 64, 4>,
-       k_selgat<__nv_bfloat16, 64, 8>},
-      {k_selgat<float, 128, 4>, k_selgat<float, 128, 8>, k_selgat<float, 64, 4>, k_selgat<float, 64, 8>}};
-  for (int dt = 0; dt < 2; ++dt) {
-    const int need_sg = (int)selgat_smem_bytes(max_visual, dt, dt == 0 ? kSgMaxW : 64);
-    for (void (*k)(StepParams) : selgat[dt]) {
-      cudaFuncAttributes attr;
-      if (e == cudaSuccess) e = cudaFuncGetAttributes(&attr, k);
-      if (e == cudaSuccess && attr.maxDynamicSharedSizeBytes < need_sg) e = set_smem(k, need_sg);
-    }
-  }
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&attr, k);
+    if (e == cudaSuccess && attr.maxDynamicSharedSizeBytes < need) e = set_smem(k, need);
+  };
+  for (void (*k)(StepParams) : {k_selgat<__nv_bfloat16, 128, 8, true, false>, k_selgat<__nv_bfloat16, 128, 8, false, false>})
+    raise(k, (int)selgat_smem_bytes(max_visual, 0));
+  for (void (*k)(StepParams) : {k_selgat<__nv_bfloat16, 128, 4, true>, k_selgat<__nv_bfloat16, 128, 4, false>,
+                                k_selgat<__nv_bfloat16, 128, 8, true>, k_selgat<__nv_bfloat16, 128, 8, false>,
+                                k_selgat<__nv_bfloat16, 64, 4, true>, k_selgat<__nv_bfloat16, 64, 4, false>,
+                                k_selgat<__nv_bfloat16, 64, 8, true>, k_selgat<__nv_bfloat16, 64, 8, false>})
+    raise(k, (int)selgat_smem_bytes(max_visual, 0, kSgMaxW));
+  for (void (*k)(StepParams) : {k_selgat<float, 128, 4, true>, k_selgat<float, 128, 4, false>, k_selgat<float, 128, 8, true>,
+                                k_selgat<float, 128, 8, false>, k_selgat<float, 64, 4, true>, k_selgat<float, 64, 4, false>,
+                                k_selgat<float, 64, 8, true>, k_selgat<float, 64, 8, false>})
+    raise(k, (int)selgat_smem_bytes(max_visual, 1, 64));
   return e == cudaSuccess ? configure_fixed_kernels() : e;
 }
 
