@@ -304,6 +304,7 @@ vp_status vp_decode_step(vp_ctx* ctx, int32_t batch, const void* q,
     return fail(ctx, VP_ERR_UNSUPPORTED, "vp_decode_step: the tcgen05 score kernel (VP_SCORE_TC) cannot serve this "
                 "call (needs bf16, head_dim 128, G <= 16, pages of >= 8 tokens, a tensor-descriptor layout)");
   p.mt_o = ctx->mt_o; p.mt_st = ctx->mt_st; p.hmax = ctx->hmax;
+  p.fused = vp::select_kind(p, kept_cap);
 
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   take_set(ctx, p, st);

@@ -188,7 +188,7 @@ struct Plan {
 
 // tc: the score splits are for the tensor-core kernel (128-row tiles).
 // beside: the score kernel runs beside the previous call's select kernel (a
-// context with two sets of its outputs); 0 if not.  It then has that kernel's time to
+// context with two sets of its outputs).  It then has that kernel's time to
 // itself, on the other SMs, while every split lengthens the select kernel's
 // merges: at most kBesideSplits splits, or as many as keep kBesideTiles tiles a
 // CTA, on the SMs the select clusters leave.  Measured, B = 1, 28/4 heads,
@@ -196,21 +196,23 @@ struct Plan {
 // 16 303, 12 312; 4 fp32 sequences of up to 2796 tokens (32 select CTAs): 19
 // splits 22.9 us a call, 16 22.8, 15 (one wave beside them) 14.9.
 // A call that runs by itself (a kernel of the caller's between two calls) pays
-// for the SMs left out: where the plan costs more than `beside` times the
-// whole GPU's by the costs below, it takes the whole GPU.  us a call, back to
-// back / by itself, on the SMs left and on all: 8 x 3857 tokens, 28/4 heads
-// 22.7 / 29.9 and 21.4 / 24.2; 9 x 4000 24.9 / 32.6 and 23.2 / 24.4; 8 x 7424,
-// 32/8 heads 46.9 / 58.2 and 43.5 / 50.5.  Below that the overlap is worth more:
-// 6 x 5000 (1.37) 17.9 / 27.6 and 23.2 / 24.0; 6 x 20480 (1.37) 39.5 / 52.4 and
-// 46.4 / 51.9; 5 x 9000 22.0 / 34.4 and 31.7 / 32.4.  A call of three kernels has
-// less to gain, its gather kernel takes the whole GPU in between: 4 x 4352 at 20%
-// (1.16) 18.3 / 26.7 and 24.4 / 26.2, but 4 x 8192 with diagnostics (1.20) 32.6 /
-// 36.0 and 32.1 / 34.3, 4 x 3328, 32/8 heads (1.21) 26.9 / 29.4 and 25.7 / 27.9,
-// 6 x 6400 (1.36) 37.8 / 39.7 and 32.5 / 33.7.
+// for the SMs left out, and back to back the overlap hides about the select
+// kernel's time.  So where a CTA's weight grows by more than kBesideMore (about
+// 6 us; kBesideMoreTc of the tensor-core kernel's units) over the whole GPU's
+// plan, or the plan does not fit beside the clusters in one wave, the call takes
+// the whole GPU.  us a call back to back / by itself, on the SMs left and on
+// all, 28/4 heads unless named: 8 x 3857 tokens (18) 22.7 / 29.9 and 21.4 / 24.2;
+// 8 x 8000, 16/2 heads (17) 20.7 / 28.2 and 22.5 / 23.8; 9 x 4000 (27) 24.9 /
+// 32.6 and 23.2 / 24.4; 7 x 6400 (22) 27.7 / 36.2 and 29.0 / 29.5; 8 x 7424, 32/8
+// heads (tensor cores, 156) 46.9 / 58.2 and 43.5 / 50.5.  Below the line: 6 x
+// 5000 (10) 17.9 / 27.6 and 23.2 / 24.0; 5 x 5000 at 20% (6) 21.3 / 29.6 and
+// 26.8 / 28.3; 6 x 20480 (tensor cores, 89) 39.5 / 52.4 and 46.4 / 51.9.  Calls
+// with diagnostics lose either way and do not plan so (8 x 1482 tokens 22.8 /
+// 24.5 and 21.5 / 23.3; 6 x 6400 37.8 / 39.7 and 32.5 / 33.7).
 constexpr int kBesideSplits = 16, kBesideTiles = 18;
-constexpr double kBesideCost = 1.5, kBesideCost3 = 1.18;  // calls of two and of three kernels
+constexpr double kBesideMore = 16.0, kBesideMoreTc = 100.0;
 inline Plan make_plan(int batch, int Hkv, int D, int num_sms, int max_visual, int max_seq, int kept_cap,
-                      int granularity, bool tc = false, double beside = 0.0) {
+                      int granularity, bool tc = false, bool beside = false) {
   const long long units = (long long)batch * Hkv;
   const int TR = tc ? kTcRows : 32;
   // Fixed-weight splits sized for the longest sequence (tiles wholly inside
@@ -228,7 +230,7 @@ inline Plan make_plan(int batch, int Hkv, int D, int num_sms, int max_visual, in
   int cl = 1;
   while (cl < 8 && sel * cl * 2 <= num_sms) cl *= 2;
   const long long slots = 2LL * num_sms;
-  const long long score_slots = beside > 0.0 && sel * cl <= num_sms / 2 ? slots - 2 * sel * cl : slots;
+  const long long score_slots = beside && sel * cl <= num_sms / 2 ? slots - 2 * sel * cl : slots;
   // Split count: minimise (waves of CTAs) x (tiles per CTA + a fixed cost per
   // CTA for its start, its pipeline fill and its partial), keeping a minimum
   // of work per CTA; the smaller count wins a tie.  The costs were measured
@@ -236,7 +238,7 @@ inline Plan make_plan(int batch, int Hkv, int D, int num_sms, int max_visual, in
   // kernel, about 6 weight units of 128 rows for the tensor-core kernel.
   long long ns_hi = tiles / (tc ? 2 * kTcWv : 8);
   if (ns_hi > kNsMax) ns_hi = kNsMax;
-  if (beside > 0.0) {
+  if (beside) {
     const long long units_per = tc ? 2 * kTcWv * kBesideTiles / 8 : kBesideTiles;  // as 8 tiles to 2 K-only ones above
     const long long least = (tiles + units_per - 1) / units_per;
     const long long cap = least > kBesideSplits ? least : kBesideSplits;
@@ -244,19 +246,21 @@ inline Plan make_plan(int batch, int Hkv, int D, int num_sms, int max_visual, in
   }
   if (ns_hi < 1) ns_hi = 1;
   const double fixed = tc ? 6.0 * kTcWv : 12.0;
-  auto cost = [&](long long c, long long on) {
-    return (double)((units * c + on - 1) / on) * ((double)tiles / (double)c + fixed);
-  };
   auto best_of = [&](long long on) {
     long long n = 1;
-    for (long long c = 2; c <= ns_hi; ++c)
-      if (cost(c, on) < cost(n, on) * (1.0 - 1e-9)) n = c;
+    double best = 0.0;
+    for (long long c = 1; c <= ns_hi; ++c) {
+      const double waves = (double)((units * c + on - 1) / on);
+      const double cost = waves * ((double)tiles / (double)c + fixed);
+      if (c == 1 || cost < best * (1.0 - 1e-9)) { best = cost; n = c; }
+    }
     return n;
   };
   long long ns = best_of(score_slots);
   if (score_slots < slots) {
     const long long whole = best_of(slots);
-    if (cost(ns, slots) > beside * cost(whole, slots)) ns = whole;
+    const double more = (double)w_max / (double)ns - (double)w_max / (double)whole;
+    if (more > (tc ? kBesideMoreTc : kBesideMore) || units * ns > score_slots) ns = whole;
   }
   // Kept chunks of about 2048 rows, smaller (down to 256) while the gather
   // grid would not fill the GPU once (measured against 1024-row chunks and a
@@ -302,11 +306,11 @@ inline int split_floor(const Plan& pl, int batch, int Hkv, int num_sms, bool tc,
 // keeps the splits it has on the whole GPU (paged, 8-token pages, 8 sequences
 // of 65536 tokens, one kv-head: 22 splits of 33 tiles, 38 of 19 fit).
 inline Plan step_plan(int batch, int Hkv, int D, int num_sms, int max_visual, int max_seq, int kept_cap,
-                      int granularity, bool tc, double beside, int paged, int page_size) {
-  for (;; beside = 0.0) {
+                      int granularity, bool tc, bool beside, int paged, int page_size) {
+  for (;; beside = false) {
     Plan pl = make_plan(batch, Hkv, D, num_sms, max_visual, max_seq, kept_cap, granularity, tc, beside);
     pl.split_w = split_floor(pl, batch, Hkv, num_sms, tc, pl.split_w);
-    if (beside == 0.0 || page_ids_fit(paged, page_size, max_seq, pl.ns, pl.split_w, tc)) return pl;
+    if (!beside || page_ids_fit(paged, page_size, max_seq, pl.ns, pl.split_w, tc)) return pl;
   }
 }
 
@@ -401,9 +405,8 @@ inline WsLayout ws_layout(int batch, int H, int Hkv, int D, int max_visual, int 
   for (int bb = 1; bb <= batch; ++bb)
     for (int tc = 0; tc < 2; ++tc)
       for (int gran = 0; gran < (second_set ? 2 : 1); ++gran)
-        for (double beside : {0.0, kBesideCost, kBesideCost3}) {
-          if (beside > 0.0 && !second_set) continue;
-          const Plan pl = make_plan(bb, Hkv, D, num_sms, max_visual, max_seq, 0, gran, tc != 0, beside);
+        for (int beside = 0; beside < (second_set ? 2 : 1); ++beside) {
+          const Plan pl = make_plan(bb, Hkv, D, num_sms, max_visual, max_seq, 0, gran, tc != 0, beside != 0);
           if (pl.ns > w.nsp_max) w.nsp_max = pl.ns;
         }
   const size_t B = (size_t)batch, G = (size_t)(H / Hkv);
@@ -515,9 +518,7 @@ inline int select_kind(const StepParams& p, int kept_cap) {
 // two_sets: the context has two sets of the score kernels' outputs.
 inline bool plan_step(StepParams& p, int num_sms, int kept_cap, int granularity, int path = 0, bool two_sets = false) {
   p.num_sms = num_sms;
-  p.cl = make_plan(p.B, p.Hkv, p.D, num_sms, p.max_visual, p.max_seq, kept_cap, granularity).cl;
-  p.fused = select_kind(p, kept_cap);
-  const double beside = !two_sets ? 0.0 : p.fused == 1 ? kBesideCost : kBesideCost3;
+  const bool beside = two_sets && !p.n_act && !p.act_bits;
   const long long w_tc = 2LL * ((p.max_seq + kTcRows - 1) / kTcRows) - p.max_visual / kTcRows;
   const bool eligible = tc_eligible(p.dtype, p.D, p.G, p.paged, p.page_size);
   const bool tc = path == 2 ? eligible

@@ -129,8 +129,8 @@ int check_beside() {
               const WsLayout ws = ws_layout(max_batch, H, Hkv, D, mv, ms, sms, true);
               for (int B = 1; B <= max_batch; ++B)
                 for (int tc = 0; tc < 2; ++tc)
-                  for (int gran = 0; gran < 2; ++gran) for (double beside : {kBesideCost, kBesideCost3}) {
-                    const Plan pl = make_plan(B, Hkv, D, sms, mv, ms, 64, gran, tc != 0, beside);
+                  for (int gran = 0; gran < 2; ++gran) {
+                    const Plan pl = make_plan(B, Hkv, D, sms, mv, ms, 64, gran, tc != 0, true);
                     ++plans;
                     check(pl.ns >= 1 && pl.ns <= kNsMax && pl.ns <= ws.nsp_max, "beside: ns within the workspace", B, Hkv,
                           D, sms, mv, ms, 64, tc, gran);
@@ -140,20 +140,19 @@ int check_beside() {
                   }
             }
   std::printf("%lld plans beside a select kernel, %d violations\n", plans, fails - before);
-  // Splits of such plans: on the SMs the select clusters leave, unless that
-  // would cost a call that runs by itself too much.
-  struct { int B, Hkv, D, mv, ms, tc, want, want3; } cases[] = {
-      {1, 4, 128, 1296, 3920, 0, 16, 16}, {4, 4, 128, 4096, 8255, 0, 15, 19}, {4, 4, 128, 2304, 4415, 0, 15, 15}, {6, 4, 128, 4096, 20543, 1, 8, 12},
-      {6, 4, 128, 2304, 6463, 0, 8, 12}, {8, 4, 128, 1296, 3920, 0, 9, 9}, {9, 4, 128, 1296, 4059, 0, 8, 8},
-      {8, 8, 64, 1296, 5059, 0, 4, 4}, {8, 8, 128, 6400, 7487, 1, 4, 4},
+  // Splits of such plans: on the SMs the select clusters leave, unless a CTA's
+  // work grows too much by that, or they do not fit in one wave.
+  struct { int B, Hkv, D, mv, ms, tc, want; } cases[] = {
+      {1, 4, 128, 1296, 3920, 0, 16}, {4, 4, 128, 4096, 8255, 0, 15}, {6, 4, 128, 2304, 5067, 0, 8},
+      {6, 4, 128, 4096, 20543, 1, 8}, {7, 4, 128, 2304, 6463, 0, 10}, {8, 4, 128, 1296, 3920, 0, 9},
+      {8, 2, 128, 2304, 8067, 0, 19}, {9, 4, 128, 1296, 4059, 0, 8}, {8, 8, 64, 1296, 5059, 0, 4}, {8, 8, 128, 6400, 7487, 1, 4},
   };
   int bad = 0;
   for (const auto& c : cases) {
-    const Plan pl = make_plan(c.B, c.Hkv, c.D, 152, c.mv, c.ms, 64, 0, c.tc != 0, kBesideCost);
-    const Plan pl3 = make_plan(c.B, c.Hkv, c.D, 152, c.mv, c.ms, 64, 0, c.tc != 0, kBesideCost3);
-    if (pl.ns != c.want || pl3.ns != c.want3) {
-      std::printf("FAIL splits beside a select kernel: B=%d Hkv=%d D=%d max_visual=%d max_seq=%d tc=%d: %d, %d (want %d, %d)\n",
-                  c.B, c.Hkv, c.D, c.mv, c.ms, c.tc, pl.ns, pl3.ns, c.want, c.want3);
+    const Plan pl = make_plan(c.B, c.Hkv, c.D, 152, c.mv, c.ms, 64, 0, c.tc != 0, true);
+    if (pl.ns != c.want) {
+      std::printf("FAIL splits beside a select kernel: B=%d Hkv=%d D=%d max_visual=%d max_seq=%d tc=%d: %d (want %d)\n", c.B,
+                  c.Hkv, c.D, c.mv, c.ms, c.tc, pl.ns, c.want);
       ++bad;
     }
   }
@@ -209,8 +208,8 @@ int check_page_ids() {
               if (two_sets(B, Hkv, D, T, 2))
                 for (int gran = 0; gran < 2; ++gran)
                   for (int tc = 0; tc < 2; ++tc) {
-                    const Plan whole = step_plan(bsz, Hkv, D, 152, mv, T, 64, gran, tc != 0, 0.0, 1, page);
-                    const Plan pl = step_plan(bsz, Hkv, D, 152, mv, T, 64, gran, tc != 0, kBesideCost, 1, page);
+                    const Plan whole = step_plan(bsz, Hkv, D, 152, mv, T, 64, gran, tc != 0, false, 1, page);
+                    const Plan pl = step_plan(bsz, Hkv, D, 152, mv, T, 64, gran, tc != 0, true, 1, page);
                     fewer += pl.ns < whole.ns;
                     if (page_ids_fit(1, page, T, whole.ns, whole.split_w, tc != 0) &&
                         !page_ids_fit(1, page, T, pl.ns, pl.split_w, tc != 0) && ++bad <= 10)
